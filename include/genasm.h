@@ -72,11 +72,11 @@ typedef struct CUstream_st* ga_stream_t; /* = cudaStream_t; NULL = legacy defaul
 #define GA_OP_MATCH 7 /* '=' */
 #define GA_OP_SUBST 8 /* 'X' */
 
-/* Largest window: ga_align_batch, _tuned, _order and the workspace sizes
- * take W <= GA_MAX_W; windows of 65..128 bases run on a kernel with 128-bit
- * window vectors and tables in the workspace. The other entry points (the
+/* Largest window: ga_align_batch, _tuned, _order, _locate and the workspace
+ * sizes take W <= GA_MAX_W; windows of 65..128 bases run on builds of the
+ * batched kernel with vectors of 96 and 128 bits. The other entry points (the
  * plain kernel, the server, the no-alloc form, the autotuner and graph, the
- * ablation) keep their tables on chip and take W <= GA_MAX_W_ONCHIP. */
+ * ablation) take W <= GA_MAX_W_ONCHIP. */
 #define GA_MAX_W 128
 #define GA_MAX_W_ONCHIP 64
 
@@ -112,30 +112,24 @@ int ga_workspace_size(uint32_t n_pairs, int W, int O, int k, size_t* bytes_out);
 /*
  * Tuning of the batched kernel. ga_align_batch uses the library's defaults
  * (or what ga_autotune stored for this device); ga_align_batch_tuned takes an
- * explicit choice. All fields 0 = default.
- *   lanes_per_pair : lanes that run one pair's DC wavefront: 4, 8, 16 or 32
- *                    (each lane owns 64 / lanes_per_pair text columns).
- *   pairs_per_block: pairs resident per thread block.
- *   table_rows     : error rows of a window's table kept in shared memory
- *                    (for windows that are not the last); a window whose
- *                    solution row does not fit is recomputed into the
- *                    workspace. With O >= 16 such windows keep 32-bit
- *                    entries (the 32 bits of each cell around the
- *                    traceback's diagonal; a window whose traceback leaves
- *                    that band is redone with 64-bit entries in the
- *                    workspace), otherwise 64-bit entries.
+ * explicit choice. All fields 0 = default. The kernel runs one lane per pair
+ * and sizes its grid and tables from the number of pairs and W, so the first
+ * three fields and max_registers no longer change how a batch runs; their
+ * values are still checked, and tunings saved by earlier versions stay valid.
+ *   lanes_per_pair : 4, 8, 16 or 32.
+ *   pairs_per_block: lanes_per_pair * pairs_per_block a multiple of 32, at
+ *                    most 256.
+ *   table_rows     : the shape's tables (of rows of the row form) must fit a
+ *                    block's shared memory.
  *   lpt            : 1 = hand out pairs longest read first, -1 = in index
  *                    order (0 = default, longest first).
- *   max_registers  : 0 = the kernel as compiled; 168 or 128 (with
- *                    lanes_per_pair 8) = a variant capped at that many
- *                    registers per thread, so that more blocks fit an SM
- *                    when the tables are small.
+ *   max_registers  : 0, or 168 or 128 with lanes_per_pair 8.
  *   slice_windows  : pairs take turns of this many windows through a FIFO
  *                    queue (their window state is saved between turns), so
  *                    that all pairs finish together instead of the last
  *                    ones running alone; -1 = off (a pair runs to its end);
  *                    0 = automatic (turns of 64 windows when the pairs
- *                    outnumber the resident groups, but less than 16 times).
+ *                    outnumber the resident lanes, but less than 16 times).
  */
 typedef struct ga_tuning_s {
   int lanes_per_pair;
@@ -158,16 +152,15 @@ int ga_tuning_set(int W, int O, int k, const ga_tuning* tuning);
 
 /*
  * ga_autotune - the autotuner of the batched kernel. Runs the current
- * default once on the caller's sample (with statistics, to estimate the
- * typical d_min), then times a candidate set of (lanes_per_pair,
- * pairs_per_block, table_rows) with CUDA events, one warm-up
+ * default once on the caller's sample (with statistics), then times a
+ * candidate set of (lpt, slice_windows) with CUDA events, one warm-up
  * and one timed run each, and stores the fastest as the default for this
  * device and (W, O, k). Arguments as ga_align_batch (outputs are
  * overwritten; d_n_windows and d_cells are required); the workspace must hold
  * ga_autotune_workspace_size(n_pairs, W, O, k) bytes. Synchronous: returns
  * once every run has finished. *best / *best_ms (either may be NULL) receive
  * the choice and its time. The paper gives no tuning procedure.
- * Errors: GA_EINVAL (also for W > GA_MAX_W_ONCHIP: the 128-bit kernel has no
+ * Errors: GA_EINVAL (also for W > GA_MAX_W_ONCHIP: wider windows take no
  * tuning), GA_ENOSPC (no candidate fits the workspace), GA_ECUDA.
  */
 int ga_autotune(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_t* d_read_len,
@@ -231,9 +224,8 @@ int ga_workspace_size_tuned(uint32_t n_pairs, int W, int O, int k, const ga_tuni
  * again in the same process. Every
  * call shares the array and overwrites what the previous call left there, so
  * calls whose work overlaps on the GPU (other streams, other host threads)
- * race: order them on one stream or wait between them. It runs with tables
- * sized for all 65 error rows in shared memory, so it is slower than
- * ga_align_batch.
+ * race: order them on one stream or wait between them. It runs without the
+ * turns of the sliced queue, whose ring needs memory.
  * Errors: GA_ENOSPC if n_pairs > GA_NOALLOC_MAX_PAIRS, GA_EINVAL, GA_ECUDA.
  */
 #define GA_NOALLOC_MAX_PAIRS 262144
@@ -393,8 +385,7 @@ int ga_measure_smem_peak(double out[2], ga_stream_t stream);
  * Workspace: d_workspace of ws_bytes >= ga_workspace_size(...); its contents
  * on entry do not matter. Concurrent calls need separate workspaces.
  * Limits: 1 <= W <= GA_MAX_W (128), 0 <= O < W, k >= 0 (k >= W means no
- * cap). Windows wider than GA_MAX_W_ONCHIP (64) run on the 128-bit kernel:
- * 16 lanes per pair, tables in the workspace, no tuning.
+ * cap). Windows wider than GA_MAX_W_ONCHIP (64) take no tuning.
  * Errors: GA_EINVAL, GA_ENOSPC (workspace too small), GA_ECUDA.
  */
 int ga_align_batch(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_t* d_read_len,
@@ -433,7 +424,7 @@ int ga_align_batch(const uint8_t* d_reads, const uint64_t* d_read_off, const uin
  * GA_PAIR_EXCEEDS_K. Tuning: the one ga_autotune_locate stored for this
  * device and (W, O, k), else the library default (ga_align_batch_locate_tuned
  * takes an explicit one). Windows of 65..128 bases run the same search and
- * alignment with 128-bit vectors (tuning ignored). Workspace:
+ * alignment with wider vectors (tuning ignored). Workspace:
  * ga_workspace_size_locate(n_pairs, W, O, k, tuning) bytes. Asynchronous on
  * `stream`. Errors: GA_EINVAL (also NULL start spans / starts), GA_ENOSPC,
  * GA_ECUDA.
@@ -529,11 +520,12 @@ int ga_align_batch_tuned(const uint8_t* d_reads, const uint64_t* d_read_off,
  *   variant 1: only their AND (idea 1);
  *   variant 2: and only rows 0..d_min (ideas 1, 2);
  *   variant 3: and only the columns the traceback can reach (ideas 1-3).
- * ga_align_batch is the further step: only the reachable bits, on chip.
  * Every variant gives ga_align_batch's outputs exactly (same arguments and
  * contract, no tuning). d_table_bytes (NULL to skip; n_pairs x 5 uint64,
  * overwritten) receives per pair the bytes of window table that variants
- * 0..3 and ga_align_batch (column 4) write, summed over the pair's windows.
+ * 0..3 write and (column 4) those of the rows cut down to the 32 bits around
+ * the diagonal that the traceback can reach, summed over the pair's windows.
+ * (ga_align_batch itself keeps no rows: it stores 16 bytes per text column.)
  * Workspace: ga_ablation_workspace_size(n_pairs, W, O, k, variant) bytes
  * (variant 0 holds 137 KB of table per resident pair).
  * Errors: GA_EINVAL (also variant outside 0..3), GA_ENOSPC, GA_ECUDA.

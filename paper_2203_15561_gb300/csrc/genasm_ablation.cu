@@ -7,11 +7,10 @@
 //   variant 2: + idea (2): only rows 0..d_min (row early termination);
 //   variant 3: + idea (3): only the columns the traceback can reach (0..W-O
 //              in a window that is not the last).
-// The production kernel (genasm_align.cu) further keeps only the bits the
-// traceback can reach (band entries) and holds the table on chip. Every
-// variant gives the same alignment. When asked, each window also adds to
-// table_bytes[5 * pair + v] the table bytes that variant v (v = 4: the
-// production kernel) writes for it, so one run gives the footprint of all.
+// Every variant gives the same alignment. When asked, each window also adds to
+// table_bytes[5 * pair + v] the table bytes that variant v writes for it (v =
+// 4: variant 3 with 32-bit entries, the bits around the diagonal that the
+// traceback can reach), so one run gives the footprint of all.
 #include <algorithm>
 #include <cstdint>
 
@@ -42,7 +41,7 @@ struct AblationArgs {
 
 template <int V>
 __device__ __forceinline__ void ablation_window(const AlignParams& p, int r, int gbase,
-                                                PairState& st, GroupSmem* gs, uint64_t* pmcol,
+                                                PairState& st, uint64_t* pmcol,
                                                 uint64_t* tab, uint64_t* table_bytes) {
   constexpr int G = kAblG;
   const bool writer = r == 0;
@@ -66,29 +65,26 @@ __device__ __forceinline__ void ablation_window(const AlignParams& p, int r, int
   __syncwarp();
   int dmin;
   if constexpr (V == 0) {
-    dmin = dc_window<G, kFmtWide, false, false, true>(r, gbase, ga, wp, wt, p.kmax, ncols, S,
-                                                      kMaxRows, 0, pm, gs->pmb, tab);
+    dmin = dc_window<G, false, false, true>(r, gbase, ga, wp, wt, p.kmax, ncols, S, kMaxRows, pm,
+                                            tab);
   } else if constexpr (V == 1) {
-    dmin = dc_window<G, kFmtWide, false, false, false>(r, gbase, ga, wp, wt, p.kmax, ncols, S,
-                                                       kMaxRows, 0, pm, gs->pmb, tab);
+    dmin = dc_window<G, false, false, false>(r, gbase, ga, wp, wt, p.kmax, ncols, S, kMaxRows, pm,
+                                             tab);
   } else {
-    dmin = dc_window<G, kFmtWide, false>(r, gbase, ga, wp, wt, p.kmax, ncols, S, kMaxRows, 0, pm,
-                                         gs->pmb, tab);
+    dmin = dc_window<G, false>(r, gbase, ga, wp, wt, p.kmax, ncols, S, kMaxRows, pm, tab);
   }
   __syncwarp();
   const bool exceeds = ga && dmin < 0;
   const bool trace = ga && !exceeds;
   int cp = 0, ct = 0;
-  bool unused = false;
   const bool ok =
-      tb_window<G, kFmtWide, V == 0>(r, gbase, trace, wp, wt, dmin, last, commit, ncols, S, 0,
-                                     p.tb_table, pmcol, gs->pmb, tab, st.rw, writer, cp, ct,
-                                     st.edits, unused);
+      tb_window<G, V == 0>(r, gbase, trace, wp, wt, dmin, last, commit, ncols, S, p.tb_table, pmcol,
+                           tab, st.rw, writer, cp, ct, st.edits);
   __syncwarp();
   if (ga) {
     if (table_bytes && writer && !exceeds) {
       const uint64_t rows_all = static_cast<uint64_t>(p.kmax) + 1, rows = dmin + 1;
-      const bool band = !last && p.O >= 16;  // the production kernel's band rule
+      const bool band = !last && p.O >= 16;  // windows whose walk stays in 32 bits
       uint64_t* tb = table_bytes + 5ull * st.pair;
       tb[0] += rows_all * static_cast<uint64_t>(wt) * 32;  // four 8-byte vectors per cell
       tb[1] += rows_all * static_cast<uint64_t>(wt + 1) * 8;
@@ -116,7 +112,6 @@ template <int V>
 __global__ void __launch_bounds__(kAblG * kAblPpb, 1) align_ablation_kernel(const AlignParams p,
                                                                           const AblationArgs a) {
   __shared__ __align__(16) uint64_t pmcols[kAblPpb][kPmCols];
-  __shared__ __align__(16) GroupSmem gsm[kAblPpb];
   constexpr int G = kAblG;
   const int lane = threadIdx.x & 31;
   const int gib = threadIdx.x / G;
@@ -138,7 +133,7 @@ __global__ void __launch_bounds__(kAblG * kAblPpb, 1) align_ablation_kernel(cons
     }
     if (!__any_sync(kFull, st.busy || !drained)) break;
     if (__any_sync(kFull, st.busy))
-      ablation_window<V>(p, r, gbase, st, &gsm[gib], pmcols[gib], tab, a.table_bytes);
+      ablation_window<V>(p, r, gbase, st, pmcols[gib], tab, a.table_bytes);
   }
 }
 

@@ -1,0 +1,423 @@
+// The batched alignment kernel, the server's step kernel and the locate step
+// as templates over the window width (VW 32-bit words per vector) and the
+// traceback order; genasm_align.cu instantiates VW = 1 and 2 (windows of up
+// to 32 and 64 bases), genasm_wide.cu VW = 3 and 4 (up to 96 and 128).
+//
+// Batched: a persistent grid of one-warp blocks; each lane pulls pairs from a
+// device queue and aligns them one at a time, one window per round of its
+// warp. With LPT the queue starts in longest-read-first order (a counting
+// sort), so the lanes of a warp hold pairs of about the same length.
+//
+// Sliced form (slice > 0): the queue is a FIFO of pairs, and a lane runs a
+// pair for at most `slice` windows, saves its window state (positions, edit
+// count, statistics, open CIGAR run) and puts it back at the tail. Every pair
+// then moves forward at the same pace, and a batch whose pairs outnumber the
+// resident lanes but not by a whole multiple does not end with a round in
+// which a few lanes run alone.
+//
+// The FIFO is a bounded ring of 2n slots (n = pairs) with a sequence number
+// per slot: position x lives in slot x % 2n; the slot holds position x's
+// pair once its number is x + 1, and is free for position x + 2n once its
+// number is x + 2n. A lane that wants a pair reserves the next head position
+// with atomicAdd and takes the pair once that position is published; until
+// then it stays idle while the other lanes of its warp go on (it checks
+// again after each of their windows), and it stops once no pair is left
+// unfinished. A lane that ends a turn claims the next tail position with
+// atomicAdd; the slot it lands in held position y - 2n, which was published
+// at least n pushes earlier and taken as soon as its reserver looked (at most
+// n pairs are ever in the ring), so the slot is free; the lane writes the
+// pair and publishes it. The wait for a free slot is bounded: should it run
+// out, the lane keeps its pair for another turn and flags the launch, and the
+// reserver of the lost position stops with the others at the end. Every pair
+// not yet finished is held by a running lane or published in the ring. A
+// warp whose lanes all wait for a pair also waits a bounded time only
+// (behind a lost position published pairs could otherwise be left without a
+// reserver); the pairs a run-out wait leaves unfinished keep the timed-out
+// status that the ring's set-up kernel gives every pair.
+#pragma once
+
+#include <algorithm>
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+#include "genasm.h"
+#include "genasm_internal.h"
+#include "genasm_lane.cuh"
+
+namespace ga {
+
+struct BatchArgs {
+  uint32_t* queue;        // [0] hand-out counter (unsliced); ring: [1] head, [2] tail,
+                          // [3] pairs not finished, [4] a warp's wait ran out
+  const uint32_t* order;  // hand-out order (nullptr: index order)
+  int cols;               // columns of a lane's table
+  int lanes;              // lanes of a warp that take pairs
+  uint32_t slice;         // windows per turn (0: a pair runs to its end)
+  uint32_t* ring;         // 2n ring slots: pair ids
+  uint32_t* ring_seq;     // 2n: each slot's sequence number
+  SlotState* state;       // per pair: saved window state (all zero: not started)
+  uint32_t idle_polls;    // bound of a warp's wait for a published pair
+  uint32_t push_polls;    // bound of a push's wait for its slot
+};
+
+constexpr uint32_t kNoPair = 0xffffffffu;
+
+// The pair at reserved ring position x, or kNoPair while it is not published.
+__device__ __forceinline__ uint32_t ring_take(const BatchArgs& a, uint32_t cap, uint32_t x) {
+  volatile uint32_t* seq = a.ring_seq;
+  volatile uint32_t* slot = a.ring;
+  const uint32_t s = x % cap;
+  if (seq[s] != x + 1u) return kNoPair;
+  __threadfence();
+  const uint32_t pair = slot[s];
+  __threadfence();
+  seq[s] = x + cap;  // free for position x + cap
+  return pair;
+}
+
+// Puts a pair (its state already saved) at the ring's tail; false (the pair
+// stays with its lane) only if the slot's wait ran out.
+__device__ __forceinline__ bool ring_push(const BatchArgs& a, uint32_t cap, uint32_t pair) {
+  volatile uint32_t* seq = a.ring_seq;
+  volatile uint32_t* slot = a.ring;
+  __threadfence();  // the saved state before the publication
+  const uint32_t y = atomicAdd(a.queue + 2, 1u);
+  const uint32_t s = y % cap;
+  for (uint32_t polls = 0; seq[s] != y; ++polls) {
+    if (polls >= a.push_polls) {
+      atomicExch(a.queue + 4, 1u);
+      return false;
+    }
+    __nanosleep(200);
+  }
+  slot[s] = pair;
+  __threadfence();
+  seq[s] = y + 1u;
+  return true;
+}
+
+// The dynamic shared memory of a one-warp block, from its first multiple of
+// the Eq masks' size on (their addresses are formed with OR).
+template <int VW>
+__device__ __forceinline__ uint32_t lane_smem_base() {
+  extern __shared__ __align__(1024) uint32_t lane_smem[];
+  constexpr uint32_t kAlign = LaneShape<VW>::kEqBytes;
+  return (smem_addr(lane_smem) + kAlign - 1u) & ~(kAlign - 1u);
+}
+constexpr size_t lane_block_smem(int VW, int cols, bool any_order) {
+  return lane_smem_bytes(VW, cols, any_order) + (VW >= 3 ? 1024u : 0u);
+}
+
+template <int VW, bool kAny>
+__global__ void __launch_bounds__(32) align_batched_kernel(const AlignParams p, const BatchArgs a) {
+  const uint32_t base = lane_smem_base<VW>();
+  const uint32_t lane = threadIdx.x;
+  LanePair st;
+  st.busy = false;
+  bool drained = lane >= static_cast<uint32_t>(a.lanes);
+  uint32_t budget = 0;
+  uint32_t resv = kNoPair;  // the ring position this lane has reserved
+  uint32_t idle = 0;        // consecutive polls of a warp with no pair to work on
+  for (;;) {
+    // Lanes without a pair take the next one from the queue.
+    const bool want = !st.busy && !drained;
+    const uint32_t wants = __ballot_sync(kFull, want);
+    bool ended = false;  // a pair that finished at its start
+    if (wants) {
+      uint32_t pair = kNoPair;
+      bool quit = false;
+      if (a.slice) {
+        if (want) {
+          if (resv == kNoPair) resv = atomicAdd(a.queue + 1, 1u);
+          pair = ring_take(a, 2u * p.n_pairs, resv);
+          if (pair != kNoPair) resv = kNoPair;
+          else quit = *reinterpret_cast<volatile uint32_t*>(a.queue + 3) == 0u;  // all finished
+        }
+      } else {
+        const int first = __ffs(wants) - 1;
+        uint32_t idx = 0;
+        if (static_cast<int>(lane) == first) idx = atomicAdd(a.queue, __popc(wants));
+        idx = __shfl_sync(kFull, idx, first) + __popc(wants & ((1u << lane) - 1u));
+        if (want) {
+          if (idx < p.n_pairs) pair = a.order ? a.order[idx] : idx;
+          else quit = true;
+        }
+      }
+      if (want) {
+        if (pair != kNoPair) {
+          lane_begin(p, pair, st);
+          ended = !st.busy;
+          if (a.slice) {
+            // Another SM may have saved this state: read it from L2, not L1.
+            const SlotState* sp = a.state + pair;
+            SlotState s;
+            s.pos_p = __ldcg(&sp->pos_p);
+            s.pos_t = __ldcg(&sp->pos_t);
+            s.edits = __ldcg(&sp->edits);
+            s.windows = __ldcg(&sp->windows);
+            s.cells = __ldcg(reinterpret_cast<const unsigned long long*>(&sp->cells));
+            s.runs = __ldcg(&sp->runs);
+            s.run_op = __ldcg(&sp->run_op);
+            s.run_len = __ldcg(&sp->run_len);
+            if (s.windows > 0) lane_resume(s, st);  // a pair that had turns already
+            budget = a.slice;
+          }
+        } else if (quit) {
+          drained = true;
+        }
+      }
+      __syncwarp();
+    }
+    if (!__any_sync(kFull, st.busy || !drained)) break;
+    const bool was_busy = st.busy;
+    if (__any_sync(kFull, st.busy)) {
+      lane_window<VW, kAny>(p, st, base, a.cols);
+      if (was_busy && (st.status != kPairOk || st.pos_p >= st.m)) lane_finish(p, st);
+      idle = 0;
+    } else {
+      // Every lane of the warp waits for a pair: poll again shortly.
+      __nanosleep(200);
+      if (++idle >= a.idle_polls) {
+        if (lane == 0) atomicExch(a.queue + 4, 1u);
+        drained = true;
+      }
+    }
+    if (a.slice) {
+      if ((was_busy && !st.busy) || ended) atomicSub(a.queue + 3, 1u);  // this pair is finished
+      // End of a turn: the pair goes back to the queue's tail (or, if the ring
+      // cannot take it now, stays for another turn).
+      if (st.busy && --budget == 0) {
+        lane_save(st, a.state[st.pair]);
+        if (ring_push(a, 2u * p.n_pairs, st.pair)) st.busy = false;
+        else budget = a.slice;
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// Serving step: resumable alignment. Every pair in the active list advances by
+// at most `max_windows` windows; its window state is kept in device memory
+// between steps, so pairs admitted at different times share one launch.
+template <int VW>
+__global__ void __launch_bounds__(32) align_step_kernel(const AlignParams p, const StepArgs a) {
+  const uint32_t base = lane_smem_base<VW>();
+  const uint32_t lane = threadIdx.x;
+  const uint32_t n_active = a.counters[2];
+  const uint32_t max_windows = a.counters[3];
+  // Few pairs spread over all warps, one lane each first.
+  const uint32_t lanes = min(32u, (n_active + gridDim.x - 1) / gridDim.x);
+  LanePair st;
+  st.busy = false;
+  bool drained = lane >= lanes;
+  uint32_t slot = 0, budget = 0;
+  for (;;) {
+    const bool want = !st.busy && !drained;
+    const uint32_t wants = __ballot_sync(kFull, want);
+    bool finished = false;
+    if (wants) {
+      const int first = __ffs(wants) - 1;
+      uint32_t idx = 0;
+      if (static_cast<int>(lane) == first) idx = atomicAdd(&a.counters[0], __popc(wants));
+      idx = __shfl_sync(kFull, idx, first) + __popc(wants & ((1u << lane) - 1u));
+      if (want) {
+        if (idx < n_active) {
+          slot = a.active[idx];
+          lane_begin(p, slot, st);  // a fresh slot (all zero) starts here
+          if (st.busy) lane_resume(a.state[slot], st);
+          budget = max_windows;
+          finished = !st.busy;
+        } else {
+          drained = true;
+        }
+      }
+      __syncwarp();
+    }
+    if (!__any_sync(kFull, st.busy || !drained || finished)) break;
+    const bool was_busy = st.busy;
+    if (__any_sync(kFull, st.busy)) lane_window<VW, false>(p, st, base, a.cols);
+    if (was_busy) {
+      if (st.status != kPairOk || st.pos_p >= st.m) {
+        lane_finish(p, st);
+        finished = true;
+      } else if (--budget == 0) {
+        lane_save(st, a.state[slot]);
+        st.busy = false;  // resumes at the next step
+      }
+    }
+    if (finished) a.done[atomicAdd(&a.counters[1], 1u)] = slot;
+    __syncwarp();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Free-start first window: the locate step. For a pair with start span S > 0
+// the first read window's pattern (wp = min(W, m) bases) is searched in the
+// reference's first L = min(n, S + W) bases with the recurrence of the
+// windows; every start column s = 0..min(S, L) is a candidate (s = L, the
+// empty text, costs wp insertions) and the leftmost column with the fewest
+// edits is where the alignment begins.
+//
+// 2^log_q lanes search a pair, each a range of start columns. A start's edits
+// are at most wp, so its alignment spans at most 2 wp text bases: a lane whose
+// recurrence begins 2 wp columns right of its range has every value of the
+// range exactly. Within a lane the columns run right to left and the pattern's
+// last row is followed by its horizontal differences; a column that does not
+// cost more than the best one so far takes its place (ties go left).
+// ---------------------------------------------------------------------------
+
+constexpr int kLocateWarps = 4;  // per block
+
+struct LocateArgs {
+  const uint32_t* start_span;
+  int32_t* ref_start;
+  int32_t* locate_d;
+};
+
+template <int VW>
+__global__ void __launch_bounds__(32 * kLocateWarps)
+    locate_kernel(const AlignParams p, const LocateArgs a, int log_q) {
+  using Shape = LaneShape<VW>;
+  // The Eq masks start at a multiple of their size (shared memory itself is
+  // aligned to 1 KB at most).
+  constexpr uint32_t kAlign = Shape::kEqBytes;
+  __shared__ __align__(1024) uint32_t eqs[(kLocateWarps * kAlign + (VW >= 3 ? 1024u : 0u)) / 4];
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t eq_lane = ((smem_addr(eqs) + kAlign - 1u) & ~(kAlign - 1u)) +
+                           (threadIdx.x >> 5) * kAlign + lane * Shape::kEqLane;
+  const uint64_t gid = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const uint32_t q = 1u << log_q, part = lane & (q - 1u);
+  const uint64_t pair = gid >> log_q;
+  const bool valid = pair < p.n_pairs;
+  uint32_t m = 0, n = 0, S = 0;
+  if (valid) {
+    m = p.read_len[pair];
+    n = p.ref_len[pair];
+    S = a.start_span[pair];
+  }
+  const bool go = valid && S > 0 && m > 0;
+  const int wp = go ? static_cast<int>(min(m, static_cast<uint32_t>(p.W))) : 1;
+  const uint64_t span_end = static_cast<uint64_t>(S) + static_cast<uint64_t>(p.W);
+  const uint32_t L = go ? static_cast<uint32_t>(min(static_cast<uint64_t>(n), span_end)) : 0u;
+  // The empty text (s = L) is a candidate when S reaches it: wp insertions.
+  uint64_t best = ~0ull;
+  if (go && S >= L && wp <= p.kmax) best = (static_cast<uint64_t>(wp) << 32) | L;
+  // This lane's start columns [lo, hi) and the column its recurrence begins at.
+  const uint32_t starts = go ? min(S == 0xffffffffu ? S : S + 1u, L) : 0u;
+  const uint32_t per = (starts + q - 1u) >> log_q;
+  const uint32_t lo = min(part * per, starts);
+  const uint32_t hi = min(lo + per, starts);
+  if (lo < hi) {
+    uint32_t pw[2 * VW], PL[VW], PH[VW];
+    load_bases<VW>(p.reads + p.read_off[pair], m, 0u, pw);
+    bit_planes<VW>(pw, PL, PH);
+    store_eq<VW>(eq_lane, wp, PL, PH);
+    const uint32_t x0 = static_cast<uint32_t>(min(static_cast<uint64_t>(L), static_cast<uint64_t>(hi) - 1u + 2u * wp));
+    const uint8_t* ref = p.refs + p.ref_off[pair];
+    const uintptr_t at = reinterpret_cast<uintptr_t>(ref);
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(at & ~static_cast<uintptr_t>(3));
+    const uint32_t o = 4u * static_cast<uint32_t>(at & 3u);  // base 0's place in word 0
+    uint32_t vp[VW], vn[VW], top[VW];
+#pragma unroll
+    for (int k = 0; k < VW; ++k) {
+      vp[k] = ~0u;
+      vn[k] = 0u;
+      top[k] = (wp - 1) >> 5 == k ? 1u << ((wp - 1) & 31) : 0u;
+    }
+    int score = wp, found = 0x7fffffff;
+    uint32_t pos = 0;
+    const int64_t w0 = (static_cast<int64_t>(o) + lo) >> 4;
+    uint32_t next = __ldg(words + ((static_cast<uint64_t>(o) + x0 - 1u) >> 4));
+    for (int64_t w = (static_cast<int64_t>(o) + x0 - 1) >> 4; w >= w0; --w) {
+      const uint32_t tw = next;
+      if (w > w0) next = __ldg(words + w - 1);
+      const int64_t i0 = 16 * w - o;  // the word's first base
+      // Columns of the word at or past x0 keep the initial column.
+      const int left = x0 - i0 < 16 ? static_cast<int>(x0 - i0) : 16;
+      // Start columns of the word: places from .. to - 1.
+      const int to = hi - i0 < 16 ? static_cast<int>(static_cast<int64_t>(hi) - i0) : 16;
+      const int from = i0 < lo ? static_cast<int>(lo - i0) : 0;
+#pragma unroll
+      for (int x = 15; x >= 0; --x) {
+        uint32_t eq[VW], d0[VW], hp[VW], hn[VW];
+        load_eq<VW>(eq_at<VW>(eq_lane, tw, x), eq);
+#pragma unroll
+        for (int k = 0; k < VW; ++k) eq[k] = x < left ? eq[k] : 0u;
+        column_step<VW>(eq, vp, vn, d0, hp, hn);
+        uint32_t up = 0, down = 0;
+#pragma unroll
+        for (int k = 0; k < VW; ++k) {
+          up |= hp[k] & top[k];
+          down |= hn[k] & top[k];
+        }
+        score += up ? 1 : 0;
+        score -= down ? 1 : 0;
+        if (x < to && x >= from && score <= found) {
+          found = score;
+          pos = static_cast<uint32_t>(i0 + x);
+        }
+      }
+    }
+    if (found <= p.kmax)
+      best = min(best, (static_cast<uint64_t>(found) << 32) | pos);
+  }
+  __syncwarp();
+  for (uint32_t s = q >> 1; s > 0; s >>= 1) best = min(best, __shfl_xor_sync(kFull, best, s));
+  if (valid && part == 0) {
+    if (!go) {
+      a.ref_start[pair] = 0;
+      a.locate_d[pair] = -1;
+    } else if (best == ~0ull) {
+      a.ref_start[pair] = -1;
+      a.locate_d[pair] = -1;
+    } else {
+      a.ref_start[pair] = static_cast<int32_t>(best & 0xffffffffu);
+      a.locate_d[pair] = static_cast<int32_t>(best >> 32);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Launch shapes
+// ---------------------------------------------------------------------------
+
+// Sets the batched kernel's shared memory and returns its resident warps per SM.
+template <int VW, bool kAny>
+cudaError_t lane_setup(int cols, int* warps_per_sm) {
+  const size_t smem = lane_block_smem(VW, cols, kAny);
+  cudaError_t e = cudaFuncSetAttribute(align_batched_kernel<VW, kAny>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(warps_per_sm, align_batched_kernel<VW, kAny>,
+                                                       32, smem);
+}
+
+template <int VW>
+cudaError_t lane_setup_order(int cols, bool any_order, int* warps_per_sm) {
+  return any_order ? lane_setup<VW, true>(cols, warps_per_sm)
+                   : lane_setup<VW, false>(cols, warps_per_sm);
+}
+
+template <int VW>
+void lane_launch(const AlignParams& p, const LanePlan& plan, const BatchArgs& a, cudaStream_t s) {
+  const size_t smem = lane_block_smem(VW, plan.cols, plan.any_order);
+  if (plan.any_order) align_batched_kernel<VW, true><<<plan.warps, 32, smem, s>>>(p, a);
+  else align_batched_kernel<VW, false><<<plan.warps, 32, smem, s>>>(p, a);
+}
+
+template <int VW>
+void locate_launch(const AlignParams& p, const LocateArgs& a, int log_q, cudaStream_t s) {
+  const uint64_t threads = static_cast<uint64_t>(p.n_pairs) << log_q;
+  const uint32_t per = 32u * kLocateWarps;
+  locate_kernel<VW><<<static_cast<uint32_t>((threads + per - 1) / per), per, 0, s>>>(p, a, log_q);
+}
+
+// Windows of 65..128 bases (genasm_wide.cu).
+cudaError_t wide_lane_setup(int vw, int cols, bool any_order, int* warps_per_sm);
+void wide_lane_launch(int vw, const AlignParams& p, const LanePlan& plan, const BatchArgs& a,
+                      cudaStream_t s);
+void wide_locate_launch(int vw, const AlignParams& p, const LocateArgs& a, int log_q, cudaStream_t s);
+
+}  // namespace ga

@@ -8,7 +8,6 @@
 
 #include "genasm.h"
 #include "genasm_internal.h"
-#include "genasm_wide.h"
 #include "genasm_window.cuh"
 
 namespace ga {
@@ -65,37 +64,33 @@ int fill_params(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32
   return GA_OK;
 }
 
-int resolve(int W, int O, int k, const ga_tuning* t, ga::BatchPlan* plan, int mode = 0) {
-  int G = 0, ppb = 0, entries = 0, lpt = 1, regs = 0, slice = 0;
-  cudaError_t e = ga::default_tuning(W, O, k, &G, &ppb, &entries, &lpt, &regs, &slice, mode);
-  if (e != cudaSuccess) return cuda_fail(e);
-  if (t) {
-    if (t->lanes_per_pair) G = t->lanes_per_pair;
-    if (t->pairs_per_block) ppb = t->pairs_per_block;
-    if (t->table_rows) entries = ga::table_entries_for(G, W, O, t->table_rows, ga::band_top_for(O) >= 0);
-    if (t->lpt) lpt = t->lpt > 0 ? 1 : 0;
-    regs = t->max_registers;
-    slice = t->slice_windows;
-    if (!ga::batch_variant_exists(G, regs) || ppb < 1 || ppb * G > 256 || (ppb * G) % 32 != 0 ||
-        t->table_rows < 0 || slice < -1)
-      return GA_EINVAL;
+// Windows wider than 64 bases take no tuning.
+int resolve(int W, int O, int k, const ga_tuning* t, ga_tuning* out, int mode = 0) {
+  if (wide_window(W)) {
+    *out = ga_tuning{8, 8, 39, 1, 0, 0};
+    return GA_OK;
   }
-  e = ga::resolve_plan(W, O, k, G, ppb, entries, lpt, true, plan, regs, slice);
-  if (e == cudaErrorInvalidValue || e == cudaErrorInvalidConfiguration) {
-    cudaGetLastError();
-    return GA_EINVAL;
-  }
-  return cuda_fail(e);
+  const cudaError_t e = ga::resolve_tuning(W, O, k, t, mode, out);
+  return e == cudaErrorInvalidValue ? GA_EINVAL : cuda_fail(e);
 }
 
-int launch_wide_checked(const ga::AlignParams& p, void* d_workspace, size_t ws_bytes,
-                        ga_stream_t stream) {
-  size_t need = 0;
-  const cudaError_t e = ga::wide_workspace_bytes(p.n_pairs, &need);
-  if (e != cudaSuccess) return cuda_fail(e);
-  if (!d_workspace || ws_bytes < need) return GA_ENOSPC;
-  return cuda_fail(
-      ga::launch_wide(p, true, d_workspace, ws_bytes, reinterpret_cast<cudaStream_t>(stream)));
+int workspace_bytes(uint32_t n_pairs, int W, int O, int k, const ga_tuning* t, int mode,
+                    size_t* bytes_out) {
+  if (!bytes_out || bad_wok(W, O, k)) return GA_EINVAL;
+  ga_tuning r;
+  const int rc = resolve(W, O, k, t, &r, mode);
+  if (rc == GA_OK) *bytes_out = ga::workspace_layout(n_pairs).total;
+  return rc;
+}
+
+// The checks and the launch shape of a batched call whose parameters are filled.
+int plan_batched(const ga::AlignParams& p, int k, const ga_tuning* t, int mode, const void* d_workspace,
+                 size_t ws_bytes, ga::LanePlan* plan) {
+  ga_tuning r;
+  const int rc = resolve(p.W, p.O, k, t, &r, mode);
+  if (rc != GA_OK) return rc;
+  if (!d_workspace || ws_bytes < ga::workspace_layout(p.n_pairs).total) return GA_ENOSPC;
+  return cuda_fail(ga::lane_plan(p, r.slice_windows, r.lpt > 0, plan));
 }
 
 }  // namespace
@@ -127,24 +122,12 @@ int ga_pack_2bit(const uint8_t* d_ascii, uint64_t n_chars, uint8_t* d_packed,
 }
 
 int ga_workspace_size(uint32_t n_pairs, int W, int O, int k, size_t* bytes_out) {
-  if (!bytes_out || bad_wok(W, O, k)) return GA_EINVAL;
-  if (wide_window(W)) return cuda_fail(ga::wide_workspace_bytes(n_pairs, bytes_out));
-  ga::BatchPlan plan{};
-  const int rc = resolve(W, O, k, nullptr, &plan);
-  if (rc != GA_OK) return rc;
-  *bytes_out = ga::workspace_layout(n_pairs, plan).total;
-  return GA_OK;
+  return workspace_bytes(n_pairs, W, O, k, nullptr, 0, bytes_out);
 }
 
 int ga_workspace_size_tuned(uint32_t n_pairs, int W, int O, int k, const ga_tuning* tuning,
                             size_t* bytes_out) {
-  if (!bytes_out || bad_wok(W, O, k)) return GA_EINVAL;
-  if (wide_window(W)) return cuda_fail(ga::wide_workspace_bytes(n_pairs, bytes_out));
-  ga::BatchPlan plan{};
-  const int rc = resolve(W, O, k, tuning, &plan);
-  if (rc != GA_OK) return rc;
-  *bytes_out = ga::workspace_layout(n_pairs, plan).total;
-  return GA_OK;
+  return workspace_bytes(n_pairs, W, O, k, tuning, 0, bytes_out);
 }
 
 uint64_t ga_launch_count(void) { return ga::launch_count(); }
@@ -194,12 +177,9 @@ int ga_align_batch_tuned(const uint8_t* d_reads, const uint64_t* d_read_off,
                        d_n_windows, d_cells, &p);
   if (rc != GA_OK) return rc;
   if (n_pairs == 0) return GA_OK;
-  if (wide_window(W)) return launch_wide_checked(p, d_workspace, ws_bytes, stream);
-  ga::BatchPlan plan{};
-  rc = resolve(W, O, k, tuning, &plan);
+  ga::LanePlan plan{};
+  rc = plan_batched(p, k, tuning, 0, d_workspace, ws_bytes, &plan);
   if (rc != GA_OK) return rc;
-  const ga::WorkspaceLayout L = ga::workspace_layout(n_pairs, plan);
-  if (!d_workspace || ws_bytes < L.total) return GA_ENOSPC;
   return cuda_fail(ga::launch_batched(p, plan, d_workspace, reinterpret_cast<cudaStream_t>(stream)));
 }
 
@@ -221,24 +201,15 @@ int ga_align_batch_order(const uint8_t* d_reads, const uint64_t* d_read_off,
   if (rc != GA_OK) return rc;
   if (n_pairs == 0) return GA_OK;
   p.tb_table = ga::tb_table(static_cast<uint32_t>(tb_order));
-  if (wide_window(W)) return launch_wide_checked(p, d_workspace, ws_bytes, stream);
-  ga::BatchPlan plan{};
-  rc = resolve(W, O, k, nullptr, &plan);
+  ga::LanePlan plan{};
+  rc = plan_batched(p, k, nullptr, 0, d_workspace, ws_bytes, &plan);
   if (rc != GA_OK) return rc;
-  const ga::WorkspaceLayout L = ga::workspace_layout(n_pairs, plan);
-  if (!d_workspace || ws_bytes < L.total) return GA_ENOSPC;
   return cuda_fail(ga::launch_batched(p, plan, d_workspace, reinterpret_cast<cudaStream_t>(stream)));
 }
 
 int ga_workspace_size_locate(uint32_t n_pairs, int W, int O, int k, const ga_tuning* tuning,
                              size_t* bytes_out) {
-  if (!bytes_out || bad_wok(W, O, k)) return GA_EINVAL;
-  if (wide_window(W)) return cuda_fail(ga::wide_workspace_bytes(n_pairs, bytes_out));
-  ga::BatchPlan plan{};
-  const int rc = resolve(W, O, k, tuning, &plan, 1);
-  if (rc != GA_OK) return rc;
-  *bytes_out = ga::workspace_layout(n_pairs, plan).total;
-  return GA_OK;
+  return workspace_bytes(n_pairs, W, O, k, tuning, 1, bytes_out);
 }
 
 int ga_align_batch_locate_tuned(const uint8_t* d_reads, const uint64_t* d_read_off,
@@ -257,19 +228,9 @@ int ga_align_batch_locate_tuned(const uint8_t* d_reads, const uint64_t* d_read_o
   if (rc != GA_OK) return rc;
   if (n_pairs > 0 && (!d_start_span || !d_ref_start)) return GA_EINVAL;
   if (n_pairs == 0) return GA_OK;
-  if (wide_window(W)) {  // 128-bit windows: the wide locate step and kernel (no tuning)
-    size_t need = 0;
-    const cudaError_t e = ga::wide_workspace_bytes(n_pairs, &need);
-    if (e != cudaSuccess) return cuda_fail(e);
-    if (!d_workspace || ws_bytes < need) return GA_ENOSPC;
-    return cuda_fail(ga::launch_wide_locate(p, d_start_span, d_ref_start, d_workspace, ws_bytes,
-                                            reinterpret_cast<cudaStream_t>(stream)));
-  }
-  ga::BatchPlan plan{};
-  rc = resolve(W, O, k, tuning, &plan, 1);
+  ga::LanePlan plan{};
+  rc = plan_batched(p, k, tuning, 1, d_workspace, ws_bytes, &plan);
   if (rc != GA_OK) return rc;
-  const ga::WorkspaceLayout L = ga::workspace_layout(n_pairs, plan);
-  if (!d_workspace || ws_bytes < L.total) return GA_ENOSPC;
   return cuda_fail(ga::launch_batched_locate(p, plan, d_start_span, d_ref_start, d_workspace,
                                              reinterpret_cast<cudaStream_t>(stream)));
 }
@@ -323,7 +284,6 @@ int ga_align_ablation(const uint8_t* d_reads, const uint64_t* d_read_off,
                              d_cigar_off, d_n_runs, d_n_windows, d_cells, &p);
   if (rc != GA_OK) return rc;
   if (n_pairs == 0) return GA_OK;
-  p.band_top = -1;
   size_t need = 0;
   const cudaError_t e = ga::ablation_workspace_bytes(n_pairs, variant, &need);
   if (e != cudaSuccess) return cuda_fail(e);

@@ -23,7 +23,6 @@ struct AlignParams {
   const uint32_t* ref_len;
   uint32_t n_pairs;
   int W, O, kmax;  // kmax = min(k, W): no window needs rows above W
-  int band_top;    // band tables for windows that are not the last (-1: wide only); set by the launchers
   uint64_t tb_table;  // traceback decision table (tb_table(order) in genasm_window.cuh)
   int32_t* dist;
   int32_t* status;
@@ -44,17 +43,15 @@ struct AlignParams {
   int32_t* locate_d;
 };
 
-// Resolved tuning of the batched kernel.
-struct BatchPlan {
-  int lanes_per_pair;   // G (each lane owns 64 / G text columns)
-  int pairs_per_block;  // groups per block
-  int table_entries;    // 64-bit table entries per group kept in shared memory
-  int lpt;              // longest-first hand-out
-  int band_top;         // band table offset A, or -1 (wide tables only)
-  int blocks;           // persistent grid size
-  size_t smem_bytes;    // dynamic shared memory per block
-  int max_registers;    // register cap of the kernel variant (0: none)
-  int slice_windows;    // windows per turn of the sliced queue (0: automatic, -1: off)
+// Launch shape of the batched kernel (one lane per pair, one-warp blocks).
+struct LanePlan {
+  int vw;          // 32-bit words per window vector
+  int cols;        // columns of a lane's table
+  int warps;       // persistent grid size
+  int lanes;       // lanes of a warp that take pairs
+  bool any_order;  // a traceback order other than the default
+  bool lpt;        // longest-first hand-out
+  uint32_t slice;  // windows per turn of the sliced queue (0: off)
 };
 
 // Workspace layout of the batched kernel (byte offsets).
@@ -66,7 +63,6 @@ struct WorkspaceLayout {
   size_t ring;    // uint32[2 n_pairs]: slots of the sliced queue's ring
   size_t ring_seq;  // uint32[2 n_pairs]: their sequence numbers
   size_t state;   // SlotState[n_pairs]: window state of pairs between turns
-  size_t spill;   // uint64[groups][kMaxRows * kMaxCols]
   size_t total;
 };
 
@@ -85,28 +81,21 @@ struct StepArgs {
                            // [2] active slots, [3] windows per step (set before each step)
   SlotState* state;        // per slot
   uint32_t* done;          // slots that finished this step
-  uint64_t* spill;         // [groups][65 * 66]
-  int table_entries;
+  int cols;                // columns of a lane's table
 };
 
 // The serving step kernel reads its active count and window budget from
 // device memory (counters[2], counters[3]), so one captured launch serves every
-// step. prepare_step sets the kernel's shared-memory attribute (once, outside
-// any capture); launch_step launches it; launch_step_copyout copies the
+// step. prepare_step fills the launch shape for windows of W <= 64 bases and
+// sets the kernel's shared-memory attribute (once, outside any capture); launch_step launches it; launch_step_copyout copies the
 // finished count and the finished slots into host-mapped memory after it.
-cudaError_t prepare_step(const BatchPlan& plan);
-cudaError_t launch_step(const AlignParams& p, const BatchPlan& plan, const StepArgs& a,
+cudaError_t prepare_step(int W, LanePlan* plan);
+cudaError_t launch_step(const AlignParams& p, const LanePlan& plan, const StepArgs& a,
                         cudaStream_t s);
 cudaError_t launch_step_copyout(const uint32_t* counters, const uint32_t* done,
                                 uint32_t* host_count, uint32_t* host_done, cudaStream_t s);
-bool step_variant_exists(int G);
 
-WorkspaceLayout workspace_layout(uint32_t n_pairs, const BatchPlan& plan);
-
-// Windows of 65..128 bases (genasm_wide.cu): 128-bit vectors, tables in the
-// workspace, one warp per pair, pairs longest first when lpt is set.
-cudaError_t wide_workspace_bytes(uint32_t n_pairs, size_t* bytes);
-cudaError_t launch_wide(const AlignParams& p, bool lpt, void* ws, size_t ws_bytes, cudaStream_t s);
+WorkspaceLayout workspace_layout(uint32_t n_pairs);
 
 // Ablation kernels (genasm_ablation.cu): variant 0..3, see ga_align_ablation.
 // Bounds of the sliced queue's waits (polls; 0 = the default of seconds).
@@ -143,35 +132,23 @@ cudaError_t launch_compact(const uint32_t* cigar, const uint64_t* cigar_off, con
 cudaError_t launch_pack(const uint8_t* ascii, uint64_t n, uint8_t* packed, uint32_t* n_invalid,
                         cudaStream_t s);
 cudaError_t launch_plain(const AlignParams& p, cudaStream_t s);
-// spill_area = false runs without the per-group global spill area (the kernel
-// gets a null spill pointer): only for plans whose shared tables hold every
-// error row of a wide window and that use no band tables, so that no window
-// can need it.
-cudaError_t launch_batched(const AlignParams& p, const BatchPlan& plan, void* ws, cudaStream_t s,
-                           bool spill_area = true);
+cudaError_t launch_batched(const AlignParams& p, const LanePlan& plan, void* ws, cudaStream_t s);
 
 // The batched alignment with a free-start first window: the locate kernel
 // over every pair (start spans d_start_span, starts into d_ref_start), then
 // the batched kernel starting each pair there.
-cudaError_t launch_batched_locate(const AlignParams& p, const BatchPlan& plan,
+cudaError_t launch_batched_locate(const AlignParams& p, const LanePlan& plan,
                                   const uint32_t* start_span, int32_t* ref_start, void* ws,
                                   cudaStream_t s);
 
-// Default tuning for (W, O, k) on the current device (the stored one of
-// `mode`, else the library's); fills G / pairs per block / table entries /
-// lpt / register cap. Returns cudaSuccess or the device query error.
-cudaError_t default_tuning(int W, int O, int k, int* G, int* ppb, int* table_entries, int* lpt,
-                           int* max_registers, int* slice_windows, int mode = 0);
-bool batch_variant_exists(int G, int max_registers = 0);
-cudaError_t resolve_plan(int W, int O, int k, int G, int ppb, int table_entries, int lpt,
-                         bool band, BatchPlan* plan, int max_registers = 0, int slice_windows = 0);
-uint32_t slice_for(uint32_t n_pairs, const BatchPlan& plan);
+// The tuning in force for (W, O, k) on the current device: `t` (nullptr: none)
+// over the stored one of `mode` over the library's. cudaErrorInvalidValue for
+// one that names no launch shape.
+cudaError_t resolve_tuning(int W, int O, int k, const struct ga_tuning_s* t, int mode,
+                           struct ga_tuning_s* out);
 
-// Band tables (32-bit entries around the diagonal) are used for windows that
-// are not the last when O >= 16, with offset A = min(22, O - 1). Table sizes
-// in 64-bit words for `rows` rows of a window that is not the last, and back.
-int band_top_for(int O);
-int table_entries_for(int G, int W, int O, int rows, bool band);
-int table_rows_for(int G, int W, int O, int entries, bool band);
+// Launch shape of the batched kernel for p (p.n_pairs, W, O, order) on the
+// current device; slice_windows and lpt as in ga_tuning.
+cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePlan* plan);
 
 }  // namespace ga

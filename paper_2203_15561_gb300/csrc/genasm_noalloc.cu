@@ -9,10 +9,10 @@
 // latency-critical loop may not afford cudaMalloc, which can synchronize the
 // device. They pass inputs and outputs and nothing else.
 //
-// How it differs from ga_align_batch: the same persistent work-queue kernel,
-// run with every window's table sized for all 65 error rows in shared memory,
-// so no window ever needs the global spill area; the queue counter, the
-// longest-first histogram and the pair order use the static array below.
+// How it differs from ga_align_batch: the same persistent work-queue kernel
+// without turns (the sliced queue's ring and window states need memory); the
+// queue counter, the longest-first histogram and the pair order use the
+// static array below.
 #include <cstdint>
 #include <mutex>
 
@@ -92,22 +92,11 @@ extern "C" int ga_align_batch_noalloc(const uint8_t* d_reads, const uint64_t* d_
   p.n_windows = d_n_windows;
   p.cells = d_cells;
 
-  // 16 lanes per pair, 2 pairs per block, and a wide table of 65 rows x 66
-  // entries per pair: every window fits in shared memory, so the kernel
-  // never needs a spill area (and runs without band tables, whose overflow
-  // would need one).
-  constexpr int kAllRows = ga::kMaxRows * ga::kMaxStride + ga::kPmCols;
-  ga::BatchPlan plan{};
-  cudaError_t e = ga::resolve_plan(W, O, k, 16, 2, kAllRows, 1, false, &plan);
-  if (e == cudaErrorInvalidValue || e == cudaErrorInvalidConfiguration) {
-    cudaGetLastError();  // a refused launch shape, not a sticky error
-    return GA_EINVAL;
-  }
+  // No sliced queue: its ring and window states are not in the scratch.
+  ga::LanePlan plan{};
+  cudaError_t e = ga::lane_plan(p, -1, true, &plan);
   if (e != cudaSuccess) return ga::cuda_fail(e);
-  // The kernel runs without a spill area: every window must fit the shared
-  // table (all 65 rows of a wide table), and no band table may overflow.
-  if (plan.table_entries < kAllRows || plan.band_top >= 0) return GA_EINVAL;
-  const ga::WorkspaceLayout L = ga::workspace_layout(n_pairs, plan);
+  const ga::WorkspaceLayout L = ga::workspace_layout(n_pairs);
   if (L.order != kOrderOffset || L.order + 4ull * n_pairs > kScratchBytes) return GA_ENOSPC;
 
   void* scratch = nullptr;
@@ -115,7 +104,6 @@ extern "C" int ga_align_batch_noalloc(const uint8_t* d_reads, const uint64_t* d_
   if (se != 0) return ga::cuda_fail(static_cast<cudaError_t>(se));
   // launch_batched clears the queue counters and the histogram (the array
   // keeps the previous call's contents) and rebuilds the pair order.
-  e = ga::launch_batched(p, plan, scratch, reinterpret_cast<cudaStream_t>(stream),
-                         /*spill_area=*/false);
+  e = ga::launch_batched(p, plan, scratch, reinterpret_cast<cudaStream_t>(stream));
   return ga::cuda_fail(e);
 }

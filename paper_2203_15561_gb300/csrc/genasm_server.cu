@@ -284,7 +284,7 @@ unsigned copy_workers() {
 struct ga_server {
   int W = 64, O = 24, k = 64, device = 0;
   uint32_t max_windows = 32;
-  ga::BatchPlan plan{};
+  ga::LanePlan plan{};
   cudaStream_t stream = nullptr;
   std::chrono::steady_clock::time_point t0;
   // device arenas
@@ -300,7 +300,6 @@ struct ga_server {
   uint32_t *d_n_runs = nullptr, *d_n_windows = nullptr;
   ga::SlotState* d_state = nullptr;
   uint32_t *d_active = nullptr, *d_done = nullptr, *d_counters = nullptr;
-  uint64_t* d_spill = nullptr;
   uint64_t* d_list = nullptr;    // gather list (3 x uint64 per pair)
   uint32_t* d_out = nullptr;     // gathered runs of finished requests
   uint64_t out_cap = 0;
@@ -386,7 +385,6 @@ void server_free(ga_server* s) {
   cudaFree(s->d_active);
   cudaFree(s->d_done);
   cudaFree(s->d_counters);
-  cudaFree(s->d_spill);
   cudaFree(s->d_list);
   cudaFree(s->d_out);
   cudaFreeHost(s->h_ascii);
@@ -466,17 +464,14 @@ ga::AlignParams step_params(const ga_server* s) {
 
 // Captures the step's device work into a graph (once, at creation).
 cudaError_t capture_step(ga_server* s) {
-  cudaError_t e = ga::prepare_step(s->plan);
-  if (e != cudaSuccess) return e;
   ga::StepArgs a{};
   a.active = s->d_active;
   a.counters = s->d_counters;
   a.state = s->d_state;
   a.done = s->d_done;
-  a.spill = s->d_spill;
-  a.table_entries = s->plan.table_entries;
+  a.cols = s->plan.cols;
   const uint64_t before = ga_launch_count();
-  e = cudaStreamBeginCapture(s->cstream, cudaStreamCaptureModeThreadLocal);
+  cudaError_t e = cudaStreamBeginCapture(s->cstream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
   cudaError_t e1 = cudaMemsetAsync(s->d_counters, 0, 8, s->cstream);
   if (e1 == cudaSuccess) e1 = ga::launch_step(step_params(s), s->plan, a, s->cstream);
@@ -503,32 +498,18 @@ extern "C" int ga_server_create(size_t budget_bytes, int W, int O, int k, ga_ser
   s->copies.reset(new CopyPool(copy_workers()));
   s->pending_cap = std::min<uint64_t>(std::max<uint64_t>(budget_bytes / 16, 64ull << 20), 2ull << 30);
   cudaError_t e = cudaGetDevice(&s->device);
-  // Step kernel tuning: the stored/default tuning when it has a step variant.
-  ga_tuning t{};
-  int G = 8, ppb = 8, rows = 39;
-  if (ga_tuning_get(W, O, k, &t) == GA_OK && ga::step_variant_exists(t.lanes_per_pair) &&
-      t.max_registers == 0) {
-    G = t.lanes_per_pair;
-    ppb = t.pairs_per_block;
-    rows = t.table_rows;
-  }
-  if (e == cudaSuccess)
-    e = ga::resolve_plan(W, O, k, G, ppb,
-                         ga::table_entries_for(G, W, O, rows, ga::band_top_for(O) >= 0), 1, true,
-                         &s->plan);
+  if (e == cudaSuccess) e = ga::prepare_step(W, &s->plan);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->cstream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev_admit, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev_step, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev_staged, cudaEventDisableTiming);
   // Fixed parts first, then the arenas from what is left of the budget.
-  const uint64_t groups = static_cast<uint64_t>(s->plan.blocks) * s->plan.pairs_per_block;
-  const uint64_t spill_bytes = groups * 8ull * ga::kMaxRows * ga::kMaxStride;
   s->max_slots = static_cast<uint32_t>(std::min<uint64_t>(1u << 20, budget_bytes / 8192 + 64));
   const uint64_t per_slot = 8 * 4 + 4 * 6 + 4 * 2 + sizeof(ga::SlotState);
   const uint64_t staging =
       std::min(kAsciiStagingMax, std::max(kAsciiStagingMin, static_cast<uint64_t>(budget_bytes) / 8));
-  const uint64_t fixed = spill_bytes + staging + kOutRuns * 4 + kListPairs * (24 + 4 + 16) +
+  const uint64_t fixed = staging + kOutRuns * 4 + kListPairs * (24 + 4 + 16) +
                          kAdmitRequests * sizeof(ga::PackSegment) +
                          kAdmitPairs * sizeof(ga::SlotRecord) +
                          static_cast<uint64_t>(s->max_slots) * per_slot;
@@ -560,7 +541,6 @@ extern "C" int ga_server_create(size_t budget_bytes, int W, int O, int k, ga_ser
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_active, M);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_done, M);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_counters, 64);
-  if (e == cudaSuccess) e = dev_alloc(s, &s->d_spill, spill_bytes / 8);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_list, 3 * kListPairs);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_out, kOutRuns);
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_ascii, staging);

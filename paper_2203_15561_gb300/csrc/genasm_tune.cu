@@ -1,19 +1,16 @@
 // Autotuner and CUDA-graph capture of the batched alignment step.
 //
-// Autotuner: the batched kernel's speed depends on how many lanes work on a
-// pair (G; each lane owns 64/G text columns), how many pairs share a block and how many table rows a window keeps in shared memory (which sets
-// how many pairs fit on an SM). The best choice depends on the workload's
-// typical d_min. ga_autotune measures a d_min estimate on the caller's sample,
-// times a candidate set on it with CUDA events, and stores the fastest as the
-// default for (device, W, O, k); ga_align_batch and ga_workspace_size use the
-// stored default from then on.
+// Autotuner: how fast a batch runs depends on the order in which its pairs are
+// handed out and on the windows per turn of the sliced queue. ga_autotune times
+// a candidate set on the caller's batch with CUDA events and stores the fastest
+// as the default for (device, W, O, k); ga_align_batch uses the stored default
+// from then on.
 //
 // Graph: ga_graph_create captures one whole step (2-bit packing of the ASCII
 // inputs, the workspace reset, the longest-first ordering and the alignment
 // kernel) into a CUDA graph for fixed buffers; ga_graph_launch replays it with
 // one call.
 #include <algorithm>
-#include <cmath>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -67,29 +64,12 @@ int bad_wok(int W, int O, int k) {
   return W < 1 || W > GA_MAX_W_ONCHIP || O < 0 || O >= W || k < 0;
 }
 
-// Candidate tunings for a workload whose windows keep about `rows` rows:
-// lanes per pair, pairs per block, two table sizes, and for eight-lane groups
-// the register-capped variants (which pay off when small tables leave room
-// for more blocks per SM).
-std::vector<ga_tuning> candidates(int rows) {
-  // `rows` is the mean d_min + 1; windows whose d_min does not fit are redone in
-  // global memory, so larger tables that cover the tail of d_min are tried too.
-  const int lo = std::min(65, std::max(4, rows + 5));
-  const int hi = std::min(65, std::max(6, rows + 8));
-  // The mean hides the windows that lose the read's path (random-versus-random
-  // windows with d_min near 32 amid windows near 8): the library's 39 rows,
-  // which hold those too, are always a candidate.
-  const int tail = std::min(65, std::max(8, rows + 16));
-  std::vector<int> row_set;
-  for (int r : {lo, hi, tail, 39})
-    if (std::find(row_set.begin(), row_set.end(), r) == row_set.end()) row_set.push_back(r);
+// Candidate tunings: hand-out order and windows per turn. (The batched kernel
+// runs one lane per pair; the launch shape follows from the number of pairs.)
+std::vector<ga_tuning> candidates() {
   std::vector<ga_tuning> c;
-  const int shapes[][2] = {{4, 8}, {4, 16}, {8, 4}, {8, 8}, {16, 2}, {16, 4}, {32, 1}, {32, 2}};
-  for (const auto& s : shapes)
-    for (int r : row_set) c.push_back(ga_tuning{s[0], s[1], r, 1, 0, 0});
-  for (int regs : {168, 128})
-    for (int ppb : {4, 8})
-      for (int r : row_set) c.push_back(ga_tuning{8, ppb, r, 1, regs, 0});
+  for (int lpt : {1, -1})
+    for (int slice : {0, -1, 32, 64, 128}) c.push_back(ga_tuning{8, 8, 39, lpt, 0, slice});
   return c;
 }
 
@@ -98,11 +78,7 @@ std::vector<ga_tuning> candidates(int rows) {
 extern "C" int ga_tuning_get(int W, int O, int k, ga_tuning* out) {
   if (!out || bad_wok(W, O, k)) return GA_EINVAL;
   if (ga::stored_tuning(W, O, k, out)) return GA_OK;
-  int G, ppb, entries, lpt, regs, slice;
-  if (ga::default_tuning(W, O, k, &G, &ppb, &entries, &lpt, &regs, &slice) != cudaSuccess)
-    return GA_ECUDA;
-  *out = ga_tuning{G, ppb, ga::table_rows_for(G, W, O, entries, ga::band_top_for(O) >= 0),
-                   lpt ? 1 : -1, regs, slice};
+  *out = ga_tuning{8, 8, 39, 1, 0, 0};
   return GA_OK;
 }
 
@@ -120,11 +96,9 @@ extern "C" int ga_tuning_set(int W, int O, int k, const ga_tuning* t) {
 extern "C" int ga_autotune_workspace_size(uint32_t n_pairs, int W, int O, int k, size_t* bytes) {
   if (!bytes || bad_wok(W, O, k)) return GA_EINVAL;
   size_t best = 0;
-  for (int rows : {4, 16, 32, 40, 61, 65}) {
-    for (const ga_tuning& t : candidates(rows)) {
-      size_t b = 0;
-      if (ga_workspace_size_tuned(n_pairs, W, O, k, &t, &b) == GA_OK) best = std::max(best, b);
-    }
+  for (const ga_tuning& t : candidates()) {
+    size_t b = 0;
+    if (ga_workspace_size_tuned(n_pairs, W, O, k, &t, &b) == GA_OK) best = std::max(best, b);
   }
   size_t b = 0;
   const int rc = ga_workspace_size(n_pairs, W, O, k, &b);
@@ -173,29 +147,14 @@ int autotune(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_t*
   const bool locate = d_start_span != nullptr;
   const int mode = locate ? 1 : 0;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  // 1. d_min estimate: run the current default once with statistics.
+  // One run with statistics: they are part of the call's outputs.
   int rc = align_once(d_reads, d_read_off, d_read_len, d_refs, d_ref_off, d_ref_len, n_pairs, W, O,
                       k, d_start_span, d_ref_start, d_dist, d_status, d_ref_consumed, d_cigar,
                       d_cigar_off, d_n_runs, d_n_windows, d_cells, d_workspace, ws_bytes, nullptr,
                       stream);
   if (rc != GA_OK) return rc;
-  const uint32_t n_probe = std::min<uint32_t>(n_pairs, 4096);
-  std::vector<uint32_t> nw(n_probe);
-  std::vector<uint64_t> cells(n_probe);
-  if (cudaMemcpyAsync(nw.data(), d_n_windows, 4ull * n_probe, cudaMemcpyDeviceToHost, s) !=
-          cudaSuccess ||
-      cudaMemcpyAsync(cells.data(), d_cells, 8ull * n_probe, cudaMemcpyDeviceToHost, s) !=
-          cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
-    return GA_ECUDA;
-  double tw = 0, tc = 0;
-  for (uint32_t q = 0; q < n_probe; ++q) {
-    tw += nw[q];
-    tc += static_cast<double>(cells[q]);
-  }
-  const int rows = tw > 0 ? static_cast<int>(std::ceil(tc / (tw * W))) : 8;  // mean d_min + 1
 
-  // 2. time every candidate (one warm-up run, then one timed run).
+  // Time every candidate (one warm-up run, then one timed run).
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return GA_ECUDA;
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -205,7 +164,7 @@ int autotune(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_t*
   float best_t = 1e30f;
   ga_tuning best_c{};
   rc = GA_OK;
-  for (const ga_tuning& c : candidates(rows)) {
+  for (const ga_tuning& c : candidates()) {
     size_t need = 0;
     if (workspace_for(n_pairs, W, O, k, &c, locate, &need) != GA_OK || need > ws_bytes) continue;
     int r1 = align_once(d_reads, d_read_off, d_read_len, d_refs, d_ref_off, d_ref_len, n_pairs, W,

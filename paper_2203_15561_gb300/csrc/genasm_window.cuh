@@ -1,5 +1,7 @@
-// Device code for GenASM windows processed by groups of G lanes, shared by
-// the plain and the batched alignment kernels.
+// Device code for GenASM windows in the paper's row form, processed by groups
+// of G lanes: the plain kernel (G = 32) and the ablation of the improvements
+// (G = 8). The batched kernel computes the same windows as edit-distance
+// columns (genasm_lane.cuh).
 //
 // A warp holds 32/G groups; each group works on its own (read, reference)
 // pair, one window at a time. Every loop below runs with warp-uniform trip
@@ -8,9 +10,8 @@
 //
 // Per window (pattern = read window P of wp <= 64 bases, text = reference
 // window T of wt <= 64 bases) a group
-//   1. builds the pattern masks PM[c] (bit j clear iff P[wp-1-j] == c) from
-//      the window's bases, prefetched into registers one window ahead, and
-//      each lane's columns PM[T[i]] in registers;
+//   1. builds the pattern masks PM[c] (bit j clear iff P[wp-1-j] == c) and the
+//      columns PM[T[i]], each lane's own in registers;
 //   2. runs the distance calculation (DC) as a wavefront over text columns:
 //      lane c owns 64/G consecutive columns and computes one error row per
 //      step, one row behind lane c+1, whose leftmost cell it receives with
@@ -103,18 +104,6 @@ __device__ __forceinline__ void st1_if(bool p, uint64_t* a, uint64_t x) {
       ::"l"(a), "l"(x), "r"(static_cast<uint32_t>(p)) : "memory");
 }
 
-__device__ __forceinline__ void st32x4_if(bool p, uint32_t a, uint32_t x, uint32_t y, uint32_t z,
-                                          uint32_t w) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\t@q st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n\t}"
-      ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w), "r"(static_cast<uint32_t>(p)) : "memory");
-}
-__device__ __forceinline__ void st32x2_if(bool p, uint32_t a, uint32_t x, uint32_t y) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q st.shared.v2.u32 [%0], {%1, %2};\n\t}"
-      ::"r"(a), "r"(x), "r"(y), "r"(static_cast<uint32_t>(p)) : "memory");
-}
-
 // Table addressing: a shared-memory table by 32-bit shared address, the
 // global spill table by pointer.
 template <bool kShared>
@@ -139,140 +128,12 @@ __device__ __forceinline__ uint32_t group_bits(uint32_t ballot, int gbase) {
 }
 
 // Columns of the per-window PM[T[i]] buffer: 0..wt-1 hold the masks, wt..63
-// hold all ones ("virtual" text columns past the window end). The 64-bit
-// buffer (pmcol) lives in the last kPmCols words of the group's table area:
-// a band window needs it only until its DC has loaded it into registers, a
-// wide window keeps it out of its table rows.
+// hold all ones ("virtual" text columns past the window end).
 constexpr int kPmCols = kMaxW;
 
-// Shared-memory working set of one group besides its table area.
-struct GroupSmem {
-  uint32_t pmb[kPmCols];  // band windows: PM[T[i]] in band coordinates
-};
-
-// Step 1: the window's bases, pattern masks and PM[T[i]] columns.
-//
-// Bases come from 8-word blocks of the packed sequences held across the
-// group's lanes (word w in lane w % G, slot w / G). A block is loaded at a
-// window's (word-aligned) start and serves that window and the next one:
-// a window advances at most W-O bases, so the next window's 64 bases lie in
-// the same 128-base block for W-O <= 49. The group loads the block for the
-// next window while the current one runs, so its latency is hidden; the
-// first window of a pair (or one past its block) loads its block directly.
-constexpr int kPfWords = 8;
-
-struct SeqBlock {
-  uint32_t w[2];  // this lane's words of the block (slot 1 only when G < 8)
-  uint32_t pos;   // the base position the block was loaded at
-  uint32_t o0;    // bit offset of that base in word 0
-};
-
-// Loads the block holding bases pos.. of `seq` (len bases) for groups with
-// go set. Only words that hold a base of the sequence are read.
-template <int G>
-__device__ __forceinline__ void load_block(bool go, int r, const uint8_t* seq, uint32_t len,
-                                           uint32_t pos, SeqBlock& b) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(seq) + (pos >> 2);
-  const uint32_t* wa = reinterpret_cast<const uint32_t*>(a & ~static_cast<uintptr_t>(3));
-  const uint32_t o0 = 8u * static_cast<uint32_t>(a & 3u) + 2u * (pos & 3u);
-  const uint64_t lim = o0 + 2ull * (len > pos ? len - pos : 0u);  // first bit past the sequence
-#pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    const int wi = r + s * G;
-    const bool v = go && (s == 0 || G < kPfWords) && wi < kPfWords &&
-                   32ull * static_cast<uint64_t>(wi) < lim;
-    b.w[s] = v ? __ldg(wa + wi) : 0u;
-  }
-  b.pos = pos;
-  b.o0 = o0;
-}
-
-// The 64 bases starting at `pos` (inside block b) as 4 words, base pos+u at
-// bits 2u%32.. of word u/16; every lane of the group receives them.
-template <int G>
-__device__ __forceinline__ void block_window(int gbase, const SeqBlock& b, uint32_t pos,
-                                             uint32_t (&out)[4]) {
-  const uint32_t o = b.o0 + 2u * (pos - b.pos);
-  const int k0 = static_cast<int>(min(o >> 5, static_cast<uint32_t>(kPfWords - 1)));
-  const uint32_t sh = o & 31u;
-  uint32_t x[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    const int wi = min(k0 + k, kPfWords - 1);
-    const uint32_t mine = (G < kPfWords && wi >= G) ? b.w[1] : b.w[0];
-    x[k] = __shfl_sync(kFull, mine, gbase + (wi & (G - 1)));
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) out[k] = __funnelshift_r(x[k], x[k + 1], sh);
-}
-
-// Bits 0, 2, ..., 30 of x, packed into bits 0..15.
-__device__ __forceinline__ uint32_t even_bits16(uint32_t x) {
-  x &= 0x55555555u;
-  x = (x | (x >> 1)) & 0x33333333u;
-  x = (x | (x >> 2)) & 0x0F0F0F0Fu;
-  x = (x | (x >> 4)) & 0x00FF00FFu;
-  return __byte_perm(x, 0u, 0x4420);
-}
-
-__device__ __forceinline__ uint64_t rev64(uint64_t x) {
-  return (static_cast<uint64_t>(__brev(static_cast<uint32_t>(x))) << 32) |
-         __brev(static_cast<uint32_t>(x >> 32));
-}
-
-// Pattern masks PM[c] (bit j clear iff P[wp-1-j] == c) of the pattern
-// window's 2-bit codes (base u at bits 2u%32.. of word u/16), from the codes'
-// low and high bit planes.
-__device__ __forceinline__ void pattern_masks(int wp, const uint32_t (&P)[4], uint64_t& pm0,
-                                              uint64_t& pm1, uint64_t& pm2, uint64_t& pm3) {
-  uint32_t l16[4], h16[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    l16[k] = even_bits16(P[k]);
-    h16[k] = even_bits16(P[k] >> 1);
-  }
-  // Bit u of Lu / Hu: low / high code bit of pattern base u.
-  const uint64_t Lu = (static_cast<uint64_t>(__byte_perm(l16[2], l16[3], 0x5410)) << 32) |
-                      __byte_perm(l16[0], l16[1], 0x5410);
-  const uint64_t Hu = (static_cast<uint64_t>(__byte_perm(h16[2], h16[3], 0x5410)) << 32) |
-                      __byte_perm(h16[0], h16[1], 0x5410);
-  // Bit j <-> pattern base wp-1-j (bits at and above wp: zero).
-  const uint32_t sh = static_cast<uint32_t>(64 - wp);
-  const uint64_t L = rev64(Lu) >> sh;
-  const uint64_t H = rev64(Hu) >> sh;
-  pm0 = L | H;     // clear where code 0 (A)
-  pm1 = ~L | H;    // clear where code 1 (C)
-  pm2 = L | ~H;    // clear where code 2 (G)
-  pm3 = ~(L & H);  // clear where code 3 (T)
-}
-
-// Pattern masks and this lane's columns PM[T[c0 + x]] (all ones at
-// c0 + x >= wt).
-template <int G>
-__device__ __forceinline__ void window_masks(int r, int wp, int wt, const uint32_t (&P)[4],
-                                             const uint32_t (&T)[4], uint64_t (&pm)[64 / G]) {
-  constexpr int C = 64 / G;
-  uint64_t pm0, pm1, pm2, pm3;
-  pattern_masks(wp, P, pm0, pm1, pm2, pm3);
-  const int c0 = r * C;
-  const int wi = (2 * c0) >> 5;
-  uint32_t tw = T[0];
-  tw = wi == 1 ? T[1] : tw;
-  tw = wi == 2 ? T[2] : tw;
-  tw = wi == 3 ? T[3] : tw;
-  tw >>= (2 * c0) & 31;
-#pragma unroll
-  for (int x = 0; x < C; ++x) {
-    const uint32_t c = (tw >> (2 * x)) & 3u;
-    const uint64_t v = c == 0 ? pm0 : c == 1 ? pm1 : c == 2 ? pm2 : pm3;
-    pm[x] = c0 + x < wt ? v : ~0ull;
-  }
-}
-
-// Step 1 for wide groups (G >= 16, where a pattern mask takes at most 8
-// ballots): pattern masks by warp ballots over bases loaded directly, then
-// PM[T[i]] per text column into the 64-bit buffer. Groups with ga == false
-// take part in the ballots only.
+// Step 1: pattern masks by warp ballots over the window's bases, then PM[T[i]]
+// per text column into the buffer. Groups with ga == false take part in the
+// ballots only.
 template <int G>
 __device__ __forceinline__ void build_masks(int r, int gbase, bool ga,
                                             const uint8_t* __restrict__ read, uint32_t pos_p,
@@ -318,16 +179,6 @@ __device__ __forceinline__ void build_masks(int r, int gbase, bool ga,
   }
 }
 
-// This lane's PM[T[i]] columns into the 64-bit buffer (groups with go).
-template <int G>
-__device__ __forceinline__ void store_pmcol(bool go, int r, const uint64_t (&pm)[64 / G],
-                                            uint64_t* pmcol) {
-  constexpr int C = 64 / G;
-  const uint32_t a = smem_addr(pmcol + r * C);
-#pragma unroll
-  for (int x = 0; x < C; x += 2) st2_if(go, a + 8u * x, pm[x], pm[x + 1]);
-}
-
 // Steps 2-4: distance calculation with row early termination.
 //
 // Column strips: lane c of the group owns the C = 64/G text columns
@@ -359,28 +210,11 @@ __device__ __forceinline__ void store_pmcol(bool go, int r, const uint64_t (&pm)
 // kDcUnroll - 1 further rows may be computed and stored (rows above d_min are
 // never read).
 //
-// The table `tab` (shared memory, or the global spill area) receives rows
-// below `store_rows` at row stride S, columns below `ncols` (improvements (1)
-// and (3)). Two formats:
-//   kFmtWide  : 64-bit entries R_i[d]; column wt holds R_wt[d] for the
-//               traceback (shared memory or the global spill area).
-//   kFmtBand  : 32-bit entries holding bits [e_i, e_i + 31] of R_i[d] with
-//               e_i = wp - 1 - A - i (A = band_top): the bits around the
-//               diagonal that the traceback can read while its offset
-//               (read bases - text bases committed) stays in [A-30, A-1]
-//               (shared memory; windows that are not the last, with
-//               e_i >= 0 for every stored column).
+// The table `tab` (shared or global memory) receives rows below `store_rows`
+// at row stride S, columns below `ncols` (improvements (1) and (3)), as 64-bit
+// entries R_i[d]; column wt holds R_wt[d] for the traceback.
 // Returns d_min, or -1 if it is above kmax (groups with ga == false get -1).
 constexpr int kDcUnroll = 4;
-enum TableFmt { kFmtWide, kFmtBand };
-
-// Row stride (entries) of a band table with `ncols` stored columns: whole
-// 16-byte chunks of 4 entries (8-byte chunks of 2 when a strip has C = 2
-// columns), each written by one store.
-__host__ __device__ __forceinline__ int band_stride(int G, int ncols) {
-  const int q = G == 32 ? 2 : 4;
-  return (ncols + q - 1) / q * q;
-}
 
 //
 // Two switches serve the ablation of the paper's improvements (defaults: the
@@ -388,13 +222,12 @@ __host__ __device__ __forceinline__ int band_stride(int G, int ncols) {
 // stopping at d_min (plain GenASM); kFour stores, per cell, the four vectors
 // M, S, I, D of plain GenASM (entry 4*(d*S + i) + {0, 1, 2, 3}; wide, global)
 // instead of their AND.
-template <int G, TableFmt kFmt, bool kShared, bool kEt = true, bool kFour = false>
+template <int G, bool kShared, bool kEt = true, bool kFour = false>
 __device__ __forceinline__ int dc_window(int r, int gbase, bool ga, int wp, int wt, int kmax,
-                                         int ncols, int S, int store_rows, int band_top,
-                                         const uint64_t (&pmr)[64 / G], uint32_t* pmb, void* tab) {
+                                         int ncols, int S, int store_rows,
+                                         const uint64_t (&pmr)[64 / G], void* tab) {
   constexpr int C = 64 / G;
-  static_assert(!kFour || (kFmt == kFmtWide && !kShared), "four-vector tables are wide, global");
-  static_assert(kFmt == kFmtWide || kShared, "band tables live in shared memory");
+  static_assert(!kFour || !kShared, "four-vector tables are global");
   const int c0 = r * C;
   uint64_t pm[C];
 #pragma unroll
@@ -408,34 +241,12 @@ __device__ __forceinline__ int dc_window(int r, int gbase, bool ga, int wp, int 
     PS[x] = ~0ull;
   }
   uint64_t Pr = ~0ull, PrS = ~0ull, leftmost = ~0ull, initv = ~0ull;
-  // Wide: the strip's stored columns are [c0, c0 + n_store), written in
-  // pairs (a pair may end in the padding column of an odd-width row, which
-  // the even stride provides); lane G-1 also stores column 64 (= R_wt[d])
-  // when the table needs it. Band: every chunk of the strip that starts
-  // inside the stored columns is written whole (the stride covers whole
-  // chunks).
+  // The strip's stored columns are [c0, c0 + n_store), written in pairs (a
+  // pair may end in the padding column of an odd-width row, which the even
+  // stride provides); lane G-1 also stores column 64 (= R_wt[d]) when the
+  // table needs it.
   const int n_store = max(0, min(C, ncols - c0));
-  const bool store64 = kFmt == kFmtWide && r == G - 1 && ncols > 64;
-  int band_sh[C];
-#pragma unroll
-  for (int x = 0; x < C; ++x) band_sh[x] = max(wp - 1 - band_top - c0 - x, 0);
-  if constexpr (kFmt == kFmtBand) {
-    // The traceback of a band window tests PM[T[i]] in band coordinates
-    // too. After this the 64-bit masks are dead: the band rows may overwrite
-    // them (a window redone with a wide table rebuilds them).
-    __syncwarp();
-    uint32_t pb[C];
-#pragma unroll
-    for (int x = 0; x < C; ++x) pb[x] = static_cast<uint32_t>(pm[x] >> band_sh[x]);
-    const uint32_t pa = smem_addr(pmb) + 4u * static_cast<uint32_t>(c0);
-    if constexpr (C == 2) {
-      st32x2_if(ga, pa, pb[0], pb[1]);
-    } else {
-#pragma unroll
-      for (int x = 0; x + 3 < C; x += 4) st32x4_if(ga, pa + 4u * x, pb[x], pb[x + 1], pb[x + 2], pb[x + 3]);
-    }
-    __syncwarp();
-  }
+  const bool store64 = r == G - 1 && ncols > 64;
   const TableRef<kShared> tref(static_cast<uint64_t*>(tab));
   const uint64_t msb_mask = 1ull << (wp - 1);
   const int t_last = kmax + G - 1;  // the step at which lane 0 computes row kmax
@@ -486,23 +297,11 @@ __device__ __forceinline__ int dc_window(int r, int gbase, bool ga, int wp, int 
           st2_if(st_row && x < n_store, tref.at(4 * (off + x)), V4[4 * x], V4[4 * x + 1]);
           st2_if(st_row && x < n_store, tref.at(4 * (off + x) + 2), V4[4 * x + 2], V4[4 * x + 3]);
         }
-      } else if constexpr (kFmt == kFmtWide) {
+      } else {
 #pragma unroll
         for (int x = 0; x < C; x += 2)
           st2_if(st_row && x < n_store, tref.at(off + x), P[x], P[x + 1]);
         st1_if(st_row && store64, tref.at(off + 64 - c0), right);
-      } else {
-        uint32_t E[C];
-#pragma unroll
-        for (int x = 0; x < C; ++x) E[x] = static_cast<uint32_t>(P[x] >> band_sh[x]);
-        const uint32_t a = tref.base + 4u * static_cast<uint32_t>(off);
-        if constexpr (C == 2) {
-          st32x2_if(st_row && n_store > 0, a, E[0], E[C - 1]);
-        } else {
-#pragma unroll
-          for (int x = 0; x + 3 < C; x += 4)
-            st32x4_if(st_row && x < n_store, a + 4u * x, E[x], E[x + 1], E[x + 2], E[x + 3]);
-        }
       }
       if (first < 0 && static_cast<unsigned>(d) <= static_cast<unsigned>(kmax) &&
           !(P[0] & msb_mask))
@@ -604,12 +403,6 @@ constexpr uint32_t kTbOrderDefault = 0xE4u;
 // done only take part in the votes. Returns false for a group whose walk
 // found no edge (never expected).
 //
-// With a band table (kFmtBand) the bits a lane tests sit at k-1, k and k+1
-// of its entries, k = A - (cp - ct), the same for every lane of the group
-// (the lanes look ahead along one diagonal). A group whose offset leaves the
-// band stops before the iteration that would need it and sets `over`; its
-// caller redoes the window with a wide table.
-//
 // The match edge needs no table entry: the walk only visits active cells,
 // and at an active cell whose bases match, bit j-1 of R_{i+1}[d] is active
 // too (equal leading bases can always be paired at no cost), so M is
@@ -619,13 +412,12 @@ constexpr uint32_t kTbOrderDefault = 0xE4u;
 // kFour walks a plain GenASM four-vector table (see dc_window): at cell (i,
 // d) the edge is M if bit j of M_i[d] is 0 (i < wt), else S, I, D by bit j of
 // S_i[d], I_i[d], D_i[d] (all ones in row 0).
-template <int G, TableFmt kFmt, bool kFour = false>
+template <int G, bool kFour = false>
 __device__ __forceinline__ bool tb_window(int r, int gbase, bool ga, int wp, int wt, int dmin,
-                                          bool last, int commit, int ncols, int S, int band_top,
+                                          bool last, int commit, int ncols, int S,
                                           uint64_t order_table, const uint64_t* pmcol,
-                                          const uint32_t* pmb, const void* tab,
-                                          RunWriter& rw, bool writer, int& cp_out, int& ct_out,
-                                          uint32_t& edits, bool& over) {
+                                          const void* tab, RunWriter& rw, bool writer, int& cp_out,
+                                          int& ct_out, uint32_t& edits) {
   // The walk is at text column ct and pattern bit wp-1-cp.
   int d = dmin, cp = 0, ct = 0;
   bool run = ga, ok = true;
@@ -635,14 +427,6 @@ __device__ __forceinline__ bool tb_window(int r, int gbase, bool ga, int wp, int
   // Columns c and c+1 of a row are read for c <= cmax (always inside the row).
   const int cmax = ncols >= 2 ? ncols - 2 : 0;
   while (__any_sync(kFull, run)) {
-    int kb = 0;
-    if constexpr (kFmt == kFmtBand) {
-      kb = band_top - (cp - ct);
-      const bool in_band = static_cast<unsigned>(kb - 1) <= 29u;
-      over = over || (run && !in_band);
-      run = run && in_band;
-      kb &= 31;
-    }
     // Lanes r >= lim look at or past the stop point (group-uniform).
     const int lim = last ? wp - cp : min(commit - cp, commit - ct);
     const bool stop = r >= lim;
@@ -658,7 +442,7 @@ __device__ __forceinline__ bool tb_window(int r, int gbase, bool ga, int wp, int
       s_ok = (t4[1] & bit) == 0ull;
       i_ok = (t4[2] & bit) == 0ull;
       d_ok = (t4[3] & bit) == 0ull;
-    } else if constexpr (kFmt == kFmtWide) {
+    } else {
       const int jl = wp - 1 - cp - r;
       const uint64_t* tw = static_cast<const uint64_t*>(tab);
       const uint64_t pm = pmcol[min(il, kPmCols - 1)];
@@ -672,18 +456,6 @@ __device__ __forceinline__ bool tb_window(int r, int gbase, bool ga, int wp, int
       s_ok = d > 0 && (s & below) == 0ull;
       i_ok = d > 0 && (in & below) == 0ull;
       d_ok = d > 0 && (s & bit) == 0ull;
-    } else {
-      // Band entries: bit j of PM[T[i]], bit j-1 of column i+1, bit j of
-      // column i+1 and bit j-1 of column i sit at kb, kb, kb+1 and kb-1.
-      const uint32_t* tn = static_cast<const uint32_t*>(tab);
-      const uint32_t pmv = pmb[min(il, kPmCols - 1)];
-      const uint32_t mk = 1u << kb;
-      const uint32_t s = tn[rowm + ic + 1];
-      const uint32_t in = tn[rowm + ic];
-      m_ok = (pmv & mk) == 0u;
-      s_ok = d > 0 && (s & mk) == 0u;
-      i_ok = d > 0 && (in & (mk >> 1)) == 0u;
-      d_ok = d > 0 && (s & (mk << 1)) == 0u;
     }
     uint32_t valid = static_cast<uint32_t>(m_ok) << kTbM | static_cast<uint32_t>(s_ok) << kTbS |
                      static_cast<uint32_t>(i_ok) << kTbI | static_cast<uint32_t>(d_ok) << kTbD;
