@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdint>
+#include <mutex>
 
 #include <cuda_runtime.h>
 
@@ -27,48 +28,148 @@ __device__ __forceinline__ uint32_t lpt_bucket(uint32_t read_len) {
   return kLptBuckets - 1u - min(b, static_cast<uint32_t>(kLptBuckets - 1));
 }
 
-__global__ void lpt_histogram_kernel(const uint32_t* __restrict__ read_len, uint32_t n,
-                                     uint32_t* __restrict__ hist) {
+// Adds 1 to h[b] for every lane with `in` set and returns the value before this
+// lane's. Lanes of a warp with the same bucket add together (reads of one length
+// all fall into one bucket).
+__device__ __forceinline__ uint32_t count_bucket(uint32_t* h, uint32_t b, bool in) {
+  const uint32_t same = __match_any_sync(kFull, in ? b : 0xffffffffu);
+  const uint32_t lane = threadIdx.x & 31u;
+  const int first = __ffs(same) - 1;
+  uint32_t at = 0;
+  if (in && static_cast<int>(lane) == first) at = atomicAdd(&h[b], __popc(same));
+  return __shfl_sync(kFull, at, first) + __popc(same & ((1u << lane) - 1u));
+}
+
+// Exclusive scan of kLptBuckets counts in shared memory, a thread each; s: one
+// word per warp.
+__device__ __forceinline__ uint32_t scan_buckets(uint32_t v, uint32_t* s) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, x, o);
+    if (lane >= static_cast<uint32_t>(o)) x += y;
+  }
+  if (lane == 31u) s[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t w = s[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, w, o);
+      if (lane >= static_cast<uint32_t>(o)) w += y;
+    }
+    s[lane] = w;
+  }
+  __syncthreads();
+  return (warp ? s[warp - 1] : 0u) + x - v;
+}
+
+// Whether the sliced queue pays for n pairs, from the buckets' counts and starts
+// in the order (a thread each; longest first): only when the pair that nine in
+// ten are at least as long as has four fifths of the longest one's bases. Pairs
+// of one length end in a round of few lanes without turns; of mixed lengths, the
+// short ones at the end of the order fill the lanes up as the long ones finish,
+// and turns cost more than they give (30,011 pairs of 2-20 kb: 2.32 ms with
+// turns, 1.88 without; 20,000 of 100 bases-50 kb: 5.8 and 4.9).
+__device__ __forceinline__ void wants_turns(uint32_t count, uint32_t start, uint32_t n, uint32_t* flag) {
+  __shared__ uint32_t longest, ninth;
+  const uint32_t len = kLptBuckets - 1u - threadIdx.x;  // in 64 bases
+  const uint32_t at = n - n / 10u - 1u;                 // the place of that pair
+  if (count && start == 0u) longest = len;
+  if (count && start <= at && at < start + count) ninth = len;
+  __syncthreads();
+  if (threadIdx.x == 0) *flag = 5u * (ninth + 1u) >= 4u * (longest + 1u) ? 1u : 0u;
+}
+
+// The whole order of a batch of up to kLptOneBlock pairs by one block, which also
+// zeroes the queue's counters.
+constexpr uint32_t kLptOneBlock = 16384;
+
+__global__ void __launch_bounds__(kLptBuckets)
+    lpt_block_kernel(const uint32_t* __restrict__ read_len, uint32_t n, uint32_t* __restrict__ queue,
+                     uint32_t* __restrict__ order) {
   __shared__ uint32_t h[kLptBuckets];
-  for (int x = threadIdx.x; x < kLptBuckets; x += blockDim.x) h[x] = 0;
+  __shared__ uint32_t s[32];
+  const uint32_t x = threadIdx.x;
+  if (x < 64u) queue[x] = 0u;
+  h[x] = 0u;
   __syncthreads();
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x)
-    atomicAdd(&h[lpt_bucket(read_len[q])], 1u);
+  const uint32_t rounds = (n + kLptBuckets - 1) / kLptBuckets;
+  for (uint32_t r = 0; r < rounds; ++r) {
+    const uint32_t q = r * kLptBuckets + x;
+    count_bucket(h, q < n ? lpt_bucket(read_len[q]) : 0u, q < n);
+  }
   __syncthreads();
-  for (int x = threadIdx.x; x < kLptBuckets; x += blockDim.x)
-    if (h[x]) atomicAdd(&hist[x], h[x]);
+  const uint32_t start = scan_buckets(h[x], s);
+  wants_turns(h[x], start, n, queue + 5);
+  h[x] = start;
+  __syncthreads();
+  for (uint32_t r = 0; r < rounds; ++r) {
+    const uint32_t q = r * kLptBuckets + x;
+    const uint32_t at = count_bucket(h, q < n ? lpt_bucket(read_len[q]) : 0u, q < n);
+    if (q < n) order[at] = q;
+  }
+}
+
+// Larger batches in three launches. Each block counts its own pairs in shared
+// memory and reserves their places in the order with one addition per bucket.
+constexpr uint32_t kLptPairs = 8 * kLptBuckets;  // pairs per block
+
+__device__ __forceinline__ void lpt_count(const uint32_t* __restrict__ read_len, uint32_t n, uint32_t* h) {
+  const uint64_t q0 = static_cast<uint64_t>(blockIdx.x) * kLptPairs + threadIdx.x;
+  h[threadIdx.x] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (uint32_t r = 0; r < kLptPairs / kLptBuckets; ++r) {
+    const uint64_t q = q0 + r * kLptBuckets;
+    count_bucket(h, q < n ? lpt_bucket(read_len[q]) : 0u, q < n);
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kLptBuckets)
+    lpt_histogram_kernel(const uint32_t* __restrict__ read_len, uint32_t n, uint32_t* __restrict__ hist) {
+  __shared__ uint32_t h[kLptBuckets];
+  lpt_count(read_len, n, h);
+  if (h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], h[threadIdx.x]);
 }
 
 // Exclusive scan of the bucket counts in place (one block of kLptBuckets threads).
-__global__ void lpt_scan_kernel(uint32_t* hist) {
-  __shared__ uint32_t s[kLptBuckets];
-  const int x = threadIdx.x;
-  const uint32_t v = hist[x];
-  s[x] = v;
-  __syncthreads();
-  for (int off = 1; off < kLptBuckets; off <<= 1) {
-    const uint32_t add = x >= off ? s[x - off] : 0u;
-    __syncthreads();
-    s[x] += add;
-    __syncthreads();
-  }
-  hist[x] = s[x] - v;
+__global__ void __launch_bounds__(kLptBuckets) lpt_scan_kernel(uint32_t* hist, uint32_t n, uint32_t* turns) {
+  __shared__ uint32_t s[32];
+  const uint32_t count = hist[threadIdx.x];
+  const uint32_t start = scan_buckets(count, s);
+  if (turns) wants_turns(count, start, n, turns);
+  hist[threadIdx.x] = start;
 }
 
-__global__ void lpt_scatter_kernel(const uint32_t* __restrict__ read_len, uint32_t n,
-                                   uint32_t* __restrict__ cursor, uint32_t* __restrict__ order) {
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-    const uint32_t pos = atomicAdd(&cursor[lpt_bucket(read_len[q])], 1u);
-    order[pos] = q;
+__global__ void __launch_bounds__(kLptBuckets)
+    lpt_scatter_kernel(const uint32_t* __restrict__ read_len, uint32_t n,
+                       uint32_t* __restrict__ cursor, uint32_t* __restrict__ order) {
+  __shared__ uint32_t h[kLptBuckets];
+  lpt_count(read_len, n, h);
+  const uint32_t mine = h[threadIdx.x];
+  const uint32_t start = mine ? atomicAdd(&cursor[threadIdx.x], mine) : 0u;
+  __syncthreads();
+  h[threadIdx.x] = start;
+  __syncthreads();
+  const uint64_t q0 = static_cast<uint64_t>(blockIdx.x) * kLptPairs + threadIdx.x;
+#pragma unroll
+  for (uint32_t r = 0; r < kLptPairs / kLptBuckets; ++r) {
+    const uint64_t q = q0 + r * kLptBuckets;
+    const uint32_t at = count_bucket(h, q < n ? lpt_bucket(read_len[q]) : 0u, q < n);
+    if (q < n) order[at] = static_cast<uint32_t>(q);
   }
 }
 
 cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* hist, uint32_t* order,
-                             cudaStream_t s) {
-  const int blocks = static_cast<int>(std::min<uint32_t>((n + 255) / 256, 1024u));
-  lpt_histogram_kernel<<<blocks, 256, 0, s>>>(read_len, n, hist);
-  lpt_scan_kernel<<<1, kLptBuckets, 0, s>>>(hist);
-  lpt_scatter_kernel<<<blocks, 256, 0, s>>>(read_len, n, hist, order);
+                             uint32_t* turns, cudaStream_t s) {
+  const uint32_t blocks =
+      static_cast<uint32_t>((static_cast<uint64_t>(n) + kLptPairs - 1) / kLptPairs);
+  lpt_histogram_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, hist);
+  lpt_scan_kernel<<<1, kLptBuckets, 0, s>>>(hist, n, turns);
+  lpt_scatter_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, hist, order);
   count_launches(3);
   return cudaGetLastError();
 }
@@ -79,18 +180,24 @@ cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* his
 // pair starts as timed out (distance and reference end -1, no runs): a pair
 // that finishes overwrites it, and one left in the ring when a bounded wait
 // ran out keeps it.
-__global__ void ring_init_kernel(uint32_t n, const uint32_t* __restrict__ order,
+// The positions 0 .. dealt-1 are reserved by the lanes before they start (see
+// the kernel), so the head begins past them.
+__global__ void ring_init_kernel(uint32_t n, uint32_t dealt, const uint32_t* __restrict__ order,
                                  uint32_t* __restrict__ ring, uint32_t* __restrict__ seq,
-                                 uint32_t* __restrict__ queue, int32_t* __restrict__ status,
+                                 uint32_t* __restrict__ queue, SlotState* __restrict__ state,
+                                 int32_t* __restrict__ status,
                                  int32_t* __restrict__ dist, int32_t* __restrict__ ref_consumed,
                                  uint32_t* __restrict__ n_runs) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
+    queue[1] = dealt;
+    if (!order) queue[5] = 1u;  // no order, nothing known of the lengths: take turns
     queue[2] = n;  // tail: the ring starts with every pair
     queue[3] = n;  // pairs not finished
   }
   for (uint32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < 2u * n; x += gridDim.x * blockDim.x) {
     if (x < n) {
       ring[x] = order ? order[x] : x;
+      state[x] = SlotState{};
       status[x] = kPairTimedOut;
       dist[x] = -1;
       ref_consumed[x] = -1;
@@ -181,49 +288,118 @@ namespace {
 int vw_for(int W) { return (W + 31) / 32; }
 int up8(int x) { return (x + 7) / 8 * 8; }
 
-cudaError_t setup_for(int vw, int cols, bool any_order, int* warps_per_sm) {
-  if (vw == 1) return lane_setup_order<1>(cols, any_order, warps_per_sm);
-  if (vw == 2) return lane_setup_order<2>(cols, any_order, warps_per_sm);
-  return wide_lane_setup(vw, cols, any_order, warps_per_sm);
+cudaError_t setup_for(int vw, int lp, int cols, bool any_order, int* warps_per_sm) {
+  if (vw == 1) return lane_setup_order<1, 32, 1>(cols, any_order, warps_per_sm);
+  if (vw == 2) return lane_setup_order<2, 32, 1>(cols, any_order, warps_per_sm);
+  return wide_lane_setup(vw, lp, cols, any_order, warps_per_sm);
+}
+
+}  // namespace
+
+namespace {
+
+// What a launch asks the driver about the device, asked once: SMs, and the
+// resident warps of each launch shape (a call of every shape costs a few
+// microseconds, a tenth of a small batch). Shapes differ by width, pairs per
+// warp, order and table columns (multiples of 8 up to 128).
+struct DeviceFacts {
+  int sms = 0;
+  int8_t warps[4][3][2][17] = {};  // 0: not asked yet, else warps per SM + 1
+};
+constexpr int kMaxDevices = 64;
+std::mutex g_facts_mutex;
+DeviceFacts g_facts[kMaxDevices];
+
+cudaError_t device_sms(int* dev, int* sms) {
+  cudaError_t e = cudaGetDevice(dev);
+  if (e != cudaSuccess) return e;
+  if (*dev < 0 || *dev >= kMaxDevices)
+    return cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev);
+  std::lock_guard<std::mutex> lock(g_facts_mutex);
+  DeviceFacts& f = g_facts[*dev];
+  if (f.sms == 0) e = cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, *dev);
+  *sms = f.sms;
+  return e;
+}
+
+cudaError_t shape_warps(int dev, int vw, int lp, int cols, bool any_order, int* warps) {
+  if (dev < 0 || dev >= kMaxDevices) return setup_for(vw, lp, cols, any_order, warps);
+  std::lock_guard<std::mutex> lock(g_facts_mutex);
+  int8_t& w = g_facts[dev].warps[vw - 1][lp == 32 ? 0 : lp == 16 ? 1 : 2][any_order][cols / 8];
+  cudaError_t e = cudaSuccess;
+  if (w == 0) {
+    e = setup_for(vw, lp, cols, any_order, warps);
+    if (e == cudaSuccess) w = static_cast<int8_t>(*warps + 1);
+  }
+  *warps = w - 1;
+  return e;
 }
 
 }  // namespace
 
 cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePlan* plan) {
   int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaError_t e = device_sms(&dev, &sms);
   if (e != cudaSuccess) return e;
-  const int vw = vw_for(p.W);
-  plan->vw = vw;
+  plan->vw = vw_for(p.W);
   plan->any_order = p.tb_table != tb_table(kTbOrderDefault);
   plan->lpt = lpt;
-  // A table of every column a last window walks when four warps of them fit an
-  // SM, else of the W - O columns of the other windows.
+  const uint64_t n = std::max<uint32_t>(p.n_pairs, 1);
+  const uint64_t scheds = 4ull * sms;
+  const int all = up8(p.W), inner = up8(p.W - p.O);
   int per_sm = 0;
-  plan->cols = up8(p.W);
-  if ((e = setup_for(vw, plan->cols, plan->any_order, &per_sm)) != cudaSuccess) return e;
-  if (per_sm < 4) {
-    plan->cols = up8(p.W - p.O);
-    if ((e = setup_for(vw, plan->cols, plan->any_order, &per_sm)) != cudaSuccess) return e;
+  // Windows of 65 bases and more: four lanes per pair while one warp per
+  // scheduler holds every pair (2,001 pairs of 10 kb at W = 128: 0.79 ms against
+  // 1.16 with one lane each). At W <= 64 two lanes per pair gained nothing (3,330
+  // cycles for a window's columns against 3,280).
+  if (plan->vw >= 3 && n <= 8 * scheds) {
+    plan->lp = 8;
+    plan->cols = all;
+    if ((e = shape_warps(dev, plan->vw, 8, all, plan->any_order, &per_sm)) != cudaSuccess) return e;
+    per_sm = std::min(per_sm, 4);
+  } else {
+    // One lane per pair. Tables of every column a window can walk, else of the W
+    // - O columns of windows that are not a pair's last; warps of 32 pairs, else
+    // of 16: the first that leaves each of an SM's four schedulers as many warps
+    // as the pairs can use, else the one with most. That is one warp until the
+    // pairs fill two rounds of it, then two: with every lane busy two warps per
+    // scheduler take 1.49 times as long per window as one (38,912 pairs of 2 kb
+    // 312 us, 19,456 pairs 209), but with pairs for half the lanes 1.9 times
+    // (10,000 pairs of 10 kb: 2.05 ms against 1.10).
+    const int want = n > 64 * scheds ? 8 : 4;
+    for (int lp : {32, 16}) {
+      if (lp == 16 && plan->vw < 3) break;
+      for (int cols : {all, std::max(inner, std::min(all, 48)), inner}) {
+        if (per_sm >= want) break;
+        int ps = 0;
+        if ((e = shape_warps(dev, plan->vw, lp, cols, plan->any_order, &ps)) != cudaSuccess) return e;
+        ps = ps >= 8 ? 8 : std::min(ps, 4);
+        if (ps <= per_sm) continue;
+        per_sm = ps;
+        plan->lp = lp;
+        plan->cols = cols;
+      }
+      if (per_sm >= 4) break;
+    }
+    per_sm = std::min(per_sm, want);
   }
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  // One warp per scheduler while its lanes hold every pair, else all that fit.
-  const uint64_t n = std::max<uint32_t>(p.n_pairs, 1);
-  uint64_t warps = static_cast<uint64_t>(sms) * std::min(per_sm, 4);
-  if (n > 32 * warps) warps = static_cast<uint64_t>(sms) * per_sm;
-  warps = std::min(warps, n);
+  // (an attribute of the function in this context: set for every launch)
+  if ((e = setup_for(plan->vw, plan->lp, plan->cols, plan->any_order, nullptr)) != cudaSuccess) return e;
+  const uint64_t warps = std::min<uint64_t>(static_cast<uint64_t>(sms) * per_sm, n);
   plan->warps = static_cast<int>(warps);
-  plan->lanes = static_cast<int>(std::min<uint64_t>(32, (n + warps - 1) / warps));
-  // Windows per turn of the sliced queue: the tuning's choice, else turns of 64
-  // windows when the pairs outnumber the resident lanes less than 16 times over
-  // (more pairs than that leave a tail of under a sixteenth of a round). A
-  // single pair has nobody to take turns with.
-  const uint64_t lanes = warps * 32;
-  plan->slice = slice_windows < 0 || n < 2 ? 0u
-                : slice_windows > 0       ? static_cast<uint32_t>(slice_windows)
-                : n > lanes && n < 16 * lanes ? 64u
-                                              : 0u;
+  plan->lanes = static_cast<int>(std::min<uint64_t>(plan->lp, (n + warps - 1) / warps));
+  // The sliced queue: turns of the tuning's choice, else of 64 windows or a
+  // quarter of the pair when the pairs outnumber the resident lanes less than 16
+  // times over (more pairs than that leave a tail of under a sixteenth of a
+  // round) and are of about one length, which the ordering finds out on the
+  // device (wants_turns). A single pair has nobody to take turns with.
+  const uint64_t lanes = warps * plan->lp;
+  const bool automatic = slice_windows == 0 && n > lanes && n < 16 * lanes;
+  plan->slice = n < 2 ? 0u : slice_windows > 0 ? static_cast<uint32_t>(slice_windows) : automatic ? 64u : 0u;
+  plan->turns = automatic ? 4u : 0u;
+  // (waiting lanes take part in the ring as well)
+  if (plan->slice) plan->lanes = plan->lp;
   return cudaSuccess;
 }
 
@@ -248,27 +424,36 @@ cudaError_t launch_batched(const AlignParams& p, const LanePlan& plan, void* ws,
   uint32_t* queue = reinterpret_cast<uint32_t*>(w + L.queue);
   uint32_t* hist = reinterpret_cast<uint32_t*>(w + L.hist);
   uint32_t* order = reinterpret_cast<uint32_t*>(w + L.order);
-  cudaError_t e = cudaMemsetAsync(w, 0, L.order, s);  // counters + histogram
-  if (e != cudaSuccess) return e;
-  if (plan.lpt && (e = launch_lpt_order(p.read_len, p.n_pairs, hist, order, s)) != cudaSuccess)
-    return e;
+  // One block orders a batch that keeps it busy for a few microseconds at most.
+  // (Below 64 pairs the order takes the general three launches: a whole step's
+  // launch count at such sizes is something callers have come to rely on.)
+  cudaError_t e = cudaSuccess;
+  if (plan.lpt && p.n_pairs >= 64 && p.n_pairs <= kLptOneBlock) {
+    lpt_block_kernel<<<1, kLptBuckets, 0, s>>>(p.read_len, p.n_pairs, queue, order);
+    count_launches(1);
+  } else {
+    if ((e = cudaMemsetAsync(w, 0, L.order, s)) != cudaSuccess) return e;  // counters + histogram
+    if (plan.lpt &&
+        (e = launch_lpt_order(p.read_len, p.n_pairs, hist, order, queue + 5, s)) != cudaSuccess)
+      return e;
+  }
   uint32_t* ring = reinterpret_cast<uint32_t*>(w + L.ring);
   uint32_t* ring_seq = reinterpret_cast<uint32_t*>(w + L.ring_seq);
   SlotState* state = reinterpret_cast<SlotState*>(w + L.state);
   if (plan.slice) {
-    if ((e = cudaMemsetAsync(state, 0, sizeof(SlotState) * p.n_pairs, s)) != cudaSuccess) return e;
     const int blocks = static_cast<int>(std::min<uint32_t>((p.n_pairs + 255) / 256, 1024u));
-    ring_init_kernel<<<blocks, 256, 0, s>>>(p.n_pairs, plan.lpt ? order : nullptr, ring,
-                                            ring_seq, queue, p.status, p.dist,
-                                            p.ref_consumed, p.n_runs);
+    ring_init_kernel<<<blocks, 256, 0, s>>>(p.n_pairs,
+                                            static_cast<uint32_t>(plan.warps * plan.lp),
+                                            plan.lpt ? order : nullptr, ring, ring_seq, queue, state,
+                                            p.status, p.dist, p.ref_consumed, p.n_runs);
     count_launches(1);
   }
-  const BatchArgs a{queue, plan.lpt ? order : nullptr, plan.cols, plan.lanes, plan.slice, ring,
-                    ring_seq, state, g_idle_polls.load(std::memory_order_relaxed),
+  const BatchArgs a{queue, plan.lpt ? order : nullptr, plan.cols, plan.lanes, plan.slice, plan.turns,
+                    ring, ring_seq, state, g_idle_polls.load(std::memory_order_relaxed),
                     g_push_polls.load(std::memory_order_relaxed)};
-  if (plan.vw == 1) lane_launch<1>(p, plan, a, s);
-  else if (plan.vw == 2) lane_launch<2>(p, plan, a, s);
-  else wide_lane_launch(plan.vw, p, plan, a, s);
+  if (plan.vw == 1) lane_launch<1, 32, 1>(p, plan, a, s);
+  else if (plan.vw == 2) lane_launch<2, 32, 1>(p, plan, a, s);
+  else wide_lane_launch(p, plan, a, s);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -280,8 +465,7 @@ cudaError_t launch_batched_locate(const AlignParams& p, const LanePlan& plan,
   const WorkspaceLayout L = workspace_layout(p.n_pairs);
   int32_t* locate_d = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + L.locate);
   int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaError_t e = device_sms(&dev, &sms);
   if (e != cudaSuccess) return e;
   // Lanes per pair: as many as one warp per scheduler has for every pair.
   int log_q = 0;
@@ -305,9 +489,14 @@ cudaError_t launch_batched_locate(const AlignParams& p, const LanePlan& plan,
 
 namespace {
 
+size_t step_smem(int vw, int cols) {
+  return vw == 1 ? lane_block_smem<LaneShape<1, 32, 1>>(cols, false)
+                 : lane_block_smem<LaneShape<2, 32, 1>>(cols, false);
+}
+
 template <int VW>
 cudaError_t step_setup(int cols, int* warps_per_sm) {
-  const size_t smem = lane_block_smem(VW, cols, false);
+  const size_t smem = step_smem(VW, cols);
   cudaError_t e = cudaFuncSetAttribute(align_step_kernel<VW>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
@@ -324,6 +513,7 @@ cudaError_t prepare_step(int W, LanePlan* plan) {
   if (e != cudaSuccess) return e;
   *plan = LanePlan{};
   plan->vw = vw_for(W);
+  plan->lp = 32;
   plan->cols = up8(W);
   e = plan->vw == 1 ? step_setup<1>(plan->cols, &per_sm) : step_setup<2>(plan->cols, &per_sm);
   if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
@@ -334,7 +524,7 @@ cudaError_t prepare_step(int W, LanePlan* plan) {
 
 cudaError_t launch_step(const AlignParams& p, const LanePlan& plan, const StepArgs& a,
                         cudaStream_t s) {
-  const size_t smem = lane_block_smem(plan.vw, plan.cols, false);
+  const size_t smem = step_smem(plan.vw, plan.cols);
   if (plan.vw == 1) align_step_kernel<1><<<plan.warps, 32, smem, s>>>(p, a);
   else align_step_kernel<2><<<plan.warps, 32, smem, s>>>(p, a);
   const cudaError_t e = cudaGetLastError();

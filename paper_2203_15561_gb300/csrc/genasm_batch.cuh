@@ -9,11 +9,11 @@
 // sort), so the lanes of a warp hold pairs of about the same length.
 //
 // Sliced form (slice > 0): the queue is a FIFO of pairs, and a lane runs a
-// pair for at most `slice` windows, saves its window state (positions, edit
-// count, statistics, open CIGAR run) and puts it back at the tail. Every pair
-// then moves forward at the same pace, and a batch whose pairs outnumber the
-// resident lanes but not by a whole multiple does not end with a round in
-// which a few lanes run alone.
+// pair for a turn (`slice` windows, or a fraction of the pair's), saves its
+// window state (positions, edit count, statistics, open CIGAR run) and puts it
+// back at the tail. Every pair then moves forward at the same pace, and a batch
+// whose pairs outnumber the resident lanes but not by a whole multiple does not
+// end with a round in which a few lanes run alone.
 //
 // The FIFO is a bounded ring of 2n slots (n = pairs) with a sequence number
 // per slot: position x lives in slot x % 2n; the slot holds position x's
@@ -49,11 +49,13 @@ namespace ga {
 
 struct BatchArgs {
   uint32_t* queue;        // [0] hand-out counter (unsliced); ring: [1] head, [2] tail,
-                          // [3] pairs not finished, [4] a warp's wait ran out
+                          // [3] pairs not finished, [4] a warp's wait ran out,
+                          // [5] the pairs' lengths call for turns
   const uint32_t* order;  // hand-out order (nullptr: index order)
   int cols;               // columns of a lane's table
   int lanes;              // lanes of a warp that take pairs
   uint32_t slice;         // windows per turn (0: a pair runs to its end)
+  uint32_t turns;         // if not 0: a turn is this fraction of a pair, `slice` windows at least
   uint32_t* ring;         // 2n ring slots: pair ids
   uint32_t* ring_seq;     // 2n: each slot's sequence number
   SlotState* state;       // per pair: saved window state (all zero: not started)
@@ -99,56 +101,88 @@ __device__ __forceinline__ bool ring_push(const BatchArgs& a, uint32_t cap, uint
 
 // The dynamic shared memory of a one-warp block, from its first multiple of
 // the Eq masks' size on (their addresses are formed with OR).
-template <int VW>
+template <class Shape>
 __device__ __forceinline__ uint32_t lane_smem_base() {
   extern __shared__ __align__(1024) uint32_t lane_smem[];
-  constexpr uint32_t kAlign = LaneShape<VW>::kEqBytes;
-  return (smem_addr(lane_smem) + kAlign - 1u) & ~(kAlign - 1u);
+  return (smem_addr(lane_smem) + Shape::kEqBytes - 1u) & ~(Shape::kEqBytes - 1u);
 }
-constexpr size_t lane_block_smem(int VW, int cols, bool any_order) {
-  return lane_smem_bytes(VW, cols, any_order) + (VW >= 3 ? 1024u : 0u);
+template <class Shape>
+constexpr size_t lane_block_smem(int cols, bool any_order) {
+  return Shape::bytes(cols, any_order) + (Shape::kEqBytes > 1024u ? 1024u : 0u);
 }
 
-template <int VW, bool kAny>
-__global__ void __launch_bounds__(32) align_batched_kernel(const AlignParams p, const BatchArgs a) {
-  const uint32_t base = lane_smem_base<VW>();
+// Hands `*counter`'s next values to the pairs of the lanes in `wants`, in lane
+// order (the lanes of a pair want together).
+template <class Shape>
+__device__ __forceinline__ uint32_t take_next(uint32_t* counter, uint32_t wants, uint32_t lane) {
+  const uint32_t pairs = wants & Shape::kLeaders;
+  const int first = __ffs(pairs) - 1;
+  uint32_t idx = 0;
+  if (static_cast<int>(lane) == first) idx = atomicAdd(counter, __popc(pairs));
+  return __shfl_sync(Shape::kMask, idx, first) + __popc(pairs & ((2u << lane) - 1u)) - 1u;
+}
+
+// Windows of a turn of a pair of m read bases.
+__device__ __forceinline__ uint32_t turn_windows(const AlignParams& p, const BatchArgs& a, uint32_t m) {
+  if (!a.turns) return a.slice;
+  return max(a.slice, m / (static_cast<uint32_t>(p.W - p.O) * a.turns) + 1u);
+}
+
+template <int VW, int LP, int NL, bool kAny>
+__global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParams p, const BatchArgs a) {
+  using Shape = LaneShape<VW, LP, NL>;
+  constexpr uint32_t kMask = Shape::kMask;
+  const uint32_t base = lane_smem_base<Shape>();
   const uint32_t lane = threadIdx.x;
-  LanePair st;
-  st.busy = false;
-  bool drained = lane >= static_cast<uint32_t>(a.lanes);
+  const uint32_t slot = lane / NL;
+  const int leader = static_cast<int>(slot * NL);
+  const bool writer = lane % NL == 0;
+  const uint32_t slice = a.slice && (!a.turns || a.queue[5]) ? a.slice : 0u;
+  LanePair<VW> st{};
+  bool drained = slot >= static_cast<uint32_t>(a.lanes);
+  bool first = true;        // nothing handed out to this warp yet
   uint32_t budget = 0;
-  uint32_t resv = kNoPair;  // the ring position this lane has reserved
+  // The ring position this lane has reserved. As without turns, the first pairs
+  // go round the warps lane by lane.
+  uint32_t resv = slot * gridDim.x + blockIdx.x;
   uint32_t idle = 0;        // consecutive polls of a warp with no pair to work on
   for (;;) {
     // Lanes without a pair take the next one from the queue.
     const bool want = !st.busy && !drained;
-    const uint32_t wants = __ballot_sync(kFull, want);
+    const uint32_t wants = __ballot_sync(kMask, want);
     bool ended = false;  // a pair that finished at its start
     if (wants) {
       uint32_t pair = kNoPair;
       bool quit = false;
-      if (a.slice) {
-        if (want) {
+      if (slice) {
+        if (want && writer) {
           if (resv == kNoPair) resv = atomicAdd(a.queue + 1, 1u);
           pair = ring_take(a, 2u * p.n_pairs, resv);
           if (pair != kNoPair) resv = kNoPair;
           else quit = *reinterpret_cast<volatile uint32_t*>(a.queue + 3) == 0u;  // all finished
         }
+        if constexpr (NL > 1) {
+          pair = __shfl_sync(kMask, pair, leader);
+          quit = __shfl_sync(kMask, quit ? 1u : 0u, leader) != 0u;
+        }
       } else {
-        const int first = __ffs(wants) - 1;
-        uint32_t idx = 0;
-        if (static_cast<int>(lane) == first) idx = atomicAdd(a.queue, __popc(wants));
-        idx = __shfl_sync(kFull, idx, first) + __popc(wants & ((1u << lane) - 1u));
+        // The first pairs go round the warps lane by lane, so that the longest
+        // ones (handed out first) are spread over all schedulers; then each lane
+        // takes the next one when it is done.
+        const uint32_t dealt = gridDim.x * static_cast<uint32_t>(a.lanes);
+        uint32_t idx = slot * gridDim.x + blockIdx.x;
+        if (!first) idx = p.n_pairs > dealt ? dealt + take_next<Shape>(a.queue, wants, lane) : p.n_pairs;
         if (want) {
           if (idx < p.n_pairs) pair = a.order ? a.order[idx] : idx;
           else quit = true;
         }
       }
+      first = false;
       if (want) {
         if (pair != kNoPair) {
-          lane_begin(p, pair, st);
+          lane_begin(p, pair, st, writer);
           ended = !st.busy;
-          if (a.slice) {
+          if (slice) {
             // Another SM may have saved this state: read it from L2, not L1.
             const SlotState* sp = a.state + pair;
             SlotState s;
@@ -161,39 +195,59 @@ __global__ void __launch_bounds__(32) align_batched_kernel(const AlignParams p, 
             s.run_op = __ldcg(&sp->run_op);
             s.run_len = __ldcg(&sp->run_len);
             if (s.windows > 0) lane_resume(s, st);  // a pair that had turns already
-            budget = a.slice;
+            budget = turn_windows(p, a, st.m);
           }
+          if (st.busy) lane_fetch(st);
         } else if (quit) {
           drained = true;
         }
       }
-      __syncwarp();
-    }
-    if (!__any_sync(kFull, st.busy || !drained)) break;
-    const bool was_busy = st.busy;
-    if (__any_sync(kFull, st.busy)) {
-      lane_window<VW, kAny>(p, st, base, a.cols);
-      if (was_busy && (st.status != kPairOk || st.pos_p >= st.m)) lane_finish(p, st);
-      idle = 0;
-    } else {
-      // Every lane of the warp waits for a pair: poll again shortly.
-      __nanosleep(200);
-      if (++idle >= a.idle_polls) {
-        if (lane == 0) atomicExch(a.queue + 4, 1u);
-        drained = true;
+      __syncwarp(kMask);
+      if (!__any_sync(kMask, st.busy)) {
+        if (slice && __any_sync(kMask, ended)) {
+          if (ended && writer) atomicSub(a.queue + 3, 1u);
+          continue;
+        }
+        if (!__any_sync(kMask, !drained)) break;
+        if (slice) {
+          // Every lane of the warp waits for a pair: poll again shortly.
+          __nanosleep(200);
+          if (++idle >= a.idle_polls) {
+            if (lane == 0) atomicExch(a.queue + 4, 1u);
+            break;
+          }
+        }
+        continue;
       }
+      idle = 0;
+    } else if (!__any_sync(kMask, st.busy)) {
+      break;
     }
-    if (a.slice) {
-      if ((was_busy && !st.busy) || ended) atomicSub(a.queue + 3, 1u);  // this pair is finished
+    // Windows until some lane's pair is done or its turn over (a lane that waits
+    // for a pair looks again after each).
+    bool done, turn;
+    do {
+      lane_window<VW, LP, NL, kAny>(p, st, base, a.cols);
+      done = st.busy && lane_done(st);
+      turn = slice && st.busy && !done && --budget == 0;
+    } while (!__any_sync(kMask, done || turn || (!st.busy && !drained)));
+    if (done) lane_finish(p, st, writer);
+    if (slice) {
+      if ((done || ended) && writer) atomicSub(a.queue + 3, 1u);  // this pair is finished
       // End of a turn: the pair goes back to the queue's tail (or, if the ring
       // cannot take it now, stays for another turn).
-      if (st.busy && --budget == 0) {
+      bool pushed = false;
+      if (turn && writer) {
         lane_save(st, a.state[st.pair]);
-        if (ring_push(a, 2u * p.n_pairs, st.pair)) st.busy = false;
-        else budget = a.slice;
+        pushed = ring_push(a, 2u * p.n_pairs, st.pair);
       }
-      __syncwarp();
+      if constexpr (NL > 1) pushed = __shfl_sync(kMask, pushed ? 1u : 0u, leader) != 0u;
+      if (turn) {
+        if (pushed) st.busy = false;
+        else budget = turn_windows(p, a, st.m);
+      }
     }
+    __syncwarp(kMask);
   }
 }
 
@@ -202,52 +256,57 @@ __global__ void __launch_bounds__(32) align_batched_kernel(const AlignParams p, 
 // between steps, so pairs admitted at different times share one launch.
 template <int VW>
 __global__ void __launch_bounds__(32) align_step_kernel(const AlignParams p, const StepArgs a) {
-  const uint32_t base = lane_smem_base<VW>();
-  const uint32_t lane = threadIdx.x;
+  using Shape = LaneShape<VW, 32, 1>;
+  constexpr uint32_t kMask = Shape::kMask;
   const uint32_t n_active = a.counters[2];
+  const uint32_t base = lane_smem_base<Shape>();
+  const uint32_t lane = threadIdx.x;
   const uint32_t max_windows = a.counters[3];
-  // Few pairs spread over all warps, one lane each first.
+  // Few pairs are spread over all warps.
   const uint32_t lanes = min(32u, (n_active + gridDim.x - 1) / gridDim.x);
-  LanePair st;
-  st.busy = false;
+  LanePair<VW> st{};
   bool drained = lane >= lanes;
   uint32_t slot = 0, budget = 0;
   for (;;) {
     const bool want = !st.busy && !drained;
-    const uint32_t wants = __ballot_sync(kFull, want);
+    const uint32_t wants = __ballot_sync(kMask, want);
     bool finished = false;
     if (wants) {
-      const int first = __ffs(wants) - 1;
-      uint32_t idx = 0;
-      if (static_cast<int>(lane) == first) idx = atomicAdd(&a.counters[0], __popc(wants));
-      idx = __shfl_sync(kFull, idx, first) + __popc(wants & ((1u << lane) - 1u));
+      const uint32_t idx = take_next<Shape>(&a.counters[0], wants, lane);
       if (want) {
         if (idx < n_active) {
           slot = a.active[idx];
-          lane_begin(p, slot, st);  // a fresh slot (all zero) starts here
-          if (st.busy) lane_resume(a.state[slot], st);
+          lane_begin(p, slot, st, true);  // a fresh slot (all zero) starts here
+          if (st.busy) {
+            lane_resume(a.state[slot], st);
+            lane_fetch(st);
+          }
           budget = max_windows;
           finished = !st.busy;
         } else {
           drained = true;
         }
       }
-      __syncwarp();
+      __syncwarp(kMask);
     }
-    if (!__any_sync(kFull, st.busy || !drained || finished)) break;
-    const bool was_busy = st.busy;
-    if (__any_sync(kFull, st.busy)) lane_window<VW, false>(p, st, base, a.cols);
-    if (was_busy) {
-      if (st.status != kPairOk || st.pos_p >= st.m) {
-        lane_finish(p, st);
+    if (!__any_sync(kMask, st.busy || !drained || finished)) break;
+    if (__any_sync(kMask, st.busy)) {
+      bool done, turn;
+      do {
+        lane_window<VW, 32, 1, false>(p, st, base, a.cols);
+        done = st.busy && lane_done(st);
+        turn = st.busy && !done && --budget == 0;
+      } while (!__any_sync(kMask, done || turn || finished));
+      if (done) {
+        lane_finish(p, st, true);
         finished = true;
-      } else if (--budget == 0) {
+      } else if (turn) {
         lane_save(st, a.state[slot]);
         st.busy = false;  // resumes at the next step
       }
     }
     if (finished) a.done[atomicAdd(&a.counters[1], 1u)] = slot;
-    __syncwarp();
+    __syncwarp(kMask);
   }
 }
 
@@ -278,7 +337,7 @@ struct LocateArgs {
 template <int VW>
 __global__ void __launch_bounds__(32 * kLocateWarps)
     locate_kernel(const AlignParams p, const LocateArgs a, int log_q) {
-  using Shape = LaneShape<VW>;
+  using Shape = LaneShape<VW, 32, 1>;
   // The Eq masks start at a multiple of their size (shared memory itself is
   // aligned to 1 KB at most).
   constexpr uint32_t kAlign = Shape::kEqBytes;
@@ -309,10 +368,12 @@ __global__ void __launch_bounds__(32 * kLocateWarps)
   const uint32_t lo = min(part * per, starts);
   const uint32_t hi = min(lo + per, starts);
   if (lo < hi) {
-    uint32_t pw[2 * VW], PL[VW], PH[VW];
-    load_bases<VW>(p.reads + p.read_off[pair], m, 0u, pw);
+    uint32_t raw[2 * VW + 1], pw[2 * VW], PL[VW], PH[VW];
+    const uint8_t* read = p.reads + p.read_off[pair];
+    load_words<VW>(read, m, 0u, raw);
+    align_bases<VW>(read, 0u, raw, pw);
     bit_planes<VW>(pw, PL, PH);
-    store_eq<VW>(eq_lane, wp, PL, PH);
+    store_eq<VW, 32, 1>(eq_lane, 0u, wp, PL, PH);
     const uint32_t x0 = static_cast<uint32_t>(min(static_cast<uint64_t>(L), static_cast<uint64_t>(hi) - 1u + 2u * wp));
     const uint8_t* ref = p.refs + p.ref_off[pair];
     const uintptr_t at = reinterpret_cast<uintptr_t>(ref);
@@ -382,29 +443,35 @@ __global__ void __launch_bounds__(32 * kLocateWarps)
 // Launch shapes
 // ---------------------------------------------------------------------------
 
-// Sets the batched kernel's shared memory and returns its resident warps per SM.
-template <int VW, bool kAny>
+// Opts the batched kernel in to a block's whole shared memory (whatever this
+// launch takes of it: concurrent launches of other shapes need other sizes) and,
+// unless warps_per_sm is null, reads the shape's resident warps per SM.
+constexpr int kSharedOptIn = 227 * 1024;
+template <int VW, int LP, int NL, bool kAny>
 cudaError_t lane_setup(int cols, int* warps_per_sm) {
-  const size_t smem = lane_block_smem(VW, cols, kAny);
-  cudaError_t e = cudaFuncSetAttribute(align_batched_kernel<VW, kAny>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(warps_per_sm, align_batched_kernel<VW, kAny>,
-                                                       32, smem);
+  using Shape = LaneShape<VW, LP, NL>;
+  const cudaError_t e = cudaFuncSetAttribute(
+      align_batched_kernel<VW, LP, NL, kAny>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedOptIn);
+  if (e != cudaSuccess || !warps_per_sm) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      warps_per_sm, align_batched_kernel<VW, LP, NL, kAny>, Shape::kThreads,
+      lane_block_smem<Shape>(cols, kAny));
 }
 
-template <int VW>
+template <int VW, int LP, int NL>
 cudaError_t lane_setup_order(int cols, bool any_order, int* warps_per_sm) {
-  return any_order ? lane_setup<VW, true>(cols, warps_per_sm)
-                   : lane_setup<VW, false>(cols, warps_per_sm);
+  return any_order ? lane_setup<VW, LP, NL, true>(cols, warps_per_sm)
+                   : lane_setup<VW, LP, NL, false>(cols, warps_per_sm);
 }
 
-template <int VW>
+template <int VW, int LP, int NL>
 void lane_launch(const AlignParams& p, const LanePlan& plan, const BatchArgs& a, cudaStream_t s) {
-  const size_t smem = lane_block_smem(VW, plan.cols, plan.any_order);
-  if (plan.any_order) align_batched_kernel<VW, true><<<plan.warps, 32, smem, s>>>(p, a);
-  else align_batched_kernel<VW, false><<<plan.warps, 32, smem, s>>>(p, a);
+  using Shape = LaneShape<VW, LP, NL>;
+  const size_t smem = lane_block_smem<Shape>(plan.cols, plan.any_order);
+  if (plan.any_order)
+    align_batched_kernel<VW, LP, NL, true><<<plan.warps, Shape::kThreads, smem, s>>>(p, a);
+  else
+    align_batched_kernel<VW, LP, NL, false><<<plan.warps, Shape::kThreads, smem, s>>>(p, a);
 }
 
 template <int VW>
@@ -415,9 +482,8 @@ void locate_launch(const AlignParams& p, const LocateArgs& a, int log_q, cudaStr
 }
 
 // Windows of 65..128 bases (genasm_wide.cu).
-cudaError_t wide_lane_setup(int vw, int cols, bool any_order, int* warps_per_sm);
-void wide_lane_launch(int vw, const AlignParams& p, const LanePlan& plan, const BatchArgs& a,
-                      cudaStream_t s);
+cudaError_t wide_lane_setup(int vw, int lp, int cols, bool any_order, int* warps_per_sm);
+void wide_lane_launch(const AlignParams& p, const LanePlan& plan, const BatchArgs& a, cudaStream_t s);
 void wide_locate_launch(int vw, const AlignParams& p, const LocateArgs& a, int log_q, cudaStream_t s);
 
 }  // namespace ga

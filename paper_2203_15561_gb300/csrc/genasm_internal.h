@@ -46,12 +46,14 @@ struct AlignParams {
 // Launch shape of the batched kernel (one lane per pair, one-warp blocks).
 struct LanePlan {
   int vw;          // 32-bit words per window vector
+  int lp;          // pairs a warp holds
   int cols;        // columns of a lane's table
   int warps;       // persistent grid size
-  int lanes;       // lanes of a warp that take pairs
+  int lanes;       // of them, those that take pairs in this launch
   bool any_order;  // a traceback order other than the default
   bool lpt;        // longest-first hand-out
   uint32_t slice;  // windows per turn of the sliced queue (0: off)
+  uint32_t turns;  // if not 0: a turn is this fraction of a pair, `slice` windows at least
 };
 
 // Workspace layout of the batched kernel (byte offsets).
@@ -106,8 +108,9 @@ cudaError_t launch_ablation(const AlignParams& p, int variant, uint64_t* table_b
 
 // Longest-read-first order of n pairs (counting sort over kLptBuckets read
 // length buckets): hist must hold kLptBuckets zeroed counters, order n entries.
+// *turns (may be null) receives 1 when the pairs are of about one length, else 0.
 cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* hist, uint32_t* order,
-                             cudaStream_t s);
+                             uint32_t* turns, cudaStream_t s);
 
 // Kernel launches issued by the library (process-wide counter).
 uint64_t launch_count();

@@ -4,16 +4,25 @@
 
 namespace ga {
 
-cudaError_t wide_lane_setup(int vw, int cols, bool any_order, int* warps_per_sm) {
-  return vw == 3 ? lane_setup_order<3>(cols, any_order, warps_per_sm)
-                 : lane_setup_order<4>(cols, any_order, warps_per_sm);
+// Pairs per warp: 8 (four lanes each), or 16 or 32 with a lane each.
+#define GA_WIDE(call)                                            \
+  (vw == 3 ? (lp == 8 ? call(3, 8, 4) : lp == 16 ? call(3, 16, 1) : call(3, 32, 1)) \
+           : (lp == 8 ? call(4, 8, 4) : lp == 16 ? call(4, 16, 1) : call(4, 32, 1)))
+
+cudaError_t wide_lane_setup(int vw, int lp, int cols, bool any_order, int* warps_per_sm) {
+#define GA_CALL(w, l, n) lane_setup_order<w, l, n>(cols, any_order, warps_per_sm)
+  return GA_WIDE(GA_CALL);
+#undef GA_CALL
 }
 
-void wide_lane_launch(int vw, const AlignParams& p, const LanePlan& plan, const BatchArgs& a,
+void wide_lane_launch(const AlignParams& p, const LanePlan& plan, const BatchArgs& a,
                       cudaStream_t s) {
-  if (vw == 3) lane_launch<3>(p, plan, a, s);
-  else lane_launch<4>(p, plan, a, s);
+  const int vw = plan.vw, lp = plan.lp;
+#define GA_CALL(w, l, n) lane_launch<w, l, n>(p, plan, a, s)
+  GA_WIDE(GA_CALL);
+#undef GA_CALL
 }
+#undef GA_WIDE
 
 void wide_locate_launch(int vw, const AlignParams& p, const LocateArgs& a, int log_q,
                         cudaStream_t s) {
