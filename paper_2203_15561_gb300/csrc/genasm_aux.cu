@@ -1,9 +1,12 @@
-// Input stage of the hot path: ASCII -> 2-bit packer.
+// Input stage of the hot path: ASCII -> 2-bit packer, and the output stage:
+// dense CIGARs.
 //
-// Each thread turns 16 ASCII bytes (one 16-byte load) into 4 packed bytes
-// (one 4-byte store), two such chunks at a time, so both sides of the copy
-// are fully coalesced; the kernel is bound by HBM bandwidth (1.25 bytes moved
-// per base).
+// Packer: each thread turns 16 ASCII bytes (one 16-byte load) into 4 packed
+// bytes (one 4-byte store), four such chunks at a time, so both sides of the
+// copy are fully coalesced. 1.25 bytes move per base; a gigabase takes 184
+// microseconds at the measured copy rate, and the integer ALU would take 360 at
+// 28 operations per four bases (what a code and an exact test per letter took):
+// the word-wide forms below take 9.
 #include <algorithm>
 #include <cstdint>
 
@@ -23,23 +26,49 @@ __device__ __forceinline__ uint32_t code_of(uint32_t c, bool& ok) {
   return ok ? (((c >> 1) ^ (c >> 2)) & 3u) : 0u;
 }
 
-// 0x80 in each zero byte of v, exactly: the low 7 bits of a byte plus 0x7F
-// stay below 0x100, so no carry crosses a byte.
-__device__ __forceinline__ uint32_t zero_bytes(uint32_t v) {
-  return ~(((v & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | v) & 0x80808080u;
+// The codes of a word's four letters, code q at bits 8q + 1 and 8q + 2 (bit 2
+// of the letter, and bits 1 and 2 xored; other letters: anything).
+__device__ __forceinline__ uint32_t word_codes(uint32_t w) { return (w ^ (w >> 1)) & 0x06060606u; }
+
+// One multiplication brings the four codes together: the byte is bits 24..31.
+// (Code q moves up by 23 - 6q bits; no two of the sixteen products overlap.)
+__device__ __forceinline__ uint32_t gather_codes(uint32_t c) { return c * 0x820820u; }
+
+// Zero in each byte that is an accepted letter. Those are 01x0 or 01x1 in the
+// high half and, with b4 the bit that tells T from the others, b0 = !b4, b3 = 0
+// and b4 = b2 & !b1. (Left shifts move bits of a byte into bit 4 of the same
+// byte, whatever the neighbours hold.)
+__device__ __forceinline__ uint32_t not_letters(uint32_t w) {
+  const uint32_t x = w ^ ((w << 2) & ~(w << 3));  // bit 4: b4 ^ (b2 & !b1)
+  const uint32_t v = x | ~(w ^ (w << 4));         // bit 4: that, or b4 = b0
+  return (v & 0x10101010u) | ((w ^ 0x40404040u) & 0xC8C8C8C8u);
 }
 
-// The four bases of a word as one byte (base q at bits 2q), a word at a time:
-// code_of's bits 1-2 with G/T swapped, validity by comparing the lower-cased
-// bytes with a, c, g and t; other bytes code 0 and are counted in `bad`.
+// word_codes with 0 for other letters, which are counted in `bad`.
+__device__ __forceinline__ uint32_t checked_codes(uint32_t w, uint32_t& bad) {
+  const uint32_t t = not_letters(w);
+  const uint32_t no = (((t & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | t) & 0x80808080u;  // 0x80 in nonzero bytes
+  bad += static_cast<uint32_t>(__popc(no));
+  return word_codes(w) & ~((no >> 5) | (no >> 6));
+}
+
+// The four bases of a word as one byte (base q at bits 2q).
 __device__ __forceinline__ uint32_t pack4(uint32_t w, uint32_t& bad) {
-  const uint32_t u = w | 0x20202020u;
-  const uint32_t ok = zero_bytes(u ^ 0x61616161u) | zero_bytes(u ^ 0x63636363u) |
-                      zero_bytes(u ^ 0x67676767u) | zero_bytes(u ^ 0x74747474u);
-  bad += 4u - static_cast<uint32_t>(__popc(ok));
-  const uint32_t c = ((w >> 1) ^ (w >> 2)) & ((ok >> 7) * 3u);  // 2-bit code per byte
-  const uint32_t t = c | (c >> 6);
-  return (t | (t >> 12)) & 0xffu;
+  return gather_codes(checked_codes(w, bad)) >> 24;
+}
+
+// Sixteen bases. Other letters are rare: the words are tested together, and only
+// a chunk that holds one takes the exact form.
+__device__ __forceinline__ uint32_t pack16(const uint4& v, uint32_t& bad) {
+  uint32_t a = word_codes(v.x), b = word_codes(v.y), c = word_codes(v.z), d = word_codes(v.w);
+  if ((not_letters(v.x) | not_letters(v.y)) | (not_letters(v.z) | not_letters(v.w))) {
+    a = checked_codes(v.x, bad);
+    b = checked_codes(v.y, bad);
+    c = checked_codes(v.z, bad);
+    d = checked_codes(v.w, bad);
+  }
+  return __byte_perm(__byte_perm(gather_codes(a), gather_codes(b), 0x0073),
+                     __byte_perm(gather_codes(c), gather_codes(d), 0x0073), 0x5410);
 }
 
 __global__ void pack_kernel(const uint8_t* __restrict__ ascii, uint64_t n, uint8_t* __restrict__ out,
@@ -47,23 +76,18 @@ __global__ void pack_kernel(const uint8_t* __restrict__ ascii, uint64_t n, uint8
   const uint64_t chunks = n / 16;
   uint32_t bad = 0;
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-  // Two chunks per iteration: both 16-byte loads are in flight together.
-  for (uint64_t q = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < chunks;
-       q += 2 * stride) {
-    const bool two = q + stride < chunks;
-    const uint4 v = __ldcs(reinterpret_cast<const uint4*>(ascii) + q);
-    const uint4 v2 = two ? __ldcs(reinterpret_cast<const uint4*>(ascii) + q + stride)
-                         : make_uint4(0x41414141u, 0x41414141u, 0x41414141u, 0x41414141u);
-    reinterpret_cast<uint32_t*>(out)[q] = pack4(v.x, bad) | (pack4(v.y, bad) << 8) |
-                                          (pack4(v.z, bad) << 16) | (pack4(v.w, bad) << 24);
-    uint32_t bad2 = 0;
-    const uint32_t p2 = pack4(v2.x, bad2) | (pack4(v2.y, bad2) << 8) | (pack4(v2.z, bad2) << 16) |
-                        (pack4(v2.w, bad2) << 24);
-    if (two) {
-      reinterpret_cast<uint32_t*>(out)[q + stride] = p2;
-      bad += bad2;
-    }
+  const uint4* in = reinterpret_cast<const uint4*>(ascii);
+  uint32_t* to = reinterpret_cast<uint32_t*>(out);
+  uint64_t q = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  // Four chunks per iteration: their 16-byte loads are in flight together.
+  for (; q + 3 * stride < chunks; q += 4 * stride) {
+    uint4 v[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) v[x] = __ldcs(in + q + x * stride);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) to[q + x * stride] = pack16(v[x], bad);
   }
+  for (; q < chunks; q += stride) to[q] = pack16(__ldcs(in + q), bad);
   // Tail (n % 16 bytes): one thread, byte by byte.
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     for (uint64_t x = chunks * 16; x < n; x += 4) {
@@ -185,137 +209,199 @@ cudaError_t launch_pack(const uint8_t* ascii, uint64_t n, uint8_t* packed, uint3
 // ---------------------------------------------------------------------------
 // CIGAR compaction: gathers every pair's runs (written at fixed per-pair
 // capacities by the alignment kernels) into one dense array, with the
-// exclusive prefix sum of the run counts as offsets. Three passes: per-chunk
-// sums, a scan of the chunk sums, then per-chunk offsets and a warp-per-pair
-// copy.
+// exclusive prefix sum of the run counts as offsets. Chunks of 1,024 pairs: one
+// launch sums each chunk's counts (none for a single chunk), one does the rest:
+// a block scans its chunk's counts, adds the chunks before it, writes the
+// offsets of its tile of the chunk and copies the tile's runs. (Recounting a
+// chunk in each of its blocks costs 4 KB of reads from L2 and two barriers; the
+// two launches it saves cost more on small batches and as much on large ones.)
 // ---------------------------------------------------------------------------
 
 namespace ga {
 
-constexpr int kScanThreads = 1024;
-constexpr int kScanChunk = kScanThreads;  // pairs per block
+constexpr int kCompactThreads = 256;
+constexpr uint32_t kCompactChunk = 4 * kCompactThreads;  // pairs
 
-__device__ __forceinline__ uint64_t block_exclusive_scan(uint64_t v, uint64_t* sh, uint64_t& total) {
-  // Warp-level inclusive scan, then scan of the 32 warp totals.
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint64_t x = v;
+// Sum over the block's threads, in every thread. sh: one word per warp.
+__device__ __forceinline__ uint64_t block_sum(uint64_t v, uint64_t* sh) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) sh[warp] = x;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
-  if (warp == 0) {
-    uint64_t w = lane < (blockDim.x >> 5) ? sh[lane] : 0ull;
+  uint64_t t = 0;
+#pragma unroll
+  for (int w = 0; w < kCompactThreads / 32; ++w) t += sh[w];
+  __syncthreads();
+  return t;
+}
+
+__global__ void __launch_bounds__(kCompactThreads) chunk_sum_kernel(const uint32_t* __restrict__ n_runs,
+                                                                    uint32_t n,
+                                                                    uint64_t* __restrict__ sums) {
+  __shared__ uint64_t sh[kCompactThreads / 32];
+  uint64_t v = 0;
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const uint64_t p = static_cast<uint64_t>(blockIdx.x) * kCompactChunk + x * kCompactThreads + threadIdx.x;
+    v += p < n ? n_runs[p] : 0u;
+  }
+  v = block_sum(v, sh);
+  if (threadIdx.x == 0) sums[blockIdx.x] = v;
+}
+
+// One block, for many chunks: exclusive scan of the chunk sums in place, their
+// sum after them.
+__global__ void __launch_bounds__(kCompactThreads) scan_sums_kernel(uint64_t* sums, uint32_t n_chunks) {
+  __shared__ uint64_t sh[kCompactThreads / 32];
+  uint64_t carry = 0;
+  for (uint32_t at = 0; at < n_chunks; at += kCompactThreads) {
+    const uint32_t q = at + threadIdx.x;
+    const uint64_t v = q < n_chunks ? sums[q] : 0u;
+    uint64_t incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
+      const uint64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if ((threadIdx.x & 31) >= static_cast<uint32_t>(o)) incl += y;
     }
-    sh[lane] = w;
+    if ((threadIdx.x & 31) == 31) sh[threadIdx.x >> 5] = incl;
+    __syncthreads();
+    uint64_t before = carry + incl - v;
+#pragma unroll
+    for (uint32_t w = 0; w < kCompactThreads / 32; ++w) {
+      before += w < threadIdx.x >> 5 ? sh[w] : 0u;
+      carry += sh[w];
+    }
+    if (q < n_chunks) sums[q] = before;
+    __syncthreads();
   }
-  __syncthreads();
-  total = sh[31];
-  const uint64_t before = warp > 0 ? sh[warp - 1] : 0ull;
-  __syncthreads();
-  return before + x - v;
+  if (threadIdx.x == 0) sums[n_chunks] = carry;
 }
 
-__global__ void __launch_bounds__(kScanThreads) chunk_sum_kernel(const uint32_t* __restrict__ n_runs,
-                                                                 uint32_t n, uint64_t* __restrict__ sums) {
-  __shared__ uint64_t sh[32];
-  const uint32_t q = blockIdx.x * kScanChunk + threadIdx.x;
-  const uint64_t v = q < n ? n_runs[q] : 0u;
-  uint64_t total;
-  block_exclusive_scan(v, sh, total);
-  if (threadIdx.x == 0) sums[blockIdx.x] = total;
-}
-
-// One block: exclusive scan of the chunk sums in place, any count.
-__global__ void __launch_bounds__(kScanThreads) scan_sums_kernel(uint64_t* sums, uint32_t n_chunks,
-                                                                 uint64_t* grand_total) {
-  __shared__ uint64_t sh[32];
-  uint64_t carry = 0;
-  for (uint32_t base = 0; base < n_chunks; base += kScanThreads) {
-    const uint32_t q = base + threadIdx.x;
-    const uint64_t v = q < n_chunks ? sums[q] : 0ull;
-    uint64_t total;
-    const uint64_t ex = block_exclusive_scan(v, sh, total);
-    if (q < n_chunks) sums[q] = carry + ex;
-    carry += total;
+// Block b: tile b % tiles (of `tile` pairs, a divisor of the chunk) of chunk
+// b / tiles. `scanned`: sums holds the chunks' exclusive scan and the total.
+__global__ void __launch_bounds__(kCompactThreads)
+    compact_kernel(const uint32_t* __restrict__ cigar, const uint64_t* __restrict__ cigar_off,
+                   const uint32_t* __restrict__ n_runs, uint32_t n, uint32_t tile,
+                   uint32_t tiles, const uint64_t* __restrict__ sums, uint32_t n_chunks, bool scanned,
+                   uint64_t* __restrict__ out_off, uint64_t out_cap, uint32_t* __restrict__ out) {
+  __shared__ uint64_t sh[kCompactThreads / 32];
+  __shared__ uint64_t off[kCompactChunk + 1];  // the chunk's pairs' offsets, from the chunk's start
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t chunk = blockIdx.x / tiles;
+  const uint64_t p0 = static_cast<uint64_t>(chunk) * kCompactChunk;
+  const uint32_t first = blockIdx.x % tiles * tile;
+  if (p0 + first >= n) return;
+  // Each thread's four counts, their scan over the block.
+  uint64_t c[4], mine = 0;
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const uint64_t p = p0 + 4u * threadIdx.x + x;
+    c[x] = mine;
+    mine += p < n ? n_runs[p] : 0u;
   }
-  if (threadIdx.x == 0) *grand_total = carry;
-}
-
-__global__ void __launch_bounds__(kScanThreads) offsets_kernel(const uint32_t* __restrict__ n_runs,
-                                                               uint32_t n, const uint64_t* __restrict__ sums,
-                                                               const uint64_t* __restrict__ grand_total,
-                                                               uint64_t* __restrict__ out_off) {
-  __shared__ uint64_t sh[32];
-  const uint32_t q = blockIdx.x * kScanChunk + threadIdx.x;
-  const uint64_t v = q < n ? n_runs[q] : 0u;
-  uint64_t total;
-  const uint64_t ex = block_exclusive_scan(v, sh, total);
-  if (q < n) out_off[q] = sums[blockIdx.x] + ex;
-  if (blockIdx.x == 0 && threadIdx.x == 0) out_off[n] = *grand_total;
-}
-
-__global__ void gather_runs_kernel(const uint32_t* __restrict__ cigar, const uint64_t* __restrict__ cigar_off,
-                                   const uint32_t* __restrict__ n_runs, uint32_t n,
-                                   const uint64_t* __restrict__ out_off, uint64_t out_cap,
-                                   uint32_t* __restrict__ out) {
-  if (out_off[n] > out_cap) return;  // caller's buffer too small: copy nothing
-  const uint32_t lane = threadIdx.x & 31;
-  const uint64_t warps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;
-  for (uint64_t p = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; p < n;
-       p += warps) {
-    const uint32_t* src = cigar + cigar_off[p];
-    uint32_t* dst = out + out_off[p];
-    const uint32_t cnt = n_runs[p];
-    // Four loads in flight per lane (the copy is bound by memory latency,
-    // not bandwidth, with one warp per pair).
-    uint32_t x = lane;
-    for (; x + 96 < cnt; x += 128) {
-      const uint32_t v0 = __ldcs(src + x), v1 = __ldcs(src + x + 32);
-      const uint32_t v2 = __ldcs(src + x + 64), v3 = __ldcs(src + x + 96);
-      dst[x] = v0;
-      dst[x + 32] = v1;
-      dst[x + 64] = v2;
-      dst[x + 96] = v3;
+  uint64_t incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= static_cast<uint32_t>(o)) incl += y;
+  }
+  if (lane == 31) sh[warp] = incl;
+  __syncthreads();
+  uint64_t before = incl - mine, total = 0;
+#pragma unroll
+  for (uint32_t w = 0; w < kCompactThreads / 32; ++w) {
+    before += w < warp ? sh[w] : 0u;
+    total += sh[w];
+  }
+#pragma unroll
+  for (int x = 0; x < 4; ++x) off[4u * threadIdx.x + x] = before + c[x];
+  if (threadIdx.x == 0) off[kCompactChunk] = total;
+  __syncthreads();
+  // The chunks before this one, and all of them.
+  uint64_t base = 0;
+  if (scanned) {
+    base = sums[chunk];
+    total = sums[n_chunks];
+  } else if (n_chunks > 1) {
+    uint64_t lo = 0, all = 0;
+    for (uint32_t q = threadIdx.x; q < n_chunks; q += kCompactThreads) {
+      const uint64_t v = sums[q];
+      all += v;
+      lo += q < chunk ? v : 0u;
+    }
+    base = block_sum(lo, sh);
+    total = block_sum(all, sh);
+  }
+  const uint32_t in_chunk = static_cast<uint32_t>(n - p0 < kCompactChunk ? n - p0 : kCompactChunk);
+  const uint32_t last = first + tile < in_chunk ? first + tile : in_chunk;
+  for (uint32_t q = first + threadIdx.x; q < last; q += kCompactThreads) out_off[p0 + q] = base + off[q];
+  if (p0 + last == n && threadIdx.x == 0) out_off[n] = total;
+  if (total > out_cap) return;  // caller's buffer too small: copy nothing
+  const uint64_t runs = off[last] - off[first];
+  if (runs < 32u * (last - first)) {
+    // Short CIGARs: a thread per run, its pair found in the offsets.
+    for (uint64_t x = threadIdx.x; x < runs; x += kCompactThreads) {
+      const uint64_t at = off[first] + x;
+      uint32_t a = first, b = last;  // off[a] <= at < off[b]
+      while (b - a > 1) {
+        const uint32_t m = (a + b) >> 1;
+        if (off[m] <= at) a = m;
+        else b = m;
+      }
+      out[base + at] = __ldcs(cigar + cigar_off[p0 + a] + (at - off[a]));
+    }
+    return;
+  }
+  for (uint32_t q = first + warp; q < last; q += kCompactThreads / 32) {
+    const uint32_t* src = cigar + cigar_off[p0 + q];
+    uint32_t* dst = out + base + off[q];
+    const uint64_t cnt = off[q + 1] - off[q];
+    // Eight loads in flight per lane (the copy is bound by memory latency, not
+    // bandwidth, with one warp per pair).
+    uint64_t x = lane;
+    for (; x + 224 < cnt; x += 256) {
+      uint32_t v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = __ldcs(src + x + 32 * u);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) dst[x + 32 * u] = v[u];
     }
     for (; x < cnt; x += 32) dst[x] = __ldcs(src + x);
   }
 }
 
 size_t compact_workspace_bytes(uint32_t n_pairs) {
-  const size_t chunks = (static_cast<size_t>(n_pairs) + kScanChunk - 1) / kScanChunk;
+  const size_t chunks = (static_cast<size_t>(n_pairs) + kCompactChunk - 1) / kCompactChunk;
   return 256 + sizeof(uint64_t) * (chunks + 1);
 }
 
 cudaError_t launch_compact(const uint32_t* cigar, const uint64_t* cigar_off, const uint32_t* n_runs,
                            uint32_t n, uint32_t* out, uint64_t out_cap, uint64_t* out_off, void* ws,
                            cudaStream_t s) {
-  const uint32_t chunks = static_cast<uint32_t>((static_cast<uint64_t>(n) + kScanChunk - 1) / kScanChunk);
-  uint64_t* grand = static_cast<uint64_t*>(ws);
-  uint64_t* sums = reinterpret_cast<uint64_t*>(static_cast<char*>(ws) + 256);
   if (n == 0) {
     const cudaError_t e = cudaMemsetAsync(out_off, 0, sizeof(uint64_t), s);
     return e;
   }
-  // The device query comes first, so that a failure leaves every output as
-  // it was (nothing is enqueued).
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  chunk_sum_kernel<<<chunks, kScanThreads, 0, s>>>(n_runs, n, sums);
-  scan_sums_kernel<<<1, kScanThreads, 0, s>>>(sums, chunks, grand);
-  offsets_kernel<<<chunks, kScanThreads, 0, s>>>(n_runs, n, sums, grand, out_off);
-  const uint64_t want = (static_cast<uint64_t>(n) * 32 + 255) / 256;
-  const int blocks = static_cast<int>(std::max<uint64_t>(1, std::min<uint64_t>(want, 16ull * sms)));
-  gather_runs_kernel<<<blocks, 256, 0, s>>>(cigar, cigar_off, n_runs, n, out_off, out_cap, out);
-  count_launches(4);
+  uint64_t* sums = static_cast<uint64_t*>(ws);
+  const uint32_t chunks = static_cast<uint32_t>((static_cast<uint64_t>(n) + kCompactChunk - 1) / kCompactChunk);
+  // Tiles of one pair per warp while that makes no more than a few thousand
+  // blocks, else of eight. Past a million pairs the blocks would spend more on
+  // adding up the chunks than a scan of them costs.
+  const uint32_t tile = n <= 32768 ? 8u : 64u;
+  const uint32_t tiles = (std::min(n, kCompactChunk) + tile - 1) / tile;
+  const bool scanned = chunks > 1024;
+  if (chunks > 1) {
+    chunk_sum_kernel<<<chunks, kCompactThreads, 0, s>>>(n_runs, n, sums);
+    count_launches(1);
+  }
+  if (scanned) {
+    scan_sums_kernel<<<1, kCompactThreads, 0, s>>>(sums, chunks);
+    count_launches(1);
+  }
+  compact_kernel<<<chunks * tiles, kCompactThreads, 0, s>>>(cigar, cigar_off, n_runs, n, tile, tiles,
+                                                            sums, chunks, scanned, out_off, out_cap,
+                                                            out);
+  count_launches(1);
   return cudaGetLastError();
 }
 
