@@ -96,19 +96,28 @@ __global__ void __launch_bounds__(kLptBuckets)
   h[x] = 0u;
   __syncthreads();
   const uint32_t rounds = (n + kLptBuckets - 1) / kLptBuckets;
-  for (uint32_t r = 0; r < rounds; ++r) {
+  constexpr uint32_t kRounds = kLptOneBlock / kLptBuckets;
+  uint32_t bucket[kRounds];  // all loads in flight at once
+#pragma unroll
+  for (uint32_t r = 0; r < kRounds; ++r) {
     const uint32_t q = r * kLptBuckets + x;
-    count_bucket(h, q < n ? lpt_bucket(read_len[q]) : 0u, q < n);
+    bucket[r] = q < n ? lpt_bucket(read_len[q]) : 0u;
   }
+#pragma unroll
+  for (uint32_t r = 0; r < kRounds; ++r)
+    if (r < rounds) count_bucket(h, bucket[r], r * kLptBuckets + x < n);
   __syncthreads();
   const uint32_t start = scan_buckets(h[x], s);
   wants_turns(h[x], start, n, queue + 5);
   h[x] = start;
   __syncthreads();
-  for (uint32_t r = 0; r < rounds; ++r) {
-    const uint32_t q = r * kLptBuckets + x;
-    const uint32_t at = count_bucket(h, q < n ? lpt_bucket(read_len[q]) : 0u, q < n);
-    if (q < n) order[at] = q;
+#pragma unroll
+  for (uint32_t r = 0; r < kRounds; ++r) {
+    if (r < rounds) {
+      const uint32_t q = r * kLptBuckets + x;
+      const uint32_t at = count_bucket(h, bucket[r], q < n);
+      if (q < n) order[at] = q;
+    }
   }
 }
 
@@ -467,9 +476,10 @@ cudaError_t launch_batched_locate(const AlignParams& p, const LanePlan& plan,
   int dev = 0, sms = 0;
   cudaError_t e = device_sms(&dev, &sms);
   if (e != cudaSuccess) return e;
-  // Lanes per pair: as many as one warp per scheduler has for every pair.
+  // Lanes per pair: the most that two or three warps per scheduler hold (each
+  // lane adds 2 W columns to the search).
   int log_q = 0;
-  while (log_q < 5 && (static_cast<uint64_t>(p.n_pairs) << log_q) <= 128ull * sms) ++log_q;
+  while (log_q < 5 && (2ull * p.n_pairs << log_q) <= 320ull * sms) ++log_q;
   const LocateArgs a{start_span, ref_start, locate_d};
   if (plan.vw == 1) locate_launch<1>(p, a, log_q, s);
   else if (plan.vw == 2) locate_launch<2>(p, a, log_q, s);

@@ -321,9 +321,11 @@ __global__ void __launch_bounds__(32) align_step_kernel(const AlignParams p, con
 // 2^log_q lanes search a pair, each a range of start columns. A start's edits
 // are at most wp, so its alignment spans at most 2 wp text bases: a lane whose
 // recurrence begins 2 wp columns right of its range has every value of the
-// range exactly. Within a lane the columns run right to left and the pattern's
-// last row is followed by its horizontal differences; a column that does not
-// cost more than the best one so far takes its place (ties go left).
+// range exactly. Within a lane the columns run right to left; the pattern's last
+// row is counted at each word of start columns and followed through it by its
+// horizontal differences; a column that does not cost more than the best one so
+// far takes its place (ties go left). Words of other columns are the recurrence
+// alone.
 // ---------------------------------------------------------------------------
 
 constexpr int kLocateWarps = 4;  // per block
@@ -386,39 +388,62 @@ __global__ void __launch_bounds__(32 * kLocateWarps)
       vn[k] = 0u;
       top[k] = (wp - 1) >> 5 == k ? 1u << ((wp - 1) & 31) : 0u;
     }
-    int score = wp, found = 0x7fffffff;
+    const uint32_t top_at = static_cast<uint32_t>(wp - 1) & 31u;
+    int found = 0x7fffffff;
     uint32_t pos = 0;
     const int64_t w0 = (static_cast<int64_t>(o) + lo) >> 4;
-    uint32_t next = __ldg(words + ((static_cast<uint64_t>(o) + x0 - 1u) >> 4));
-    for (int64_t w = (static_cast<int64_t>(o) + x0 - 1) >> 4; w >= w0; --w) {
-      const uint32_t tw = next;
-      if (w > w0) next = __ldg(words + w - 1);
+    int64_t w = (static_cast<int64_t>(o) + x0 - 1) >> 4;
+    uint32_t tw = __ldg(words + w);
+    uint32_t next = w > w0 ? __ldg(words + w - 1) : 0u;
+    uint32_t e_hi[8][VW], e_lo[8][VW];
+    load_eq8<VW>(eq_lane, tw, 8, e_hi);
+    for (; w >= w0; --w) {
       const int64_t i0 = 16 * w - o;  // the word's first base
+      load_eq8<VW>(eq_lane, tw, 0, e_lo);
       // Columns of the word at or past x0 keep the initial column.
-      const int left = x0 - i0 < 16 ? static_cast<int>(x0 - i0) : 16;
-      // Start columns of the word: places from .. to - 1.
-      const int to = hi - i0 < 16 ? static_cast<int>(static_cast<int64_t>(hi) - i0) : 16;
-      const int from = i0 < lo ? static_cast<int>(lo - i0) : 0;
+      if (x0 - i0 < 16) {
+        const int left = static_cast<int>(x0 - i0);
 #pragma unroll
-      for (int x = 15; x >= 0; --x) {
-        uint32_t eq[VW], d0[VW], hp[VW], hn[VW];
-        load_eq<VW>(eq_at<VW>(eq_lane, tw, x), eq);
+        for (int x = 0; x < 8; ++x) {
 #pragma unroll
-        for (int k = 0; k < VW; ++k) eq[k] = x < left ? eq[k] : 0u;
-        column_step<VW>(eq, vp, vn, d0, hp, hn);
-        uint32_t up = 0, down = 0;
-#pragma unroll
-        for (int k = 0; k < VW; ++k) {
-          up |= hp[k] & top[k];
-          down |= hn[k] & top[k];
-        }
-        score += up ? 1 : 0;
-        score -= down ? 1 : 0;
-        if (x < to && x >= from && score <= found) {
-          found = score;
-          pos = static_cast<uint32_t>(i0 + x);
+          for (int k = 0; k < VW; ++k) {
+            e_lo[x][k] = x < left ? e_lo[x][k] : 0u;
+            e_hi[x][k] = x + 8 < left ? e_hi[x][k] : 0u;
+          }
         }
       }
+      if (i0 >= hi) {  // no start column of this lane's in the word
+#pragma unroll
+        for (int x = 15; x >= 0; --x) {
+          uint32_t d0[VW], hp[VW], hn[VW];
+          column_step<VW>(x >= 8 ? e_hi[x & 7] : e_lo[x & 7], vp, vn, d0, hp, hn);
+        }
+      } else {
+        // Start columns of the word: places from .. to - 1.
+        const int to = hi - i0 < 16 ? static_cast<int>(static_cast<int64_t>(hi) - i0) : 16;
+        const int from = i0 < lo ? static_cast<int>(lo - i0) : 0;
+        int score = 0;
+#pragma unroll
+        for (int k = 0; k < VW; ++k) score += word_distance(wp, k, vp[k], vn[k]);
+#pragma unroll
+        for (int x = 15; x >= 0; --x) {
+          uint32_t d0[VW], hp[VW], hn[VW];
+          column_step<VW>(x >= 8 ? e_hi[x & 7] : e_lo[x & 7], vp, vn, d0, hp, hn);
+          uint32_t up = 0, down = 0;
+#pragma unroll
+          for (int k = 0; k < VW; ++k) {
+            up |= hp[k] & top[k];
+            down |= hn[k] & top[k];
+          }
+          score += static_cast<int>(up >> top_at) - static_cast<int>(down >> top_at);
+          const bool better = x < to && x >= from && score <= found;
+          found = better ? score : found;
+          pos = better ? static_cast<uint32_t>(i0 + x) : pos;
+        }
+      }
+      tw = next;
+      if (w > w0 + 1) next = __ldg(words + w - 2);
+      load_eq8<VW>(eq_lane, tw, 8, e_hi);  // (past the last word: not used)
     }
     if (found <= p.kmax)
       best = min(best, (static_cast<uint64_t>(found) << 32) | pos);

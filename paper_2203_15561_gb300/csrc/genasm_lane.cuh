@@ -467,15 +467,16 @@ __device__ __forceinline__ int split_columns(uint32_t q, int wp, int wt, int nco
   // A lane's first steps, before its own first column, match nothing (its word
   // then stays as it is): the first eight columns are always masked.
   const int cols = 16 * ncols16 - static_cast<int>(2u * q);
-  int left = min(wt_lane, cols);
+  const int left = min(wt_lane, cols);
+  const auto mask8 = [&](uint32_t (&e)[8][1], int c) {
+#pragma unroll
+    for (int x = 0; x < 8; ++x) e[x][0] = c + x < left ? e[x][0] : 0u;
+  };
+  mask8(hi, 16 * ncols16 - 8);
   for (int c0 = 16 * ncols16 - 16; c0 >= 0; c0 -= 16) {
     load_eq8<1>(eq_lane, w[2 * VW - 1], 0, lo);
     row -= 16u * Shape::kColBytes;
     hrow -= 16u * Shape::kHpBytes;
-    if (kMask || c0 == 16 * ncols16 - 16) {
-#pragma unroll
-      for (int x = 0; x < 8; ++x) hi[x][0] = c0 + 8 + x < left ? hi[x][0] : 0u;
-    }
     const bool keep_hi = c0 + 8 < end, keep_lo = c0 < end;
 #pragma unroll
     for (int x = 7; x >= 0; --x)
@@ -484,8 +485,8 @@ __device__ __forceinline__ int split_columns(uint32_t q, int wp, int wt, int nco
     for (int k = 2 * VW - 1; k > 0; --k) w[k] = w[k - 1];
     load_eq8<1>(eq_lane, w[2 * VW - 1], 8, hi);  // (past the last block: not used)
     if constexpr (kMask) {
-#pragma unroll
-      for (int x = 0; x < 8; ++x) lo[x][0] = c0 + x < left ? lo[x][0] : 0u;
+      mask8(hi, c0 - 8);
+      mask8(lo, c0);
     }
 #pragma unroll
     for (int x = 7; x >= 0; --x)
@@ -688,8 +689,10 @@ __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& 
   const uint32_t text = static_cast<uint32_t>(inner ? commit : wt);      // text bases it may take
   uint32_t cp = 0, ct = 0;
   int dmin = -1;
-  const bool mask = __any_sync(kMask, ga && wt < 16 * ncols16);
-  const int need = __any_sync(kMask, ga && !inner) ? 32 * VW : commit;  // columns a walk can reach
+  // Some lane's text or pattern ends here: masked columns, and walks that can
+  // reach all of them.
+  const bool mask = __any_sync(kMask, ga && (wt < 16 * ncols16 || !inner));
+  const int need = mask ? 32 * VW : commit;
   for (int cb = 0;; cb += cols) {
     uint32_t t2[2 * VW];
 #pragma unroll
