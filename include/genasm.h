@@ -257,7 +257,7 @@ int ga_align_batch_noalloc(const uint8_t* d_reads, const uint64_t* d_read_off,
  * again. A request is always taken when none is waiting.
  * ga_server_step waits for the step in flight (if any) and takes its
  * finished pairs, admits queued requests in arrival order while the budget
- * has room, and launches the next step (one captured CUDA graph), which
+ * has room, and launches the next step, which
  * advances every admitted pair by at most `step_windows` windows (default
  * 32) with its window state kept on the device between steps; it returns
  * while that step runs. Meanwhile it completes every request whose pairs are

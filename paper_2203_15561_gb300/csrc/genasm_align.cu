@@ -297,10 +297,10 @@ namespace {
 int vw_for(int W) { return (W + 31) / 32; }
 int up8(int x) { return (x + 7) / 8 * 8; }
 
-cudaError_t setup_for(int vw, int lp, int cols, bool any_order, int* warps_per_sm) {
-  if (vw == 1) return lane_setup_order<1, 32, 1>(cols, any_order, warps_per_sm);
-  if (vw == 2) return lane_setup_order<2, 32, 1>(cols, any_order, warps_per_sm);
-  return wide_lane_setup(vw, lp, cols, any_order, warps_per_sm);
+cudaError_t setup_for(const LanePlan& plan, int* warps_per_sm) {
+  if (plan.vw == 1) return lane_setup_order<1, 32, 1>(plan, warps_per_sm);
+  if (plan.vw == 2) return lane_setup_order<2, 32, 1>(plan, warps_per_sm);
+  return wide_lane_setup(plan, warps_per_sm);
 }
 
 }  // namespace
@@ -310,10 +310,10 @@ namespace {
 // What a launch asks the driver about the device, asked once: SMs, and the
 // resident warps of each launch shape (a call of every shape costs a few
 // microseconds, a tenth of a small batch). Shapes differ by width, pairs per
-// warp, order and table columns (multiples of 8 up to 128).
+// warp, order, staging and table columns (multiples of 8 up to 128).
 struct DeviceFacts {
   int sms = 0;
-  int8_t warps[4][3][2][17] = {};  // 0: not asked yet, else warps per SM + 1
+  int8_t warps[4][3][2][2][17] = {};  // 0: not asked yet, else warps per SM + 1
 };
 constexpr int kMaxDevices = 64;
 std::mutex g_facts_mutex;
@@ -331,13 +331,14 @@ cudaError_t device_sms(int* dev, int* sms) {
   return e;
 }
 
-cudaError_t shape_warps(int dev, int vw, int lp, int cols, bool any_order, int* warps) {
-  if (dev < 0 || dev >= kMaxDevices) return setup_for(vw, lp, cols, any_order, warps);
+cudaError_t shape_warps(int dev, const LanePlan& plan, int* warps) {
+  if (dev < 0 || dev >= kMaxDevices) return setup_for(plan, warps);
   std::lock_guard<std::mutex> lock(g_facts_mutex);
-  int8_t& w = g_facts[dev].warps[vw - 1][lp == 32 ? 0 : lp == 16 ? 1 : 2][any_order][cols / 8];
+  int8_t& w = g_facts[dev].warps[plan.vw - 1][plan.lp == 32 ? 0 : plan.lp == 16 ? 1 : 2][plan.any_order]
+                                [plan.staged][plan.cols / 8];
   cudaError_t e = cudaSuccess;
   if (w == 0) {
-    e = setup_for(vw, lp, cols, any_order, warps);
+    e = setup_for(plan, warps);
     if (e == cudaSuccess) w = static_cast<int8_t>(*warps + 1);
   }
   *warps = w - 1;
@@ -361,10 +362,11 @@ cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePla
   // scheduler holds every pair (2,001 pairs of 10 kb at W = 128: 0.79 ms against
   // 1.16 with one lane each). At W <= 64 two lanes per pair gained nothing (3,330
   // cycles for a window's columns against 3,280).
+  plan->staged = false;
   if (plan->vw >= 3 && n <= 8 * scheds) {
     plan->lp = 8;
     plan->cols = all;
-    if ((e = shape_warps(dev, plan->vw, 8, all, plan->any_order, &per_sm)) != cudaSuccess) return e;
+    if ((e = shape_warps(dev, *plan, &per_sm)) != cudaSuccess) return e;
     per_sm = std::min(per_sm, 4);
   } else {
     // One lane per pair. Tables of every column a window can walk, else of the W
@@ -376,25 +378,29 @@ cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePla
     // 312 us, 19,456 pairs 209), but with pairs for half the lanes 1.9 times
     // (10,000 pairs of 10 kb: 2.05 ms against 1.10).
     const int want = n > 64 * scheds ? 8 : 4;
+    LanePlan best = *plan, t = *plan;
+    t.staged = plan->vw <= 2 && want == 4 && n > scheds;
     for (int lp : {32, 16}) {
       if (lp == 16 && plan->vw < 3) break;
       for (int cols : {all, std::max(inner, std::min(all, 48)), inner}) {
         if (per_sm >= want) break;
+        t.lp = lp;
+        t.cols = cols;
         int ps = 0;
-        if ((e = shape_warps(dev, plan->vw, lp, cols, plan->any_order, &ps)) != cudaSuccess) return e;
+        if ((e = shape_warps(dev, t, &ps)) != cudaSuccess) return e;
         ps = ps >= 8 ? 8 : std::min(ps, 4);
         if (ps <= per_sm) continue;
         per_sm = ps;
-        plan->lp = lp;
-        plan->cols = cols;
+        best = t;
       }
       if (per_sm >= 4) break;
     }
+    *plan = best;
     per_sm = std::min(per_sm, want);
   }
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   // (an attribute of the function in this context: set for every launch)
-  if ((e = setup_for(plan->vw, plan->lp, plan->cols, plan->any_order, nullptr)) != cudaSuccess) return e;
+  if ((e = setup_for(*plan, nullptr)) != cudaSuccess) return e;
   const uint64_t warps = std::min<uint64_t>(static_cast<uint64_t>(sms) * per_sm, n);
   plan->warps = static_cast<int>(warps);
   plan->lanes = static_cast<int>(std::min<uint64_t>(plan->lp, (n + warps - 1) / warps));
@@ -500,8 +506,8 @@ cudaError_t launch_batched_locate(const AlignParams& p, const LanePlan& plan,
 namespace {
 
 size_t step_smem(int vw, int cols) {
-  return vw == 1 ? lane_block_smem<LaneShape<1, 32, 1>>(cols, false)
-                 : lane_block_smem<LaneShape<2, 32, 1>>(cols, false);
+  return vw == 1 ? lane_block_smem<LaneShape<1, 32, 1>>(cols, false, false)
+                 : lane_block_smem<LaneShape<2, 32, 1>>(cols, false, false);
 }
 
 template <int VW>
@@ -540,23 +546,6 @@ cudaError_t launch_step(const AlignParams& p, const LanePlan& plan, const StepAr
   const cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) count_launches(1);
   return e;
-}
-
-// The finished count and the finished slots of a step, into host-mapped memory
-// (one block; the host reads them once the step's event has completed).
-__global__ void step_copyout_kernel(const uint32_t* __restrict__ counters,
-                                    const uint32_t* __restrict__ done, uint32_t* host_count,
-                                    uint32_t* host_done) {
-  const uint32_t nd = counters[1];
-  for (uint32_t q = threadIdx.x; q < nd; q += blockDim.x) host_done[q] = done[q];
-  if (threadIdx.x == 0) host_count[0] = nd;
-}
-
-cudaError_t launch_step_copyout(const uint32_t* counters, const uint32_t* done,
-                                uint32_t* host_count, uint32_t* host_done, cudaStream_t s) {
-  step_copyout_kernel<<<1, 256, 0, s>>>(counters, done, host_count, host_done);
-  count_launches(1);
-  return cudaGetLastError();
 }
 
 }  // namespace ga

@@ -107,8 +107,8 @@ __device__ __forceinline__ uint32_t lane_smem_base() {
   return (smem_addr(lane_smem) + Shape::kEqBytes - 1u) & ~(Shape::kEqBytes - 1u);
 }
 template <class Shape>
-constexpr size_t lane_block_smem(int cols, bool any_order) {
-  return Shape::bytes(cols, any_order) + (Shape::kEqBytes > 1024u ? 1024u : 0u);
+constexpr size_t lane_block_smem(int cols, bool any_order, bool staged) {
+  return Shape::bytes(cols, any_order, staged) + (Shape::kEqBytes > 1024u ? 1024u : 0u);
 }
 
 // Hands `*counter`'s next values to the pairs of the lanes in `wants`, in lane
@@ -128,7 +128,7 @@ __device__ __forceinline__ uint32_t turn_windows(const AlignParams& p, const Bat
   return max(a.slice, m / (static_cast<uint32_t>(p.W - p.O) * a.turns) + 1u);
 }
 
-template <int VW, int LP, int NL, bool kAny>
+template <int VW, int LP, int NL, bool kAny, bool kStaged>
 __global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParams p, const BatchArgs a) {
   using Shape = LaneShape<VW, LP, NL>;
   constexpr uint32_t kMask = Shape::kMask;
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParam
             if (s.windows > 0) lane_resume(s, st);  // a pair that had turns already
             budget = turn_windows(p, a, st.m);
           }
-          if (st.busy) lane_fetch(st);
+          if (st.busy) lane_fetch<VW, kStaged>(st, base);
         } else if (quit) {
           drained = true;
         }
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParam
     // for a pair looks again after each).
     bool done, turn;
     do {
-      lane_window<VW, LP, NL, kAny>(p, st, base, a.cols);
+      lane_window<VW, LP, NL, kAny, kStaged>(p, st, base, a.cols);
       done = st.busy && lane_done(st);
       turn = slice && st.busy && !done && --budget == 0;
     } while (!__any_sync(kMask, done || turn || (!st.busy && !drained)));
@@ -249,21 +249,23 @@ __global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParam
     }
     __syncwarp(kMask);
   }
+  if constexpr (kStaged) copies_wait();
 }
 
 // Serving step: resumable alignment. Every pair in the active list advances by
-// at most `max_windows` windows; its window state is kept in device memory
-// between steps, so pairs admitted at different times share one launch.
+// at most `windows` windows; its window state is kept in device memory between
+// steps, so pairs admitted at different times share one launch. The active list
+// is read from, and the finished slots are written to, host memory mapped into
+// the device: the warp that is last to finish writes their count and leaves the
+// counters at zero for the next step, so that a step is this launch alone.
 template <int VW>
 __global__ void __launch_bounds__(32) align_step_kernel(const AlignParams p, const StepArgs a) {
   using Shape = LaneShape<VW, 32, 1>;
   constexpr uint32_t kMask = Shape::kMask;
-  const uint32_t n_active = a.counters[2];
   const uint32_t base = lane_smem_base<Shape>();
   const uint32_t lane = threadIdx.x;
-  const uint32_t max_windows = a.counters[3];
   // Few pairs are spread over all warps.
-  const uint32_t lanes = min(32u, (n_active + gridDim.x - 1) / gridDim.x);
+  const uint32_t lanes = min(32u, (a.n_active + gridDim.x - 1) / gridDim.x);
   LanePair<VW> st{};
   bool drained = lane >= lanes;
   uint32_t slot = 0, budget = 0;
@@ -274,14 +276,14 @@ __global__ void __launch_bounds__(32) align_step_kernel(const AlignParams p, con
     if (wants) {
       const uint32_t idx = take_next<Shape>(&a.counters[0], wants, lane);
       if (want) {
-        if (idx < n_active) {
+        if (idx < a.n_active) {
           slot = a.active[idx];
           lane_begin(p, slot, st, true);  // a fresh slot (all zero) starts here
           if (st.busy) {
             lane_resume(a.state[slot], st);
-            lane_fetch(st);
+            lane_fetch<VW, false>(st, base);
           }
-          budget = max_windows;
+          budget = a.windows;
           finished = !st.busy;
         } else {
           drained = true;
@@ -293,7 +295,7 @@ __global__ void __launch_bounds__(32) align_step_kernel(const AlignParams p, con
     if (__any_sync(kMask, st.busy)) {
       bool done, turn;
       do {
-        lane_window<VW, 32, 1, false>(p, st, base, a.cols);
+        lane_window<VW, 32, 1, false, false>(p, st, base, a.cols);
         done = st.busy && lane_done(st);
         turn = st.busy && !done && --budget == 0;
       } while (!__any_sync(kMask, done || turn || finished));
@@ -307,6 +309,14 @@ __global__ void __launch_bounds__(32) align_step_kernel(const AlignParams p, con
     }
     if (finished) a.done[atomicAdd(&a.counters[1], 1u)] = slot;
     __syncwarp(kMask);
+  }
+  __threadfence_system();  // this warp's finished slots, before its arrival
+  __syncwarp(kMask);
+  if (lane == 0 && atomicAdd(&a.counters[2], 1u) == gridDim.x - 1) {
+    __threadfence();
+    *a.n_done = atomicExch(&a.counters[1], 0u);
+    a.counters[0] = 0u;
+    a.counters[2] = 0u;
   }
 }
 
@@ -472,31 +482,47 @@ __global__ void __launch_bounds__(32 * kLocateWarps)
 // launch takes of it: concurrent launches of other shapes need other sizes) and,
 // unless warps_per_sm is null, reads the shape's resident warps per SM.
 constexpr int kSharedOptIn = 227 * 1024;
-template <int VW, int LP, int NL, bool kAny>
+
+template <int VW, int LP, int NL, bool kAny, bool kStaged>
 cudaError_t lane_setup(int cols, int* warps_per_sm) {
   using Shape = LaneShape<VW, LP, NL>;
-  const cudaError_t e = cudaFuncSetAttribute(
-      align_batched_kernel<VW, LP, NL, kAny>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedOptIn);
+  const auto kernel = align_batched_kernel<VW, LP, NL, kAny, kStaged>;
+  const cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedOptIn);
   if (e != cudaSuccess || !warps_per_sm) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      warps_per_sm, align_batched_kernel<VW, LP, NL, kAny>, Shape::kThreads,
-      lane_block_smem<Shape>(cols, kAny));
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(warps_per_sm, kernel, Shape::kThreads,
+                                                       lane_block_smem<Shape>(cols, kAny, kStaged));
 }
 
 template <int VW, int LP, int NL>
-cudaError_t lane_setup_order(int cols, bool any_order, int* warps_per_sm) {
-  return any_order ? lane_setup<VW, LP, NL, true>(cols, warps_per_sm)
-                   : lane_setup<VW, LP, NL, false>(cols, warps_per_sm);
+cudaError_t lane_setup_order(const LanePlan& plan, int* warps_per_sm) {
+  if constexpr (VW <= 2) {
+    if (plan.staged)
+      return plan.any_order ? lane_setup<VW, LP, NL, true, true>(plan.cols, warps_per_sm)
+                            : lane_setup<VW, LP, NL, false, true>(plan.cols, warps_per_sm);
+  }
+  return plan.any_order ? lane_setup<VW, LP, NL, true, false>(plan.cols, warps_per_sm)
+                        : lane_setup<VW, LP, NL, false, false>(plan.cols, warps_per_sm);
+}
+
+template <int VW, int LP, int NL, bool kAny, bool kStaged>
+void lane_launch_as(const AlignParams& p, const LanePlan& plan, const BatchArgs& a, cudaStream_t s) {
+  using Shape = LaneShape<VW, LP, NL>;
+  align_batched_kernel<VW, LP, NL, kAny, kStaged>
+      <<<plan.warps, Shape::kThreads, lane_block_smem<Shape>(plan.cols, kAny, kStaged), s>>>(p, a);
 }
 
 template <int VW, int LP, int NL>
 void lane_launch(const AlignParams& p, const LanePlan& plan, const BatchArgs& a, cudaStream_t s) {
-  using Shape = LaneShape<VW, LP, NL>;
-  const size_t smem = lane_block_smem<Shape>(plan.cols, plan.any_order);
-  if (plan.any_order)
-    align_batched_kernel<VW, LP, NL, true><<<plan.warps, Shape::kThreads, smem, s>>>(p, a);
-  else
-    align_batched_kernel<VW, LP, NL, false><<<plan.warps, Shape::kThreads, smem, s>>>(p, a);
+  if constexpr (VW <= 2) {
+    if (plan.staged) {
+      if (plan.any_order) lane_launch_as<VW, LP, NL, true, true>(p, plan, a, s);
+      else lane_launch_as<VW, LP, NL, false, true>(p, plan, a, s);
+      return;
+    }
+  }
+  if (plan.any_order) lane_launch_as<VW, LP, NL, true, false>(p, plan, a, s);
+  else lane_launch_as<VW, LP, NL, false, false>(p, plan, a, s);
 }
 
 template <int VW>
@@ -507,7 +533,7 @@ void locate_launch(const AlignParams& p, const LocateArgs& a, int log_q, cudaStr
 }
 
 // Windows of 65..128 bases (genasm_wide.cu).
-cudaError_t wide_lane_setup(int vw, int lp, int cols, bool any_order, int* warps_per_sm);
+cudaError_t wide_lane_setup(const LanePlan& plan, int* warps_per_sm);
 void wide_lane_launch(const AlignParams& p, const LanePlan& plan, const BatchArgs& a, cudaStream_t s);
 void wide_locate_launch(int vw, const AlignParams& p, const LocateArgs& a, int log_q, cudaStream_t s);
 

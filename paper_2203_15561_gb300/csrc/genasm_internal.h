@@ -51,6 +51,7 @@ struct LanePlan {
   int warps;       // persistent grid size
   int lanes;       // of them, those that take pairs in this launch
   bool any_order;  // a traceback order other than the default
+  bool staged;     // the next window's bases copied ahead (see genasm_lane.cuh)
   bool lpt;        // longest-first hand-out
   uint32_t slice;  // windows per turn of the sliced queue (0: off)
   uint32_t turns;  // if not 0: a turn is this fraction of a pair, `slice` windows at least
@@ -78,24 +79,22 @@ struct SlotState {
 };
 
 struct StepArgs {
-  const uint32_t* active;  // slots to advance this step
-  uint32_t* counters;      // [0] work counter, [1] finished count (both zeroed per step),
-                           // [2] active slots, [3] windows per step (set before each step)
+  const uint32_t* active;  // slots to advance this step (mapped host memory)
+  uint32_t n_active;
+  uint32_t windows;        // windows per pair and step
+  uint32_t* counters;      // three, zero before a step and after it: work counter,
+                           // finished slots, finished warps
   SlotState* state;        // per slot
-  uint32_t* done;          // slots that finished this step
+  uint32_t* done;          // slots that finished this step (mapped host memory)
+  uint32_t* n_done;        // their count (mapped host memory)
   int cols;                // columns of a lane's table
 };
 
-// The serving step kernel reads its active count and window budget from
-// device memory (counters[2], counters[3]), so one captured launch serves every
-// step. prepare_step fills the launch shape for windows of W <= 64 bases and
-// sets the kernel's shared-memory attribute (once, outside any capture); launch_step launches it; launch_step_copyout copies the
-// finished count and the finished slots into host-mapped memory after it.
+// prepare_step fills the launch shape of the serving step for windows of W <= 64
+// bases and sets the kernel's shared-memory attribute; launch_step launches it.
 cudaError_t prepare_step(int W, LanePlan* plan);
 cudaError_t launch_step(const AlignParams& p, const LanePlan& plan, const StepArgs& a,
                         cudaStream_t s);
-cudaError_t launch_step_copyout(const uint32_t* counters, const uint32_t* done,
-                                uint32_t* host_count, uint32_t* host_done, cudaStream_t s);
 
 WorkspaceLayout workspace_layout(uint32_t n_pairs);
 

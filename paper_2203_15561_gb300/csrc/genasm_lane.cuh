@@ -71,13 +71,16 @@ struct LaneShape {
   static constexpr uint32_t kColBytes = VW * 2u * kWord;  // {D0, VP'} of one column
   static constexpr uint32_t kHpBytes = VW * kWord;        // HP of one column
   static constexpr bool kTogether = VW == 2 && NL == 1;
+  // Staged kernels (VW <= 2): the packed words that the next window's bases can
+  // lie in, of the read and the reference, copied one window ahead.
+  static constexpr uint32_t kStageSeq = (4 * VW + 1) * 128u;
   static constexpr uint32_t kPairBytes = kTogether ? 16u : 8u;  // a pair's entry (or its word's)
   // Columns past the stored ones: one that a walk may look at, and those that
   // the lanes of a pair run ahead of its first lane.
   static constexpr int kSpare = 1 + 2 * (NL - 1);
   // The warp's bytes with tables of `cols` columns.
-  static constexpr size_t bytes(int cols, bool any_order) {
-    return kEqBytes + kPlaneBytes +
+  static constexpr size_t bytes(int cols, bool any_order, bool staged) {
+    return kEqBytes + kPlaneBytes + (staged ? 2u * kStageSeq : 0u) +
            static_cast<size_t>(cols + kSpare) * (kColBytes + (any_order ? kHpBytes : 0u));
   }
 };
@@ -97,7 +100,10 @@ struct LanePair {
   uint32_t pair, m, n, pos_p, pos_t, edits, windows;
   int32_t status;
   bool busy;
-  uint32_t pw[2 * VW + 1], tw[2 * VW + 1];  // the next window's bases, loading
+  // The next window's bases: staged from the word at the low address bits
+  // p_word / t_word on, or loading.
+  uint32_t p_word, t_word;
+  uint32_t pw[2 * VW + 1], tw[2 * VW + 1];
 };
 
 __device__ __forceinline__ uint32_t lds32(uint32_t a) {
@@ -116,6 +122,13 @@ __device__ __forceinline__ void sts32(uint32_t a, uint32_t x) {
 __device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
   asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
 }
+
+// Asynchronous copy of a word from global to shared memory, and the wait for all
+// of this lane's.
+__device__ __forceinline__ void copy_word(uint32_t to, const uint32_t* from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(from) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // One Eq mask of VW words (read-only between window starts).
 template <int VW>
@@ -203,6 +216,41 @@ __device__ __forceinline__ void load_words(const uint8_t* seq, uint32_t len, uin
   const uint32_t lim = o + 2u * min(len > pos ? len - pos : 0u, 32u * VW);  // first bit past the window
 #pragma unroll
   for (int k = 0; k <= 2 * VW; ++k) x[k] = 32u * k < lim ? __ldg(wa + k) : 0u;
+}
+
+// Starts copying the words from base `pos` on that hold its window's bases and
+// those of any window up to 32 * VW bases further to shared memory (one word of
+// every lane to 128 bytes). Only words that hold a base of the sequence are read.
+template <int VW>
+__device__ __forceinline__ uint32_t stage_words(const uint8_t* seq, uint32_t len, uint32_t pos, uint32_t to) {
+  constexpr int kWords = 4 * VW + 1;
+  const uintptr_t a = reinterpret_cast<uintptr_t>(seq) + (pos >> 2);
+  const uint32_t* wa = reinterpret_cast<const uint32_t*>(a & ~static_cast<uintptr_t>(3));
+  const uint32_t o = 8u * static_cast<uint32_t>(a & 3u) + 2u * (pos & 3u);
+  const uint32_t lim = o + 2u * min(len > pos ? len - pos : 0u, 16u * kWords);  // first bit past the end
+  if (lim >= 32u * kWords) {
+#pragma unroll
+    for (int k = 0; k < kWords; ++k) copy_word(to + 128u * k, wa + k);
+  } else {
+#pragma unroll
+    for (int k = 0; k < kWords; ++k)
+      if (32u * k < lim) copy_word(to + 128u * k, wa + k);
+  }
+  return static_cast<uint32_t>(a) & ~3u;
+}
+
+__device__ __forceinline__ uint32_t lo_word(const uint8_t* seq) {
+  return static_cast<uint32_t>(reinterpret_cast<uintptr_t>(seq)) & ~3u;
+}
+
+// The staged words of the window at `pos` (`word`: what stage_words returned).
+template <int VW>
+__device__ __forceinline__ void staged_words(const uint8_t* seq, uint32_t pos, uint32_t word, uint32_t from,
+                                             uint32_t (&x)[2 * VW + 1]) {
+  const uint32_t a = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(seq) + (pos >> 2)) & ~3u;
+  const uint32_t at = from + (a - word) * 32u;  // four bytes further on: 128 bytes
+#pragma unroll
+  for (int k = 0; k <= 2 * VW; ++k) x[k] = lds32(at + 128u * k);
 }
 
 // The bases themselves, 16 per word (past the end of the sequence: anything).
@@ -622,11 +670,20 @@ __device__ __forceinline__ void walk_step(const Walk<VW, LP, NL>& w, uint64_t tb
   }
 }
 
-// Starts loading the bases of the pair's next window.
-template <int VW>
-__device__ __forceinline__ void lane_fetch(LanePair<VW>& st) {
-  load_words<VW>(st.read, st.m, st.pos_p, st.pw);
-  load_words<VW>(st.ref, st.n, st.pos_t, st.tw);
+// Starts loading the bases of the pair's next window: to shared memory, or into
+// registers.
+template <int VW, bool kStaged>
+__device__ __forceinline__ void lane_fetch(LanePair<VW>& st, uint32_t base) {
+  using Shape = LaneShape<VW, 32, 1>;
+  if constexpr (kStaged) {
+    const uint32_t to = base + Shape::kEqBytes + (threadIdx.x & 31u) * 4u;
+    copies_wait();  // of a pair that was put back or failed: no two copies to one place
+    st.p_word = stage_words<VW>(st.read, st.m, st.pos_p, to);
+    st.t_word = stage_words<VW>(st.ref, st.n, st.pos_t, to + Shape::kStageSeq);
+  } else {
+    load_words<VW>(st.read, st.m, st.pos_p, st.pw);
+    load_words<VW>(st.ref, st.n, st.pos_t, st.tw);
+  }
 }
 
 // One window of the lane's pair (the window chain of a pair is serial: each
@@ -638,7 +695,14 @@ __device__ __forceinline__ void lane_fetch(LanePair<VW>& st) {
 // past them has the columns computed again with the next `cols` stored. With
 // several lanes per pair it holds them all; the lanes walk together, each with
 // the pair's whole state, and the first one writes its runs.
-template <int VW, int LP, int NL, bool kAny>
+//
+// kStaged: the packed words of the next window are copied to shared memory while
+// this one is computed; otherwise they are loaded into registers once its walk
+// has ended. With many pairs per warp some lane's load goes to L2 or further in
+// nearly every window (10,000 pairs of 10 kb: 1.21 ms, staged 1.14); a pair alone
+// in its warp, or two warps per scheduler, wait little and save the copies'
+// instructions (one pair 633 us, staged 660).
+template <int VW, int LP, int NL, bool kAny, bool kStaged>
 __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& st, uint32_t base,
                                             int cols) {
   using Shape = LaneShape<VW, LP, NL>;
@@ -646,7 +710,8 @@ __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& 
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t q = lane % NL, slot = lane / NL;
   const uint32_t eq_lane = base + lane * Shape::kEqLane;
-  const uint32_t tab_base = base + Shape::kEqBytes + Shape::kPlaneBytes;
+  constexpr uint32_t kStageBytes = kStaged ? 2u * Shape::kStageSeq : 0u;
+  const uint32_t tab_base = base + Shape::kEqBytes + kStageBytes + Shape::kPlaneBytes;
   const uint32_t tab_lane = tab_base + slot * Shape::kPairBytes;
   const uint32_t hp_lane =
       tab_base + static_cast<uint32_t>(cols + Shape::kSpare) * Shape::kColBytes + slot * 4u;
@@ -662,13 +727,26 @@ __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& 
   uint32_t tw[2 * VW];
   {
     uint32_t pw[2 * VW];
+    if constexpr (kStaged) {
+      // (a lane without a pair reads its first words)
+      const uint32_t from = base + Shape::kEqBytes + lane * 4u;
+      copies_wait();
+      staged_words<VW>(st.read, ga ? st.pos_p : 0u, ga ? st.p_word : lo_word(st.read), from, st.pw);
+      staged_words<VW>(st.ref, ga ? st.pos_t : 0u, ga ? st.t_word : lo_word(st.ref),
+                       from + Shape::kStageSeq, st.tw);
+    }
     align_bases<VW>(st.read, st.pos_p, st.pw, pw);
     align_bases<VW>(st.ref, st.pos_t, st.tw, tw);
     bit_planes<VW>(pw, w.pl, w.ph);
     bit_planes<VW>(tw, w.tl, w.th);
   }
+  // The next window starts W - O bases further at most: its words, while this
+  // window is computed. (This window's have been used: the planes depend on them.)
+  if constexpr (kStaged) {
+    if (ga && !last) lane_fetch<VW, true>(st, base);
+  }
   store_eq<VW, LP, NL>(eq_lane, q, wp, w.pl, w.ph);
-  w.plane_lane = base + Shape::kEqBytes + slot * 4u;
+  w.plane_lane = base + Shape::kEqBytes + kStageBytes + slot * 4u;
   if constexpr (VW >= 3) {
 #pragma unroll
     for (int k = 0; k <= VW; ++k) {
@@ -748,7 +826,9 @@ __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& 
       st.cells += static_cast<uint64_t>(wt) * static_cast<uint64_t>(dmin + 1);
       st.pos_p += cp;
       st.pos_t += ct;
-      if (st.pos_p < st.m) lane_fetch(st);
+      if constexpr (!kStaged) {
+        if (st.pos_p < st.m) lane_fetch<VW, false>(st, base);
+      }
     }
   }
 }

@@ -3,12 +3,11 @@
 // A request (1..n pairs, host ASCII) is copied at submission and waits until
 // the device-memory budget has room for it: its packed sequences, its CIGAR
 // capacity (read+ref+1 runs per pair) and one slot per pair, all carved from
-// arenas allocated once at creation. The device work of a step is one
-// captured CUDA graph (zero the step counters, the resumable step kernel over
-// every admitted, unfinished pair, then a copy of the finished slots into
-// host-mapped memory); the kernel reads the active count and the window
-// budget from device memory, so the same graph serves every step. Each
-// ga_server_step
+// arenas allocated once at creation. The device work of a step is one launch:
+// the resumable step kernel over every admitted, unfinished pair, which reads
+// the list of them from host-mapped memory and writes the finished slots there.
+// (A graph of a memset, the kernel and a copy-out kernel behind two copies of the
+// list took 15 us more of the 450 of a burst's step.) Each ga_server_step
 //   1. waits for the step launched by the previous call and takes the slots
 //      that finished in it (one event wait, no copy);
 //   2. admits waiting requests in arrival order while they fit: one H2D of
@@ -29,8 +28,9 @@
 // Requests admitted at different steps therefore share launches and overlap
 // on the device, and a finished request's memory is reused by the next
 // admission. The host copies of request ASCII (at submission, and into the
-// pinned staging buffer at admission) run on a small pool of copy threads. Every wait is a host-side event or stream synchronization; no
-// kernel waits on another.
+// pinned staging buffer at admission) run on a small pool of copy threads. Every
+// wait is a host-side event or stream synchronization; no kernel waits on
+// another.
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -299,25 +299,24 @@ struct ga_server {
   int32_t *d_dist = nullptr, *d_status = nullptr, *d_ref_consumed = nullptr;
   uint32_t *d_n_runs = nullptr, *d_n_windows = nullptr;
   ga::SlotState* d_state = nullptr;
-  uint32_t *d_active = nullptr, *d_done = nullptr, *d_counters = nullptr;
+  uint32_t* d_counters = nullptr;
   uint64_t* d_list = nullptr;    // gather list (3 x uint64 per pair)
   uint32_t* d_out = nullptr;     // gathered runs of finished requests
   uint64_t out_cap = 0;
-  // the step: a captured graph on the compute stream, its finished slots in
-  // host-mapped memory
+  // the step: one launch on the compute stream; its active slots and its finished
+  // ones are in host memory mapped into the device
   cudaStream_t cstream = nullptr;
-  cudaGraph_t step_graph = nullptr;
-  cudaGraphExec_t step_exec = nullptr;
-  uint64_t step_kernels = 0;  // kernels one replay launches
   cudaEvent_t ev_admit = nullptr, ev_step = nullptr;
   cudaEvent_t ev_staged = nullptr;  // the last H2D copy out of h_ascii has been issued before it
   bool staged = false;
   bool inflight = false;
+  bool admitted = false;            // copies on the copy stream that the next step waits for
   uint32_t* h_count_map = nullptr;  // [0] slots finished in the last step
   uint32_t* h_done_map = nullptr;   // those slots
-  uint32_t* d_count_map = nullptr;  // device views of the two
+  uint32_t* h_active_map = nullptr;  // slots of the step in flight
+  uint32_t* d_count_map = nullptr;  // device views of the three
   uint32_t* d_done_map = nullptr;
-  uint32_t* h_ctl = nullptr;        // pinned: active count, windows per step
+  uint32_t* d_active_map = nullptr;
   // pinned host staging
   uint8_t* h_ascii = nullptr;
   // one admission's packing segments and slot records (pinned, then device)
@@ -325,7 +324,6 @@ struct ga_server {
   ga::SlotRecord* h_recs = nullptr;
   ga::PackSegment* d_segs = nullptr;
   ga::SlotRecord* d_recs = nullptr;
-  uint32_t *h_active = nullptr, *h_done = nullptr, *h_counters = nullptr;
   uint64_t* h_list = nullptr;
   uint32_t* h_out = nullptr;
   int32_t* h_small = nullptr;    // a harvest chunk's dist, status, ref_consumed, n_runs
@@ -350,6 +348,7 @@ struct ga_server {
   std::vector<CopyPool::Job> copy_jobs;
   std::vector<Request*> slot_owner;  // per slot
   std::vector<uint32_t> active;
+  std::vector<char> gone;  // per slot: finished in the step being taken in
   std::deque<Result*> ready;
   std::map<uint64_t, Result*> handed_out;
   uint64_t next_ticket = 1;
@@ -382,8 +381,6 @@ void server_free(ga_server* s) {
   cudaFree(s->d_n_runs);
   cudaFree(s->d_n_windows);
   cudaFree(s->d_state);
-  cudaFree(s->d_active);
-  cudaFree(s->d_done);
   cudaFree(s->d_counters);
   cudaFree(s->d_list);
   cudaFree(s->d_out);
@@ -392,9 +389,6 @@ void server_free(ga_server* s) {
   cudaFreeHost(s->h_recs);
   cudaFree(s->d_segs);
   cudaFree(s->d_recs);
-  cudaFreeHost(s->h_active);
-  cudaFreeHost(s->h_done);
-  cudaFreeHost(s->h_counters);
   cudaFreeHost(s->h_list);
   cudaFreeHost(s->h_out);
   cudaFreeHost(s->h_small);
@@ -404,9 +398,7 @@ void server_free(ga_server* s) {
   cudaFreeHost(s->h_res);
   cudaFreeHost(s->h_count_map);
   cudaFreeHost(s->h_done_map);
-  cudaFreeHost(s->h_ctl);
-  if (s->step_exec) cudaGraphExecDestroy(s->step_exec);
-  if (s->step_graph) cudaGraphDestroy(s->step_graph);
+  cudaFreeHost(s->h_active_map);
   if (s->ev_admit) cudaEventDestroy(s->ev_admit);
   if (s->ev_step) cudaEventDestroy(s->ev_step);
   if (s->ev_staged) cudaEventDestroy(s->ev_staged);
@@ -462,28 +454,18 @@ ga::AlignParams step_params(const ga_server* s) {
   return p;
 }
 
-// Captures the step's device work into a graph (once, at creation).
-cudaError_t capture_step(ga_server* s) {
+// Launches a step over the first n slots of the active list in host memory.
+cudaError_t start_step(ga_server* s, uint32_t n) {
   ga::StepArgs a{};
-  a.active = s->d_active;
+  a.active = s->d_active_map;
+  a.n_active = n;
+  a.windows = s->max_windows;
   a.counters = s->d_counters;
   a.state = s->d_state;
-  a.done = s->d_done;
+  a.done = s->d_done_map;
+  a.n_done = s->d_count_map;
   a.cols = s->plan.cols;
-  const uint64_t before = ga_launch_count();
-  cudaError_t e = cudaStreamBeginCapture(s->cstream, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) return e;
-  cudaError_t e1 = cudaMemsetAsync(s->d_counters, 0, 8, s->cstream);
-  if (e1 == cudaSuccess) e1 = ga::launch_step(step_params(s), s->plan, a, s->cstream);
-  if (e1 == cudaSuccess)
-    e1 = ga::launch_step_copyout(s->d_counters, s->d_done, s->d_count_map, s->d_done_map,
-                                 s->cstream);
-  e = cudaStreamEndCapture(s->cstream, &s->step_graph);
-  if (e1 != cudaSuccess) return e1;
-  if (e != cudaSuccess) return e;
-  s->step_kernels = ga_launch_count() - before;
-  ga::uncount_launches(s->step_kernels);  // captured, not run: counted at each replay
-  return cudaGraphInstantiate(&s->step_exec, s->step_graph, 0);
+  return ga::launch_step(step_params(s), s->plan, a, s->cstream);
 }
 
 }  // namespace
@@ -538,8 +520,6 @@ extern "C" int ga_server_create(size_t budget_bytes, int W, int O, int k, ga_ser
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_n_runs, M);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_n_windows, M);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_state, M);
-  if (e == cudaSuccess) e = dev_alloc(s, &s->d_active, M);
-  if (e == cudaSuccess) e = dev_alloc(s, &s->d_done, M);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_counters, 64);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_list, 3 * kListPairs);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_out, kOutRuns);
@@ -548,9 +528,6 @@ extern "C" int ga_server_create(size_t budget_bytes, int W, int O, int k, ga_ser
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_recs, sizeof(ga::SlotRecord) * kAdmitPairs);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_segs, kAdmitRequests);
   if (e == cudaSuccess) e = dev_alloc(s, &s->d_recs, kAdmitPairs);
-  if (e == cudaSuccess) e = cudaMallocHost(&s->h_active, 4ull * M);
-  if (e == cudaSuccess) e = cudaMallocHost(&s->h_done, 4ull * M);
-  if (e == cudaSuccess) e = cudaMallocHost(&s->h_counters, 4ull * 64);
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_list, 24ull * kListPairs);
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_out, 4ull * kOutRuns);
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_small, 16ull * kListPairs);
@@ -563,10 +540,11 @@ extern "C" int ga_server_create(size_t budget_bytes, int W, int O, int k, ga_ser
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_res, res_bytes);
   if (e == cudaSuccess) e = cudaHostAlloc(&s->h_count_map, 64, cudaHostAllocMapped);
   if (e == cudaSuccess) e = cudaHostAlloc(&s->h_done_map, 4ull * M, cudaHostAllocMapped);
-  if (e == cudaSuccess) e = cudaMallocHost(&s->h_ctl, 64);
+  if (e == cudaSuccess) e = cudaHostAlloc(&s->h_active_map, 4ull * M, cudaHostAllocMapped);
   if (e == cudaSuccess) e = cudaHostGetDevicePointer(&s->d_count_map, s->h_count_map, 0);
   if (e == cudaSuccess) e = cudaHostGetDevicePointer(&s->d_done_map, s->h_done_map, 0);
-  if (e == cudaSuccess) e = capture_step(s);
+  if (e == cudaSuccess) e = cudaHostGetDevicePointer(&s->d_active_map, s->h_active_map, 0);
+  if (e == cudaSuccess) e = cudaMemsetAsync(s->d_counters, 0, 64 * 4, s->cstream);
   if (e != cudaSuccess) {
     server_free(s);
     delete s;
@@ -580,6 +558,7 @@ extern "C" int ga_server_create(size_t budget_bytes, int W, int O, int k, ga_ser
   s->slot_alloc = RangeAlloc(M);
   s->res_alloc = RangeAlloc(res_bytes / 4);
   s->slot_owner.assign(M, nullptr);
+  s->gone.assign(M, 0);
   *out = s;
   return GA_OK;
 }
@@ -744,6 +723,7 @@ int admit(ga_server* s, std::vector<Request*>& finished) {
       cudaEventRecord(s->ev_staged, st) != cudaSuccess)
     return GA_ECUDA;
   s->staged = true;
+  s->admitted = true;
   if (ga::launch_pack_segments(s->d_ascii, s->d_segs, n_segs, max_seg, s->d_seq, st) != cudaSuccess ||
       ga::launch_scatter_slots(s->d_recs, n_recs, s->d_read_off, s->d_ref_off, s->d_cigar_off,
                                s->d_read_len, s->d_ref_len, s->d_cigar_cap, s->d_state,
@@ -882,40 +862,35 @@ extern "C" int ga_server_step(ga_server* s, uint32_t* n_active) {
     s->inflight = false;
     const uint32_t nd = *reinterpret_cast<volatile uint32_t*>(s->h_count_map);
     if (nd > 0) {
-      std::vector<char> gone(s->max_slots, 0);
       for (uint32_t q = 0; q < nd; ++q) {
         const uint32_t slot = reinterpret_cast<volatile uint32_t*>(s->h_done_map)[q];
         if (slot >= s->max_slots || !s->slot_owner[slot]) return GA_ECUDA;
-        gone[slot] = 1;
+        s->gone[slot] = 1;
         Request* r = s->slot_owner[slot];
         if (++r->done == r->n) finished.push_back(r);
       }
       size_t w = 0;
       for (size_t q = 0; q < s->active.size(); ++q)
-        if (!gone[s->active[q]]) s->active[w++] = s->active[q];
+        if (!s->gone[s->active[q]]) s->active[w++] = s->active[q];
       s->active.resize(w);
+      for (uint32_t q = 0; q < nd; ++q) s->gone[reinterpret_cast<volatile uint32_t*>(s->h_done_map)[q]] = 0;
     }
   }
   // 2. Requests waiting for admission (requests with no pairs finish here).
   int rc = admit(s, finished);
   if (rc != GA_OK) return rc;
-  // 3. The next step, after the admission copies: active slots and sizes,
-  // then the captured launch; it runs while the host goes on.
+  // 3. The next step, after the admission copies; it runs while the host goes on.
   if (!s->active.empty()) {
     const uint32_t na = static_cast<uint32_t>(s->active.size());
-    std::memcpy(s->h_active, s->active.data(), 4ull * na);
-    s->h_ctl[0] = na;
-    s->h_ctl[1] = s->max_windows;
-    if (cudaMemcpyAsync(s->d_active, s->h_active, 4ull * na, cudaMemcpyHostToDevice, s->stream) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(s->d_counters + 2, s->h_ctl, 8, cudaMemcpyHostToDevice, s->stream) !=
-            cudaSuccess ||
-        cudaEventRecord(s->ev_admit, s->stream) != cudaSuccess ||
-        cudaStreamWaitEvent(s->cstream, s->ev_admit, 0) != cudaSuccess ||
-        cudaGraphLaunch(s->step_exec, s->cstream) != cudaSuccess ||
-        cudaEventRecord(s->ev_step, s->cstream) != cudaSuccess)
+    std::memcpy(s->h_active_map, s->active.data(), 4ull * na);
+    if (s->admitted) {
+      if (cudaEventRecord(s->ev_admit, s->stream) != cudaSuccess ||
+          cudaStreamWaitEvent(s->cstream, s->ev_admit, 0) != cudaSuccess)
+        return GA_ECUDA;
+      s->admitted = false;
+    }
+    if (start_step(s, na) != cudaSuccess || cudaEventRecord(s->ev_step, s->cstream) != cudaSuccess)
       return GA_ECUDA;
-    ga::count_launches(s->step_kernels);
     s->inflight = true;
   }
   // 4. Results of the requests that finished, while the step runs.

@@ -5,21 +5,20 @@
 namespace ga {
 
 // Pairs per warp: 8 (four lanes each), or 16 or 32 with a lane each.
-#define GA_WIDE(call)                                            \
-  (vw == 3 ? (lp == 8 ? call(3, 8, 4) : lp == 16 ? call(3, 16, 1) : call(3, 32, 1)) \
-           : (lp == 8 ? call(4, 8, 4) : lp == 16 ? call(4, 16, 1) : call(4, 32, 1)))
+#define GA_WIDE(plan, call)                                                                      \
+  ((plan).vw == 3 ? ((plan).lp == 8 ? call(3, 8, 4) : (plan).lp == 16 ? call(3, 16, 1) : call(3, 32, 1)) \
+                  : ((plan).lp == 8 ? call(4, 8, 4) : (plan).lp == 16 ? call(4, 16, 1) : call(4, 32, 1)))
 
-cudaError_t wide_lane_setup(int vw, int lp, int cols, bool any_order, int* warps_per_sm) {
-#define GA_CALL(w, l, n) lane_setup_order<w, l, n>(cols, any_order, warps_per_sm)
-  return GA_WIDE(GA_CALL);
+cudaError_t wide_lane_setup(const LanePlan& plan, int* warps_per_sm) {
+#define GA_CALL(w, l, n) lane_setup_order<w, l, n>(plan, warps_per_sm)
+  return GA_WIDE(plan, GA_CALL);
 #undef GA_CALL
 }
 
 void wide_lane_launch(const AlignParams& p, const LanePlan& plan, const BatchArgs& a,
                       cudaStream_t s) {
-  const int vw = plan.vw, lp = plan.lp;
 #define GA_CALL(w, l, n) lane_launch<w, l, n>(p, plan, a, s)
-  GA_WIDE(GA_CALL);
+  GA_WIDE(plan, GA_CALL);
 #undef GA_CALL
 }
 #undef GA_WIDE
