@@ -622,13 +622,31 @@ struct Walk {
   }
 };
 
+// The ops of an iteration: matches, then an edit (0: none). They join the runs
+// in the next iteration, once it has asked for its column: the bookkeeping then
+// fills the wait for that read instead of standing before it (10,000 pairs of
+// 10 kb: 1.133 ms, with it 1.119; one pair 644 us, with it 638).
+struct LateOps {
+  uint32_t matches, edit;
+};
+template <int VW>
+__device__ __forceinline__ void book_ops(LanePair<VW>& st, const LateOps& o) {
+  close_run(st, o.matches > 0u && st.run_op != kOpMatch);
+  st.run_op = o.matches > 0u ? kOpMatch : st.run_op;
+  st.run_len += o.matches;
+  close_run(st, o.edit != 0u && st.run_op != o.edit);
+  st.run_op = o.edit ? o.edit : st.run_op;
+  st.run_len += o.edit ? 1u : 0u;
+}
+
 // One iteration of a walk at read base cp and text base ct of the window, up
 // to `goal` and `tend`: with the default order the matches ahead (up to 32 base
 // pairs compared at once) and the edit that ends them, else one op. No
 // branches: a lane whose counts are used up appends nothing.
 template <int VW, int LP, int NL, bool kAny>
 __device__ __forceinline__ void walk_step(const Walk<VW, LP, NL>& w, uint64_t tb_table, LanePair<VW>& st,
-                                          uint32_t& cp, uint32_t& ct, uint32_t goal, uint32_t tend) {
+                                          uint32_t& cp, uint32_t& ct, uint32_t goal, uint32_t tend,
+                                          LateOps& late) {
   const uint32_t lim = min(min(goal - cp, tend - ct), 32u);
   if constexpr (!kAny) {
     const uint32_t z = leading_zeros(w.differ(cp, ct));
@@ -637,16 +655,12 @@ __device__ __forceinline__ void walk_step(const Walk<VW, LP, NL>& w, uint64_t tb
     cp += L;
     ct += L;
     const uint2 e = column_bits<VW, LP, NL>(w.tab0, ct, w.top - cp);
-    close_run(st, L > 0u && st.run_op != kOpMatch);
-    st.run_op = L > 0u ? kOpMatch : st.run_op;
-    st.run_len += L;
+    book_ops(st, late);
+    late.matches = L;
     // S (D0 clear) takes a base of both, I (VP' set) of the read, D of the text.
     const uint32_t from_p = one & (e.y | ~e.x), from_t = one & ~(e.x & e.y);
     const uint32_t code = from_p + 2u * from_t;
-    const uint32_t op = code == 3u ? kOpSubst : code;
-    close_run(st, one != 0u && st.run_op != op);
-    st.run_op = one ? op : st.run_op;
-    st.run_len += one;
+    late.edit = code == 3u ? kOpSubst : code;
     st.edits += one;
     cp += from_p;
     ct += from_t;
@@ -802,11 +816,16 @@ __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& 
     const uint32_t tend = walks ? min(text, static_cast<uint32_t>(cb + cols)) : ct;
     w.tab0 = tab_lane - at0 * Shape::kColBytes;
     w.hp0 = hp_lane - at0 * Shape::kHpBytes;
-    while (__any_sync(kMask, cp < goal && ct < tend)) {
-      // Two iterations to a vote.
-      walk_step<VW, LP, NL, kAny>(w, p.tb_table, st, cp, ct, goal, tend);
-      walk_step<VW, LP, NL, kAny>(w, p.tb_table, st, cp, ct, goal, tend);
+    LateOps late{0u, 0u};
+    // Each lane on its own until its counts are used up: a vote of the warp per
+    // round costs more than the lanes that wait for the longest walk. Two
+    // iterations to a test.
+    while (cp < goal && ct < tend) {
+      walk_step<VW, LP, NL, kAny>(w, p.tb_table, st, cp, ct, goal, tend, late);
+      walk_step<VW, LP, NL, kAny>(w, p.tb_table, st, cp, ct, goal, tend, late);
     }
+    if constexpr (!kAny) book_ops(st, late);
+    __syncwarp(kMask);
     if (cb + cols >= need || !__any_sync(kMask, cp < goal && ct < text)) break;
   }
   if (ga) {
