@@ -65,21 +65,40 @@ __device__ __forceinline__ uint32_t scan_buckets(uint32_t v, uint32_t* s) {
   return (warp ? s[warp - 1] : 0u) + x - v;
 }
 
-// Whether the sliced queue pays for n pairs, from the buckets' counts and starts
-// in the order (a thread each; longest first): only when the pair that nine in
-// ten are at least as long as has four fifths of the longest one's bases. Pairs
-// of one length end in a round of few lanes without turns; of mixed lengths, the
+// What the pairs' lengths say about the launch, from the buckets' counts and
+// starts in the order (a thread each; longest first):
+//
+// facts[0], whether the sliced queue pays: only when the pair that nine in ten
+// are at least as long as has four fifths of the longest one's bases. Pairs of
+// one length end in a round of few lanes without turns; of mixed lengths, the
 // short ones at the end of the order fill the lanes up as the long ones finish,
 // and turns cost more than they give (30,011 pairs of 2-20 kb: 2.32 ms with
 // turns, 1.88 without; 20,000 of 100 bases-50 kb: 5.8 and 4.9).
-__device__ __forceinline__ void wants_turns(uint32_t count, uint32_t start, uint32_t n, uint32_t* flag) {
+//
+// facts[1], the lanes per warp that finish all pairs by the time the longest one
+// takes, and a quarter more: where a few long pairs decide, fewer lanes share
+// their warps and their windows are shorter (the walk lasts as long as the
+// warp's longest).
+__device__ __forceinline__ void length_facts(uint32_t count, uint32_t start, uint32_t n, uint32_t warps,
+                                             uint32_t* facts) {
   __shared__ uint32_t longest, ninth;
+  __shared__ unsigned long long total;
   const uint32_t len = kLptBuckets - 1u - threadIdx.x;  // in 64 bases
   const uint32_t at = n - n / 10u - 1u;                 // the place of that pair
+  if (threadIdx.x == 0) total = 0;
+  __syncthreads();
   if (count && start == 0u) longest = len;
   if (count && start <= at && at < start + count) ninth = len;
+  unsigned long long mine = static_cast<unsigned long long>(count) * (len + 1u);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(kFull, mine, o);
+  if ((threadIdx.x & 31u) == 0u && mine) atomicAdd(&total, mine);
   __syncthreads();
-  if (threadIdx.x == 0) *flag = 5u * (ninth + 1u) >= 4u * (longest + 1u) ? 1u : 0u;
+  if (threadIdx.x == 0) {
+    facts[0] = 5u * (ninth + 1u) >= 4u * (longest + 1u) ? 1u : 0u;
+    const unsigned long long lanes = 5ull * total / (4ull * warps * (longest + 1u)) + 1ull;
+    facts[1] = lanes < 32ull ? static_cast<uint32_t>(lanes) : 32u;
+  }
 }
 
 // The whole order of a batch of up to kLptOneBlock pairs by one block, which also
@@ -87,8 +106,8 @@ __device__ __forceinline__ void wants_turns(uint32_t count, uint32_t start, uint
 constexpr uint32_t kLptOneBlock = 16384;
 
 __global__ void __launch_bounds__(kLptBuckets)
-    lpt_block_kernel(const uint32_t* __restrict__ read_len, uint32_t n, uint32_t* __restrict__ queue,
-                     uint32_t* __restrict__ order) {
+    lpt_block_kernel(const uint32_t* __restrict__ read_len, uint32_t n, uint32_t warps,
+                     uint32_t* __restrict__ queue, uint32_t* __restrict__ order) {
   __shared__ uint32_t h[kLptBuckets];
   __shared__ uint32_t s[32];
   const uint32_t x = threadIdx.x;
@@ -108,7 +127,7 @@ __global__ void __launch_bounds__(kLptBuckets)
     if (r < rounds) count_bucket(h, bucket[r], r * kLptBuckets + x < n);
   __syncthreads();
   const uint32_t start = scan_buckets(h[x], s);
-  wants_turns(h[x], start, n, queue + 5);
+  length_facts(h[x], start, n, warps, queue + 5);
   h[x] = start;
   __syncthreads();
 #pragma unroll
@@ -145,11 +164,11 @@ __global__ void __launch_bounds__(kLptBuckets)
 }
 
 // Exclusive scan of the bucket counts in place (one block of kLptBuckets threads).
-__global__ void __launch_bounds__(kLptBuckets) lpt_scan_kernel(uint32_t* hist, uint32_t n, uint32_t* turns) {
+__global__ void __launch_bounds__(kLptBuckets) lpt_scan_kernel(uint32_t* hist, uint32_t n, uint32_t warps, uint32_t* facts) {
   __shared__ uint32_t s[32];
   const uint32_t count = hist[threadIdx.x];
   const uint32_t start = scan_buckets(count, s);
-  if (turns) wants_turns(count, start, n, turns);
+  if (facts) length_facts(count, start, n, warps, facts);
   hist[threadIdx.x] = start;
 }
 
@@ -173,11 +192,11 @@ __global__ void __launch_bounds__(kLptBuckets)
 }
 
 cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* hist, uint32_t* order,
-                             uint32_t* turns, cudaStream_t s) {
+                             uint32_t warps, uint32_t* facts, cudaStream_t s) {
   const uint32_t blocks =
       static_cast<uint32_t>((static_cast<uint64_t>(n) + kLptPairs - 1) / kLptPairs);
   lpt_histogram_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, hist);
-  lpt_scan_kernel<<<1, kLptBuckets, 0, s>>>(hist, n, turns);
+  lpt_scan_kernel<<<1, kLptBuckets, 0, s>>>(hist, n, warps, facts);
   lpt_scatter_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, hist, order);
   count_launches(3);
   return cudaGetLastError();
@@ -408,7 +427,7 @@ cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePla
   // quarter of the pair when the pairs outnumber the resident lanes less than 16
   // times over (more pairs than that leave a tail of under a sixteenth of a
   // round) and are of about one length, which the ordering finds out on the
-  // device (wants_turns). A single pair has nobody to take turns with.
+  // device (length_facts). A single pair has nobody to take turns with.
   const uint64_t lanes = warps * plan->lp;
   const bool automatic = slice_windows == 0 && n > lanes && n < 16 * lanes;
   plan->slice = n < 2 ? 0u : slice_windows > 0 ? static_cast<uint32_t>(slice_windows) : automatic ? 64u : 0u;
@@ -444,12 +463,14 @@ cudaError_t launch_batched(const AlignParams& p, const LanePlan& plan, void* ws,
   // launch count at such sizes is something callers have come to rely on.)
   cudaError_t e = cudaSuccess;
   if (plan.lpt && p.n_pairs >= 64 && p.n_pairs <= kLptOneBlock) {
-    lpt_block_kernel<<<1, kLptBuckets, 0, s>>>(p.read_len, p.n_pairs, queue, order);
+    lpt_block_kernel<<<1, kLptBuckets, 0, s>>>(p.read_len, p.n_pairs, static_cast<uint32_t>(plan.warps),
+                                               queue, order);
     count_launches(1);
   } else {
     if ((e = cudaMemsetAsync(w, 0, L.order, s)) != cudaSuccess) return e;  // counters + histogram
     if (plan.lpt &&
-        (e = launch_lpt_order(p.read_len, p.n_pairs, hist, order, queue + 5, s)) != cudaSuccess)
+        (e = launch_lpt_order(p.read_len, p.n_pairs, hist, order, static_cast<uint32_t>(plan.warps),
+                              queue + 5, s)) != cudaSuccess)
       return e;
   }
   uint32_t* ring = reinterpret_cast<uint32_t*>(w + L.ring);

@@ -50,7 +50,8 @@ namespace ga {
 struct BatchArgs {
   uint32_t* queue;        // [0] hand-out counter (unsliced); ring: [1] head, [2] tail,
                           // [3] pairs not finished, [4] a warp's wait ran out,
-                          // [5] the pairs' lengths call for turns
+                          // with `order`, what the lengths say: [5] turns pay, [6]
+                          // lanes of a warp to use (0: all)
   const uint32_t* order;  // hand-out order (nullptr: index order)
   int cols;               // columns of a lane's table
   int lanes;              // lanes of a warp that take pairs
@@ -138,8 +139,10 @@ __global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParam
   const int leader = static_cast<int>(slot * NL);
   const bool writer = lane % NL == 0;
   const uint32_t slice = a.slice && (!a.turns || a.queue[5]) ? a.slice : 0u;
+  uint32_t lanes = static_cast<uint32_t>(a.lanes);
+  if (a.order && !slice && a.queue[6]) lanes = min(lanes, a.queue[6]);
   LanePair<VW> st{};
-  bool drained = slot >= static_cast<uint32_t>(a.lanes);
+  bool drained = slot >= lanes;
   bool first = true;        // nothing handed out to this warp yet
   uint32_t budget = 0;
   // The ring position this lane has reserved. As without turns, the first pairs
@@ -169,7 +172,7 @@ __global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParam
         // The first pairs go round the warps lane by lane, so that the longest
         // ones (handed out first) are spread over all schedulers; then each lane
         // takes the next one when it is done.
-        const uint32_t dealt = gridDim.x * static_cast<uint32_t>(a.lanes);
+        const uint32_t dealt = gridDim.x * lanes;
         uint32_t idx = slot * gridDim.x + blockIdx.x;
         if (!first) idx = p.n_pairs > dealt ? dealt + take_next<Shape>(a.queue, wants, lane) : p.n_pairs;
         if (want) {

@@ -107,9 +107,10 @@ cudaError_t launch_ablation(const AlignParams& p, int variant, uint64_t* table_b
 
 // Longest-read-first order of n pairs (counting sort over kLptBuckets read
 // length buckets): hist must hold kLptBuckets zeroed counters, order n entries.
-// *turns (may be null) receives 1 when the pairs are of about one length, else 0.
+// facts (may be null) receives 1 when the pairs are of about one length, else 0,
+// and the lanes of each of `warps` warps that they can use.
 cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* hist, uint32_t* order,
-                             uint32_t* turns, cudaStream_t s);
+                             uint32_t warps, uint32_t* facts, cudaStream_t s);
 
 // Kernel launches issued by the library (process-wide counter).
 uint64_t launch_count();
