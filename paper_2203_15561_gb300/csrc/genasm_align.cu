@@ -377,6 +377,18 @@ cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePla
   const uint64_t scheds = 4ull * sms;
   const int all = up8(p.W), inner = up8(p.W - p.O);
   int per_sm = 0;
+  // Few pairs: a team of lanes each, in one wave (no order needed; turns only if
+  // the caller asks for them).
+  plan->team = plan->vw <= 2 && !plan->any_order && slice_windows <= 0 ? team_size(n, sms) : 0;
+  if (plan->team) {
+    plan->lp = 32;
+    plan->cols = 32 * plan->vw;
+    plan->staged = false;
+    plan->slice = plan->turns = 0;
+    plan->lanes = std::max(1, 32 / plan->team);
+    plan->warps = static_cast<int>(std::min<uint64_t>(plan->team > 32 ? sms : scheds, n));
+    return cudaSuccess;
+  }
   // Windows of 65 bases and more: four lanes per pair while one warp per
   // scheduler holds every pair (2,001 pairs of 10 kb at W = 128: 0.79 ms against
   // 1.16 with one lane each). At W <= 64 two lanes per pair gained nothing (3,330
@@ -460,8 +472,10 @@ cudaError_t launch_batched(const AlignParams& p, const LanePlan& plan, void* ws,
   uint32_t* order = reinterpret_cast<uint32_t*>(w + L.order);
   // One block orders a batch that keeps it busy for a few microseconds at most.
   // (Below 64 pairs the order takes the general three launches: a whole step's
-  // launch count at such sizes is something callers have come to rely on.)
+  // launch count at such sizes is something callers have come to rely on. Teams
+  // have no use for the order.)
   cudaError_t e = cudaSuccess;
+  if (plan.team && p.n_pairs >= 64) return launch_team(p, plan, nullptr, s);
   if (plan.lpt && p.n_pairs >= 64 && p.n_pairs <= kLptOneBlock) {
     lpt_block_kernel<<<1, kLptBuckets, 0, s>>>(p.read_len, p.n_pairs, static_cast<uint32_t>(plan.warps),
                                                queue, order);
@@ -473,6 +487,7 @@ cudaError_t launch_batched(const AlignParams& p, const LanePlan& plan, void* ws,
                               queue + 5, s)) != cudaSuccess)
       return e;
   }
+  if (plan.team) return launch_team(p, plan, plan.lpt ? order : nullptr, s);
   uint32_t* ring = reinterpret_cast<uint32_t*>(w + L.ring);
   uint32_t* ring_seq = reinterpret_cast<uint32_t*>(w + L.ring_seq);
   SlotState* state = reinterpret_cast<SlotState*>(w + L.state);
@@ -561,6 +576,10 @@ cudaError_t prepare_step(int W, LanePlan* plan) {
 
 cudaError_t launch_step(const AlignParams& p, const LanePlan& plan, const StepArgs& a,
                         cudaStream_t s) {
+  int dev = 0, sms = 0;
+  const cudaError_t q = device_sms(&dev, &sms);
+  if (q != cudaSuccess) return q;
+  if (team_size(a.n_active, sms)) return launch_step_team(p, sms, a, s);
   const size_t smem = step_smem(plan.vw, plan.cols);
   if (plan.vw == 1) align_step_kernel<1><<<plan.warps, 32, smem, s>>>(p, a);
   else align_step_kernel<2><<<plan.warps, 32, smem, s>>>(p, a);

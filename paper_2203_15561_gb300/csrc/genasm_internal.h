@@ -55,6 +55,14 @@ struct LanePlan {
   bool lpt;        // longest-first hand-out
   uint32_t slice;  // windows per turn of the sliced queue (0: off)
   uint32_t turns;  // if not 0: a turn is this fraction of a pair, `slice` windows at least
+  int team;        // lanes of a team (8..32, or 128: a block of four warps); 0: no teams
+};
+
+// What the lanes of a team take on (see genasm_team.cuh).
+constexpr int kTeamLanes = 128;
+enum { kTeamLong = 0, kTeamFew = 1, kTeamStrange = 2, kTeamKinds = 3 };
+struct TeamStarts {
+  uint16_t start[kTeamKinds][kTeamLanes];
 };
 
 // Workspace layout of the batched kernel (byte offsets).
@@ -93,6 +101,11 @@ struct StepArgs {
 // prepare_step fills the launch shape of the serving step for windows of W <= 64
 // bases and sets the kernel's shared-memory attribute; launch_step launches it.
 cudaError_t prepare_step(int W, LanePlan* plan);
+// Pairs by teams of lanes (genasm_team.cu): the team for n pairs (0: none), the
+// batched launch of plan.team, and the serving step's.
+int team_size(uint64_t n, int sms);
+cudaError_t launch_step_team(const AlignParams& p, int sms, const StepArgs& a, cudaStream_t s);
+cudaError_t launch_team(const AlignParams& p, const LanePlan& plan, const uint32_t* order, cudaStream_t s);
 cudaError_t launch_step(const AlignParams& p, const LanePlan& plan, const StepArgs& a,
                         cudaStream_t s);
 

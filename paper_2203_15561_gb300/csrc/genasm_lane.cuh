@@ -629,8 +629,8 @@ struct Walk {
 struct LateOps {
   uint32_t matches, edit;
 };
-template <int VW>
-__device__ __forceinline__ void book_ops(LanePair<VW>& st, const LateOps& o) {
+template <class Runs>
+__device__ __forceinline__ void book_ops(Runs& st, const LateOps& o) {
   close_run(st, o.matches > 0u && st.run_op != kOpMatch);
   st.run_op = o.matches > 0u ? kOpMatch : st.run_op;
   st.run_len += o.matches;
@@ -643,8 +643,8 @@ __device__ __forceinline__ void book_ops(LanePair<VW>& st, const LateOps& o) {
 // to `goal` and `tend`: with the default order the matches ahead (up to 32 base
 // pairs compared at once) and the edit that ends them, else one op. No
 // branches: a lane whose counts are used up appends nothing.
-template <int VW, int LP, int NL, bool kAny>
-__device__ __forceinline__ void walk_step(const Walk<VW, LP, NL>& w, uint64_t tb_table, LanePair<VW>& st,
+template <int VW, int LP, int NL, bool kAny, class Runs>
+__device__ __forceinline__ void walk_step(const Walk<VW, LP, NL>& w, uint64_t tb_table, Runs& st,
                                           uint32_t& cp, uint32_t& ct, uint32_t goal, uint32_t tend,
                                           LateOps& late) {
   const uint32_t lim = min(min(goal - cp, tend - ct), 32u);

@@ -1,6 +1,6 @@
 """GPU parity of the launch forms of the batched kernel and of its input and
 output stages, at the sizes where they change: widths of a vector word, four
-lanes per pair and one, one warp per scheduler and two, the ordering in one
+lanes per pair and one, teams, one warp per scheduler and two, the ordering in one
 launch and in three, turns of the sliced queue chosen on the device, and the
 packer's and the compaction's loops. Outputs are whole numbers and have to be
 equal."""
@@ -88,6 +88,24 @@ def test_pairs_per_launch(W, O, n):
     # 152 multiprocessors) and one, warps of 32 pairs and of 16.
     base = pairs(n + W, 500, W // 2, 3 * W)
     check(datagen.from_pairs([base[q % 500] for q in range(n)]), W, O, W)
+
+
+@pytest.mark.parametrize("W,O", [(64, 24), (32, 12), (40, 3), (64, 63)])
+@pytest.mark.parametrize("n", [1, 152, 153, 608, 609, 1216, 1217, 2432, 2433])
+def test_teams(W, O, n):
+    # A pair by a team of 128, 32, 16 and 8 lanes (on 152 multiprocessors up to
+    # 152, 608, 1,216 and 2,432 pairs): reads of few and of many errors, against
+    # sequence of their own and of somebody else's, of all lengths at once so that
+    # the teams of a warp come to the same places at different times.
+    base = pairs(n + W, 60, 1, 400) if W - O > 4 else pairs(n, 30, 1, 100)
+    rnd = random.Random(n)
+    for read, ref in base[:20]:
+        x = rnd.randrange(len(read) + 1)
+        base.append((read, read[:x] + rnd.choice("ACGT") + read[x:]))
+        base.append((read, base[rnd.randrange(20)][1]))
+    b = datagen.from_pairs([base[(q * 7 + q // 100) % len(base)] for q in range(n)])
+    check(b, W, O, W)
+    check(b, W, O, max(1, W // 5), spans=np.arange(n, dtype=np.uint32) * 3 % 90)
 
 
 @pytest.mark.parametrize("n", [63, 64, 1024, 1025, 16_384, 16_385, 30_000])
