@@ -103,6 +103,60 @@ __global__ void pack_kernel(const uint8_t* __restrict__ ascii, uint64_t n, uint8
   if (n_invalid && bad) atomicAdd(n_invalid, bad);
 }
 
+// ASCII at any address, the output 4-aligned. A thread's 16 letters lie in two
+// aligned 16-byte blocks (the second is the next thread's first, in L1 by then):
+// loaded whole and shifted into place, `shift` bytes (1..15). The letters of the
+// blocks that are not wholly the sequence's, at its two ends, go byte by byte.
+__global__ void pack_shifted_kernel(const uint8_t* __restrict__ ascii, uint64_t n, uint32_t shift,
+                                    uint8_t* __restrict__ out, uint32_t* __restrict__ n_invalid) {
+  uint32_t bad = 0;
+  const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
+  const uint64_t first = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const uint4* in = reinterpret_cast<const uint4*>(ascii - shift);
+  uint32_t* to = reinterpret_cast<uint32_t*>(out);
+  // Chunk q is in blocks q and q + 1, which lie within the sequence for q = 1 ..
+  // whole - 2 (block 0 begins before it, block `whole` ends past it).
+  const uint64_t whole = (n + shift) / 16;
+  const uint64_t end = whole >= 2 ? whole - 1 : 0;
+  const bool by2 = (shift & 8u) != 0, by1 = (shift & 4u) != 0;
+  const uint32_t bits = 8u * (shift & 3u);
+  const auto chunk = [&](const uint4& x, const uint4& y) {
+    // Words from shift / 4 on, then the bits.
+    const uint32_t a0 = by2 ? x.z : x.x, a1 = by2 ? x.w : x.y, a2 = by2 ? y.x : x.z, a3 = by2 ? y.y : x.w,
+                   a4 = by2 ? y.z : y.x, a5 = by2 ? y.w : y.y;
+    const uint32_t b0 = by1 ? a1 : a0, b1 = by1 ? a2 : a1, b2 = by1 ? a3 : a2, b3 = by1 ? a4 : a3,
+                   b4 = by1 ? a5 : a4;
+    return make_uint4(__funnelshift_r(b0, b1, bits), __funnelshift_r(b1, b2, bits),
+                      __funnelshift_r(b2, b3, bits), __funnelshift_r(b3, b4, bits));
+  };
+  uint64_t q = first + 1;
+  for (; q + 3 * stride < end; q += 4 * stride) {
+    uint4 v[4], u[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      v[x] = __ldg(in + q + x * stride);
+      u[x] = __ldg(in + q + x * stride + 1);
+    }
+#pragma unroll
+    for (int x = 0; x < 4; ++x) to[q + x * stride] = pack16(chunk(v[x], u[x]), bad);
+  }
+  for (; q < end; q += stride) to[q] = pack16(chunk(__ldg(in + q), __ldg(in + q + 1)), bad);
+  // The first chunk and those from `end` on, a byte of four letters each.
+  const uint64_t nb = (n + 3) / 4, head = min(nb, static_cast<uint64_t>(4));
+  const uint64_t tail = max(head, 4 * end);
+  if (first < head + (nb - tail)) {
+    const uint64_t o = first < head ? first : tail + (first - head);
+    uint32_t byte = 0;
+    for (uint64_t y = 4 * o; y < 4 * o + 4 && y < n; ++y) {
+      bool ok;
+      byte |= code_of(ascii[y], ok) << (2 * (y - 4 * o));
+      bad += ok ? 0u : 1u;
+    }
+    out[o] = static_cast<uint8_t>(byte);
+  }
+  if (n_invalid && bad) atomicAdd(n_invalid, bad);
+}
+
 // Any alignment: one thread per output byte.
 __global__ void pack_bytes_kernel(const uint8_t* __restrict__ ascii, uint64_t n,
                                   uint8_t* __restrict__ out, uint32_t* __restrict__ n_invalid) {
@@ -195,6 +249,9 @@ cudaError_t launch_pack(const uint8_t* ascii, uint64_t n, uint8_t* packed, uint3
                        (reinterpret_cast<uintptr_t>(packed) % 4 == 0);
   if (aligned) {
     pack_kernel<<<blocks, 256, 0, s>>>(ascii, n, packed, n_invalid);
+  } else if (reinterpret_cast<uintptr_t>(packed) % 4 == 0) {
+    pack_shifted_kernel<<<blocks, 256, 0, s>>>(ascii, n, static_cast<uint32_t>(reinterpret_cast<uintptr_t>(ascii) % 16),
+                                               packed, n_invalid);
   } else {
     const uint64_t wb = ((n + 3) / 4 + 255) / 256;
     const int b2 = static_cast<int>(wb > 8ull * sms ? 8ull * sms : (wb < 1 ? 1 : wb));

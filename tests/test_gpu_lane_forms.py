@@ -157,6 +157,21 @@ def test_pack_long_inputs(n):
     assert int(bad.item()) == int((~known[a.long()]).sum())
 
 
+@pytest.mark.parametrize("shift", range(1, 16))
+def test_pack_at_any_address(shift):
+    # Every distance from a 16-byte address, with no, one and many whole blocks and
+    # other letters at both ends, against a copy at an aligned address.
+    for n in [*range(1, 70), 5 * 4096 + 7, 3_000_017]:
+        g = torch.Generator(device="cuda").manual_seed(n + shift)
+        a = torch.tensor(list(b"ACGTacgtN"), dtype=torch.uint8, device="cuda")[
+            torch.randint(0, 9, (n + shift,), generator=g, device="cuda")][shift:]
+        out = [torch.full(((n + 3) // 4 + 4,), 0xEE, dtype=torch.uint8, device="cuda") for _ in range(2)]
+        bad = [torch.zeros(1, dtype=torch.int32, device="cuda") for _ in range(2)]
+        ga.ga_pack_2bit(a, n, out[0], bad[0])
+        ga.ga_pack_2bit(a.clone(), n, out[1], bad[1])
+        assert torch.equal(out[0], out[1]) and int(bad[0]) == int(bad[1]), n
+
+
 @pytest.mark.parametrize("n,most", [(1, 3000), (7, 0), (1023, 20), (1024, 300), (1025, 300), (32_768, 40),
                                     (32_769, 40), (3000, 900), (1_050_000, 3)])
 def test_compaction(n, most):
