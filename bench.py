@@ -3,8 +3,8 @@
 
 One step = the whole hot path over one batch resident in HBM: 2-bit packing
 of the ASCII reads and references, then the batched alignment launch (window
-driver, pattern masks, distance calculation with row early termination,
-compressed table, traceback, CIGAR runs and distances). The default workload
+driver, pattern masks, edit-distance columns in difference form, traceback,
+CIGAR runs and distances). The default workload
 is 10,000 pairs of 10 kb PacBio-like reads (seed 2), W=64, O=24, k=64.
 
 Prints one JSON line (rank 0). ``--impl reference`` times the CPU oracle
@@ -30,11 +30,13 @@ import numpy as np  # noqa: E402
 METRIC = "10kb pairs/s & Gbases/s: batched+served vs plain GPU GenASM, bit-exact; p99 latency"
 WORKLOAD = 2
 W, O, K = 64, 24, 64
-OPS_PER_CELL = 6  # 2 funnel shifts + 4 three-input logic ops per 64-bit DP cell
-# Shared memory per traceback step: the three 4-byte band entries the step
-# tests (row d at column i+1, row d-1 at columns i and i+1) and its 4-byte
-# pattern-mask entry.
-SMEM_BYTES_PER_TB_STEP = 16
+# A window column: ten word operations per 32 rows (the recurrence of edit-distance
+# columns in difference form: one addition, two shifts and seven logic ops).
+OPS_PER_COLUMN = 10 * ((W + 31) // 32)
+# Shared memory: the Eq mask read and the {D0, VP'} entry stored per column, and
+# the entry read per traceback iteration (matches and the edit that ends them).
+EQ_BYTES = 4 * ((W + 31) // 32)
+ENTRY_BYTES = 8 * ((W + 31) // 32)
 WORKLOAD_NAMES = {
     2: "long-10kb-10000pairs (10 kb PacBio-like reads, 12% error, 5% flanks, seed 2)",
     3: "paper-scale-138929pairs (lengths normal(10 kb, 1.5 kb), 12% error, 5% flanks, "
@@ -267,8 +269,6 @@ def run_ours(args):
     assert (res.status == 0).all(), "alignment failed on the benchmark workload"
     cells = int(res.cells.sum())
     windows = int(res.n_windows.sum())
-    # Traceback steps: one per CIGAR op (the run lengths of every pair).
-    tb_steps = int(sum(int((res.runs(q) >> 4).sum(dtype=np.uint64)) for q in range(n)))
 
     # ---- batched (the headline): autotuned, alignment replayed from a CUDA graph ----
     if args.tuning:
@@ -341,25 +341,27 @@ def run_ours(args):
     # ---- roofline of the alignment kernel (integer ALU bound) ----
     peaks = ga.ga_measure_int_peak()
     peak_mix = peaks[2]
-    achieved = cells * OPS_PER_CELL / (align_ms * 1e-3)
+    ops = windows * W * OPS_PER_COLUMN
+    achieved = ops / (align_ms * 1e-3)
     roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_mix / 1e12,
                 "unit": "Tops/s (int32)", "frac": achieved / peak_mix, "traffic": None,
-                "kernel": "align_batched_kernel (+ 3 tiny LPT-sort kernels in the same call)",
-                "peak_source": "measured on this GPU by ga_measure_int_peak (DC cell mix: 2 SHF + 4 LOP3)",
+                "kernel": "align_batched_kernel (+ the ordering launch in the same call)",
+                "peak_source": "measured on this GPU by ga_measure_int_peak (2 SHF + 4 LOP3)",
                 "peak_lop3": peaks[0] / 1e12, "peak_shf": peaks[1] / 1e12,
-                "algorithmic_ops_per_launch": cells * OPS_PER_CELL, "cells_per_launch": cells,
+                "algorithmic_ops_per_launch": ops, "ops": "columns of all windows x %d" % OPS_PER_COLUMN,
+                "cells_per_launch": cells,
                 "rows_per_window": _rows_per_window(res.cells, res.n_windows),
                 "windows_per_launch": windows, "align_ms": align_ms, "pack_ms": pack_ms}
-    # Shared-memory side (secondary bound): the DC stores rows 0..d_min of the
-    # W-O+1 traceback columns of a window as 4-byte band entries (cells x
-    # (W-O+1)/W entries, exact for the windows with wt = W that are not the
-    # last), and each traceback step reads 16 bytes.
+    # Shared-memory side (secondary bound): every column reads an Eq mask, the W - O
+    # columns that a window commits are stored, a traceback iteration reads one
+    # (an edit each, and one per window that ends in matches at most).
     smem_peaks = ga.ga_measure_smem_peak()
-    smem_bytes = 4 * cells * (W - O + 1) // W + SMEM_BYTES_PER_TB_STEP * tb_steps
+    edits = int(res.dist.astype(np.int64).sum())
+    smem_bytes = windows * (W * EQ_BYTES + (W - O) * ENTRY_BYTES) + (edits + windows) * ENTRY_BYTES
     smem_achieved = smem_bytes / (align_ms * 1e-3)
     roofline["smem"] = {"achieved": smem_achieved / 1e9, "peak": smem_peaks[0] / 1e9,
                         "unit": "GB/s", "frac": smem_achieved / smem_peaks[0],
-                        "algorithmic_bytes_per_launch": smem_bytes, "tb_steps_per_launch": tb_steps,
+                        "algorithmic_bytes_per_launch": smem_bytes, "edits_per_launch": edits,
                         "peak_store": smem_peaks[1] / 1e9,
                         "peak_source": "measured on this GPU by ga_measure_smem_peak (16-byte loads, "
                                        "no bank conflicts, all SMs)"}
@@ -444,9 +446,9 @@ def run_ours(args):
                        "kernel": "batched (persistent, LPT work queue, CUDA graph)",
                        ("tuning" if args.tuning else "autotuned"): {**tuned.as_dict(),
                                                                            "tune_ms": tune_ms},
-                       "queue": "FIFO ring of pairs in turns of windows (slice_windows 0: turns of "
-                                "64 when the pairs outnumber the resident groups less than 16 times "
-                                "over, as here; -1: each pair to its end)",
+                       "queue": "a lane per pair, longest first; FIFO ring of turns of windows "
+                                "(slice_windows 0) when pairs of about one length outnumber the "
+                                "resident lanes less than 16 times over; -1: each pair to its end",
                        "l2": "no flush: each step streams 210 MB of ASCII input (> 126 MB L2) and "
                              "writes ~0.5 GB of CIGAR runs, which evicts the previous step's data"},
             "gbases_per_s": gbases,
@@ -753,7 +755,7 @@ def run_free_start(args, batch, db, dev, stream, ga, peak_mix, anchored, barrier
                 and int(r1.ref_consumed[p]) == int(ref.ref_consumed[q])
                 and int(r1.cells[p]) == int(ref.cells[q]) and np.array_equal(r1.runs(p), ref.runs(q))
                 for q, p in enumerate(ids))
-    achieved = cells * OPS_PER_CELL / (align_ms * 1e-3)
+    achieved = windows * W * OPS_PER_COLUMN / (align_ms * 1e-3)
     return {
         "workload": "long-10kb-10000pairs (as the headline), start span ceil(n / 20) per pair",
         "pairs_per_s": sum_over_ranks(n) / (ms * 1e-3),
@@ -763,7 +765,7 @@ def run_free_start(args, batch, db, dev, stream, ga, peak_mix, anchored, barrier
         "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_mix / 1e12,
                      "unit": "Tops/s (int32)", "frac": achieved / peak_mix,
                      "cells_per_launch": cells, "windows_per_launch": windows,
-                     "kernel": "locate_kernel + align_batched_kernel (+ LPT sort) in one call"},
+                     "kernel": "locate_kernel + align_batched_kernel (+ the ordering) in one call"},
         "mean_distance": float(r1.dist.mean()),
         "mean_distance_anchored": float(anchored.dist.mean()),
         "ref_start_mean": float(r1.ref_start.mean()),
@@ -776,7 +778,7 @@ def run_free_start(args, batch, db, dev, stream, ga, peak_mix, anchored, barrier
 
 def run_window_sweep(db, dev, ga):
     """The batched alignment of the same batch at other window sizes W (overlap O = 3W/8, the
-    64/24 ratio; no error cap): W <= 64 on the on-chip kernels, W > 64 on the 128-bit kernel.
+    64/24 ratio; no error cap), a vector word per 32 bases.
     Each W also with the free-start first window (start span ceil(n / 20), as the free-start
     leg), whose windows follow the read instead of the random left flank."""
     import torch
@@ -805,7 +807,7 @@ def run_window_sweep(db, dev, ga):
         ms = e0.elapsed_time(e1)
         row = {"W": Wv, "O": Ov, "k": Wv, "ms": ms, "pairs_per_s": n / (ms * 1e-3),
                "windows": windows, "all_ok": ok,
-               "kernel": "128-bit, tables in the workspace" if Wv > 64 else "on-chip tables"}
+               "kernel": f"{(Wv + 31) // 32} words per vector, tables in shared memory"}
         del wsb
         need = ga.ga_workspace_size_locate(n, Wv, Ov, Wv)
         wsb = torch.empty(max(need, 1), dtype=torch.uint8, device=dev)
@@ -828,7 +830,7 @@ def run_window_sweep(db, dev, ga):
 
 def run_ablation(db, dev, align_ms):
     """The paper's improvements one at a time (ga_align_ablation variants 0..3, table in
-    global memory) against the production kernel (align_ms, band table on chip): time,
+    global memory) against the production kernel (align_ms, columns on chip): time,
     window-table bytes, and the same outputs as the production kernel."""
     import torch
 
@@ -868,19 +870,26 @@ def run_ablation(db, dev, align_ms):
     foot = tb.view(-1, 5).sum(dim=0).cpu().numpy().astype(float)
     for v in range(4):
         out[v]["table_bytes_per_window"] = foot[v] / windows
-    # Table accesses: entries written (8-byte vectors; 4-byte band entries in
-    # production) plus the traceback's reads.
-    acc = [foot[v] / 8 + reads[v] for v in range(4)] + [foot[4] / 4 + reads[4]]
+    # The rows cut down to the 32 bits round the diagonal that the traceback can
+    # reach (no kernel stores them; counted): the method's smallest table.
+    band = foot[4]
+    # Production stores no rows: a 16-byte column entry per committed column.
+    column = float(windows * (W - O) * ENTRY_BYTES)
+    # Table accesses: entries written (8-byte vectors, 4-byte cut-down rows) plus the
+    # traceback's reads.
+    acc = [foot[v] / 8 + reads[v] for v in range(4)] + [band / 4 + reads[4]]
     for v in range(4):
         out[v]["table_accesses_per_window"] = acc[v] / windows
-    prod = {"what": "production (ga_align_batch): + reachable bits only (32-bit band entries), "
+    prod = {"what": "production (ga_align_batch): edit-distance columns in difference form, "
                     "table in shared memory", "ms": align_ms, "pairs_per_s": n / (align_ms * 1e-3),
-            "table_bytes_per_window": foot[4] / windows,
-            "table_accesses_per_window": acc[4] / windows}
+            "table_bytes_per_window": column / windows,
+            "table_accesses_per_window": (windows * (W - O) + edits + windows) / windows}
     return {"workload": "long-10kb-10000pairs (as the headline)", "windows": windows,
             "variants": out, "production": prod,
-            "footprint_reduction_plain_to_production": foot[0] / foot[4],
-            "access_reduction_plain_to_production": acc[0] / acc[4],
+            "footprint_reduction_plain_to_reachable_bits": foot[0] / band,
+            "footprint_reduction_plain_to_production": foot[0] / column,
+            "access_reduction_plain_to_reachable_bits": acc[0] / acc[4],
+            "access_reduction_plain_to_production": acc[0] / (windows * (W - O) + edits + windows),
             "accesses": "entries written (the footprint in entries) + traceback reads: plain "
                         "GenASM 4 per visited cell, the AND-only tables 2 per edit decision and "
                         "none per match step",

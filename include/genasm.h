@@ -130,6 +130,8 @@ int ga_workspace_size(uint32_t n_pairs, int W, int O, int k, size_t* bytes_out);
  *                    ones running alone; -1 = off (a pair runs to its end);
  *                    0 = automatic (turns of 64 windows when the pairs
  *                    outnumber the resident lanes, but less than 16 times).
+ *                    Turns asked for (> 0) run a lane per pair also where few
+ *                    pairs would get a team of lanes each.
  */
 typedef struct ga_tuning_s {
   int lanes_per_pair;
@@ -329,10 +331,10 @@ uint64_t ga_launch_count(void);
 /*
  * ga_set_queue_wait_limits - bounds, in polls of about 0.2 microseconds, of
  * the two waits of the batched kernel's sliced work queue (ga_tuning
- * slice_windows): a warp whose groups all wait for a published pair, and a
- * group waiting for its ring slot at the end of a turn. 0 restores a default
+ * slice_windows): a warp whose lanes all wait for a published pair, and a
+ * lane waiting for its ring slot at the end of a turn. 0 restores a default
  * (seconds: far beyond any legitimate wait). A wait that runs out ends its
- * group's work instead of hanging; pairs left unfinished report
+ * lane's work instead of hanging; pairs left unfinished report
  * GA_PAIR_TIMED_OUT. The defaults are never reached in normal operation;
  * short bounds exist to test that path. Applies to later launches (a
  * captured CUDA graph keeps the bounds it was captured with). Process-wide.

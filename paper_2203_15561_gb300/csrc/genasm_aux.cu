@@ -3,10 +3,10 @@
 //
 // Packer: each thread turns 16 ASCII bytes (one 16-byte load) into 4 packed
 // bytes (one 4-byte store), four such chunks at a time, so both sides of the
-// copy are fully coalesced. 1.25 bytes move per base; a gigabase takes 184
-// microseconds at the measured copy rate, and the integer ALU would take 360 at
-// 28 operations per four bases (what a code and an exact test per letter took):
-// the word-wide forms below take 9.
+// copy are fully coalesced. 1.25 bytes move per base: bound by memory, 185 us for
+// a gigabase (6.76 TB/s, 99% of the measured copy rate). The integer ALU would
+// take 360 at 28 operations per four bases (what a code and an exact test per
+// letter took: 311 us a gigabase); the word-wide forms below take 9.
 #include <algorithm>
 #include <cstdint>
 
@@ -71,11 +71,14 @@ __device__ __forceinline__ uint32_t pack16(const uint4& v, uint32_t& bad) {
                      __byte_perm(gather_codes(c), gather_codes(d), 0x0073), 0x5410);
 }
 
+// kLong: an input far larger than L2 (see launch_pack).
+template <bool kLong>
 __global__ void pack_kernel(const uint8_t* __restrict__ ascii, uint64_t n, uint8_t* __restrict__ out,
                             uint32_t* __restrict__ n_invalid) {
   const uint64_t chunks = n / 16;
   uint32_t bad = 0;
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
+  const auto letters = [](const uint4* at) { return kLong ? __ldg(at) : __ldcs(at); };
   const uint4* in = reinterpret_cast<const uint4*>(ascii);
   uint32_t* to = reinterpret_cast<uint32_t*>(out);
   uint64_t q = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -83,11 +86,11 @@ __global__ void pack_kernel(const uint8_t* __restrict__ ascii, uint64_t n, uint8
   for (; q + 3 * stride < chunks; q += 4 * stride) {
     uint4 v[4];
 #pragma unroll
-    for (int x = 0; x < 4; ++x) v[x] = __ldcs(in + q + x * stride);
+    for (int x = 0; x < 4; ++x) v[x] = letters(in + q + x * stride);
 #pragma unroll
     for (int x = 0; x < 4; ++x) to[q + x * stride] = pack16(v[x], bad);
   }
-  for (; q < chunks; q += stride) to[q] = pack16(__ldcs(in + q), bad);
+  for (; q < chunks; q += stride) to[q] = pack16(letters(in + q), bad);
   // Tail (n % 16 bytes): one thread, byte by byte.
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     for (uint64_t x = chunks * 16; x < n; x += 4) {
@@ -106,7 +109,8 @@ __global__ void pack_kernel(const uint8_t* __restrict__ ascii, uint64_t n, uint8
 // ASCII at any address, the output 4-aligned. A thread's 16 letters lie in two
 // aligned 16-byte blocks (the second is the next thread's first, in L1 by then):
 // loaded whole and shifted into place, `shift` bytes (1..15). The letters of the
-// blocks that are not wholly the sequence's, at its two ends, go byte by byte.
+// blocks that are not wholly the sequence's, at its two ends, go byte by byte. A
+// gigabase 214 us (the loads of L1 are twice the aligned form's), byte by byte 1,483.
 __global__ void pack_shifted_kernel(const uint8_t* __restrict__ ascii, uint64_t n, uint32_t shift,
                                     uint8_t* __restrict__ out, uint32_t* __restrict__ n_invalid) {
   uint32_t bad = 0;
@@ -244,11 +248,19 @@ cudaError_t launch_pack(const uint8_t* ascii, uint64_t n, uint8_t* packed, uint3
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const uint64_t chunks = n / 16;
   const uint64_t want = (chunks + 255) / 256;
-  const int blocks = static_cast<int>(want < 1 ? 1 : (want > 8ull * sms ? 8ull * sms : want));
+  // Eight resident blocks per SM, and letters marked as not to be kept, so that L2
+  // holds the packed bases for the alignment. From 320 MB on 64 blocks, that start
+  // as others end and keep the reads of all SMs close together, and plain loads
+  // (us, both ways: 100 MB 31, 38; 200 MB 48, 51; 300 MB 70, 70; 400 MB 94, 86;
+  // 600 MB 146, 118; 1 GB 234, 186).
+  const bool lng = n >= 320'000'000ull;
+  const uint64_t most = (lng ? 64ull : 8ull) * sms;
+  const int blocks = static_cast<int>(want < 1 ? 1 : std::min(want, most));
   const bool aligned = (reinterpret_cast<uintptr_t>(ascii) % 16 == 0) &&
                        (reinterpret_cast<uintptr_t>(packed) % 4 == 0);
   if (aligned) {
-    pack_kernel<<<blocks, 256, 0, s>>>(ascii, n, packed, n_invalid);
+    if (lng) pack_kernel<true><<<blocks, 256, 0, s>>>(ascii, n, packed, n_invalid);
+    else pack_kernel<false><<<blocks, 256, 0, s>>>(ascii, n, packed, n_invalid);
   } else if (reinterpret_cast<uintptr_t>(packed) % 4 == 0) {
     pack_shifted_kernel<<<blocks, 256, 0, s>>>(ascii, n, static_cast<uint32_t>(reinterpret_cast<uintptr_t>(ascii) % 16),
                                                packed, n_invalid);

@@ -133,9 +133,10 @@ def test_turns_chosen_for_pairs_of_one_length():
         assert np.array_equal(got.runs(p), ref.runs(int(order[p % 40])))
 
 
-@pytest.mark.parametrize("n", [16 * 64 - 5, 1_000_003, 62_300_000 + 13])
+@pytest.mark.parametrize("n", [16 * 64 - 5, 1_000_003, 62_300_000 + 13, 320_000_001])
 def test_pack_long_inputs(n):
-    # Past the sizes at which a thread packs four chunks at a time, with all byte
+    # Past the sizes at which a thread packs four chunks at a time, and at which the
+    # input counts as far larger than L2, with all byte
     # values among the letters (one in a hundred).
     g = torch.Generator(device="cuda").manual_seed(n)
     letters = torch.tensor(list(b"ACGTacgt"), dtype=torch.uint8, device="cuda")
