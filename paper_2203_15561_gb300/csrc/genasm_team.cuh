@@ -23,9 +23,10 @@
 //
 // A round of 128 lanes takes 8,350 cycles: 1,050 of preparation, 3,230 of columns
 // (integer ALU, one warp per scheduler), 2,320 of traceback (the longest walk of
-// the warp's lanes), 1,400 to follow the chain and write its runs; by 32 lanes
-// 7,100, the chain 770. Calls of one 10 kb pair: 625 us with one lane, 280.
-// 16 requests of up to 64 mixed pairs at the server: 5.9 ms, 3.5.
+// the warp's lanes), 1,300 to follow the chain and write its runs; by 32 lanes
+// 7,100, the chain 770. Calls of one 10 kb pair: 625 us with one lane, 277 (283
+// with all warps at every window's runs). 16 requests of up to 64 mixed pairs at
+// the server: 5.9 ms, 3.4.
 #pragma once
 
 #include <cstdint>
@@ -241,13 +242,15 @@ __device__ __forceinline__ void team_windows(const AlignParams& p, TeamPair<VW>&
   team_sync<NB>();
 
   // The chain of windows through the results, by every lane of the team alike;
-  // the next one's are read before this one's are used. `entry` is this lane's
-  // run of the window.
-  const uint32_t lists = base + Team::kTables + min(me.rank, Team::kRuns - 1u) * 128u;
+  // the next one's are read before this one's are used. The warps of a block take
+  // turns at writing the windows' runs; `entry` is this lane's run of the window.
+  const uint32_t place = NB > 1 ? lane : me.rank, places = NB > 1 ? 32u : me.size;
+  const uint32_t lists = base + Team::kTables + place * 128u;
   const auto list_of = [&](uint32_t t) {
     return lists + (NB > 1 ? (t >> 5) * Team::kWarp + (t & 31u) * 4u : t * 4u);
   };
   bool live = st.busy;
+  uint32_t turn = NB > 1 ? threadIdx.x >> 5 : 0u;
   uint4 a = lds128(posts + me.first * 32u);
   uint2 b = lds64(posts + me.first * 32u + 16u);
   uint32_t entry = lds32(list_of(me.first)), cur = me.first;
@@ -262,13 +265,13 @@ __device__ __forceinline__ void team_windows(const AlignParams& p, TeamPair<VW>&
     const bool joins = (b.x & 15u) == st.run_op;
     const uint32_t add = joins ? st.run_len : 0u;
     const uint32_t to = st.run_at + (joins ? 0u : 1u);
-    stg32_if(!joins && me.rank == 0u && r > 0u && st.run_at < st.room, st.out + st.run_at,
-             st.run_len << 4 | st.run_op);
-    stg32_if(me.rank + 1u < r && to + me.rank < st.room, st.out + to + me.rank,
-             entry + (me.rank == 0u ? add << 4 : 0u));
-    if (NB == 1 || Team::kRuns > 32u * NB) {
-      for (uint32_t i = me.rank + me.size; i + 1u < r; i += me.size)
-        stg32_if(to + i < st.room, st.out + to + i, lds32(list_of(cur) + (i - me.rank) * 128u));
+    if (NB == 1 || (turn++ & (NB - 1u)) == 0u) {
+      stg32_if(!joins && place == 0u && r > 0u && st.run_at < st.room, st.out + st.run_at,
+               st.run_len << 4 | st.run_op);
+      stg32_if(place + 1u < r && to + place < st.room, st.out + to + place,
+               entry + (place == 0u ? add << 4 : 0u));
+      for (uint32_t i = place + places; i + 1u < r; i += places)
+        stg32_if(to + i < st.room, st.out + to + i, lds32(list_of(cur) + (i - place) * 128u));
     }
     if (a.z >> 25) {
       st.status = kPairExceedsK;
