@@ -7,7 +7,7 @@
 // the resumable step kernel over every admitted, unfinished pair, which reads
 // the list of them from host-mapped memory and writes the finished slots there.
 // (A graph of a memset, the kernel and a copy-out kernel behind two copies of the
-// list took 15 us more of the 450 of a burst's step.) Each ga_server_step
+// list took 15 us more a step.) Each ga_server_step
 //   1. waits for the step launched by the previous call and takes the slots
 //      that finished in it (one event wait, no copy);
 //   2. admits waiting requests in arrival order while they fit: one H2D of
