@@ -101,12 +101,67 @@ __device__ __forceinline__ void length_facts(uint32_t count, uint32_t start, uin
   }
 }
 
+// facts[3..11], where a few long pairs decide: how the first pairs of the order are
+// split over the warps, pairs of about one length to a warp. A lane of a warp with
+// l busy lanes takes about 2.33 + 0.47 log2(l) us per window (W = 64; the longest of
+// l walks), so with a time t for the whole batch a pair of `len` may share its warp
+// with as many lanes as let len * cost(l) stay within t. Of 32 times between the
+// longest pair alone and in a full warp, the shortest whose warps suffice, all
+// other pairs in full warps. facts[3 + s]: the pairs that get at most
+// kSplitLanes(s) lanes. Only for vectors of two words and one warp per scheduler
+// (the one-word kernel lost 2% at 5,000 equal pairs). Alignment with the same
+// lanes in all warps, and split: 10,000 pairs of 2-20 kb 1.56 ms, 1.32; 5,000 of
+// 100 bases-20 kb at W = 48 1.65, 1.47; 20,000 of 100 bases-50 kb 4.52, 4.26 (a long
+// pair whose windows lose its path decides there).
+__device__ __forceinline__ float lane_cost(float lanes) { return 2.33f + 0.47f * __log2f(lanes); }
+
+__device__ __forceinline__ void length_split(uint32_t count, uint32_t start, uint32_t n, uint32_t warps,
+                                             uint32_t* s, uint32_t* facts) {
+  __shared__ uint32_t longer[kLptBuckets + 1], mass[kLptBuckets + 1];  // in buckets before x
+  const uint32_t x = threadIdx.x;
+  const uint32_t m = count * (kLptBuckets - x);
+  longer[x] = start;
+  mass[x] = scan_buckets(m, s);
+  if (x == kLptBuckets - 1u) {
+    longer[kLptBuckets] = n;
+    mass[kLptBuckets] = mass[x] + m;
+  }
+  __syncthreads();
+  if (x >= 32u || facts[0]) return;
+  uint32_t top = 0;  // the longest pair's bucket
+  for (uint32_t b = kLptBuckets / 2; b; b >>= 1)
+    if (longer[top + b] == 0u) top += b;
+  const float longest = static_cast<float>(kLptBuckets - top), all = lane_cost(32.0f);
+  const float t = longest * (lane_cost(1.0f) + (all - lane_cost(1.0f)) * static_cast<float>(x) / 31.0f);
+  uint32_t used = 0, at = kLptBuckets, given = 0;
+  uint32_t upto[kSplits];
+#pragma unroll
+  for (int k = 0; k < kSplits; ++k) {
+    const uint32_t more = k + 1 < kSplits ? kSplitLanes(k + 1) : 32u;
+    const uint32_t len = static_cast<uint32_t>(t / lane_cost(static_cast<float>(more)));  // may have `more` lanes
+    at = kLptBuckets - min(len, static_cast<uint32_t>(kLptBuckets));
+    upto[k] = longer[at];
+    used += (upto[k] - given + kSplitLanes(k) - 1u) / kSplitLanes(k);
+    given = upto[k];
+  }
+  const float rest = static_cast<float>(mass[kLptBuckets] - mass[at]) * all * 1.05f;
+  const bool fits = used < warps && rest <= t * 32.0f * static_cast<float>(warps - used);
+  const uint32_t able = __ballot_sync(kFull, fits);
+  // Against the same number of lanes in all warps.
+  const float even = max(longest, static_cast<float>(mass[kLptBuckets]) / static_cast<float>(warps * facts[1])) *
+                     lane_cost(static_cast<float>(facts[1]));
+  if (able && x == static_cast<uint32_t>(__ffs(able)) - 1u && t < 0.95f * even) {
+#pragma unroll
+    for (int k = 0; k < kSplits; ++k) facts[3 + k] = upto[k];
+  }
+}
+
 // The whole order of a batch of up to kLptOneBlock pairs by one block, which also
 // zeroes the queue's counters.
 constexpr uint32_t kLptOneBlock = 16384;
 
 __global__ void __launch_bounds__(kLptBuckets)
-    lpt_block_kernel(const uint32_t* __restrict__ read_len, uint32_t n, uint32_t warps,
+    lpt_block_kernel(const uint32_t* __restrict__ read_len, uint32_t n, uint32_t warps, bool split,
                      uint32_t* __restrict__ queue, uint32_t* __restrict__ order) {
   __shared__ uint32_t h[kLptBuckets];
   __shared__ uint32_t s[32];
@@ -128,6 +183,8 @@ __global__ void __launch_bounds__(kLptBuckets)
   __syncthreads();
   const uint32_t start = scan_buckets(h[x], s);
   length_facts(h[x], start, n, warps, queue + 5);
+  __syncthreads();
+  if (split) length_split(h[x], start, n, warps, s, queue + 5);
   h[x] = start;
   __syncthreads();
 #pragma unroll
@@ -164,11 +221,14 @@ __global__ void __launch_bounds__(kLptBuckets)
 }
 
 // Exclusive scan of the bucket counts in place (one block of kLptBuckets threads).
-__global__ void __launch_bounds__(kLptBuckets) lpt_scan_kernel(uint32_t* hist, uint32_t n, uint32_t warps, uint32_t* facts) {
+__global__ void __launch_bounds__(kLptBuckets) lpt_scan_kernel(uint32_t* hist, uint32_t n, uint32_t warps,
+                                                                bool split, uint32_t* facts) {
   __shared__ uint32_t s[32];
   const uint32_t count = hist[threadIdx.x];
   const uint32_t start = scan_buckets(count, s);
   if (facts) length_facts(count, start, n, warps, facts);
+  __syncthreads();
+  if (facts && split) length_split(count, start, n, warps, s, facts);
   hist[threadIdx.x] = start;
 }
 
@@ -192,11 +252,11 @@ __global__ void __launch_bounds__(kLptBuckets)
 }
 
 cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* hist, uint32_t* order,
-                             uint32_t warps, uint32_t* facts, cudaStream_t s) {
+                             uint32_t warps, bool split, uint32_t* facts, cudaStream_t s) {
   const uint32_t blocks =
       static_cast<uint32_t>((static_cast<uint64_t>(n) + kLptPairs - 1) / kLptPairs);
   lpt_histogram_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, hist);
-  lpt_scan_kernel<<<1, kLptBuckets, 0, s>>>(hist, n, warps, facts);
+  lpt_scan_kernel<<<1, kLptBuckets, 0, s>>>(hist, n, warps, split, facts);
   lpt_scatter_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, hist, order);
   count_launches(3);
   return cudaGetLastError();
@@ -478,13 +538,13 @@ cudaError_t launch_batched(const AlignParams& p, const LanePlan& plan, void* ws,
   if (plan.team && p.n_pairs >= 64) return launch_team(p, plan, nullptr, s);
   if (plan.lpt && p.n_pairs >= 64 && p.n_pairs <= kLptOneBlock) {
     lpt_block_kernel<<<1, kLptBuckets, 0, s>>>(p.read_len, p.n_pairs, static_cast<uint32_t>(plan.warps),
-                                               queue, order);
+                                               plan.staged && plan.vw == 2, queue, order);
     count_launches(1);
   } else {
     if ((e = cudaMemsetAsync(w, 0, L.order, s)) != cudaSuccess) return e;  // counters + histogram
     if (plan.lpt &&
         (e = launch_lpt_order(p.read_len, p.n_pairs, hist, order, static_cast<uint32_t>(plan.warps),
-                              queue + 5, s)) != cudaSuccess)
+                              plan.staged && plan.vw == 2, queue + 5, s)) != cudaSuccess)
       return e;
   }
   if (plan.team) return launch_team(p, plan, plan.lpt ? order : nullptr, s);

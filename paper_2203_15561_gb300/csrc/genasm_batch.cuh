@@ -51,7 +51,8 @@ struct BatchArgs {
   uint32_t* queue;        // [0] hand-out counter (unsliced); ring: [1] head, [2] tail,
                           // [3] pairs not finished, [4] a warp's wait ran out,
                           // with `order`, what the lengths say: [5] turns pay, [6]
-                          // lanes of a warp to use (0: all)
+                          // lanes of a warp to use (0: all), [8..16] the split of
+                          // the longest over the warps (see length_split; 0: none)
   const uint32_t* order;  // hand-out order (nullptr: index order)
   int cols;               // columns of a lane's table
   int lanes;              // lanes of a warp that take pairs
@@ -141,6 +142,34 @@ __global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParam
   const uint32_t slice = a.slice && (!a.turns || a.queue[5]) ? a.slice : 0u;
   uint32_t lanes = static_cast<uint32_t>(a.lanes);
   if (a.order && !slice && a.queue[6]) lanes = min(lanes, a.queue[6]);
+  // The first pairs go round the warps lane by lane, so that the longest ones
+  // (handed out first) are spread over all schedulers; then each lane takes the
+  // next one when it is done.
+  uint32_t deal = slot * gridDim.x + blockIdx.x, dealt = gridDim.x * lanes;
+  if constexpr (kStaged && VW == 2) {
+    if (a.order && !slice && a.queue[8 + kSplits - 1]) {
+      // The long ones are split over the first warps, few lanes each; the others go
+      // round the rest, all lanes.
+      uint32_t warps = 0, given = 0, end = p.n_pairs;
+      lanes = 0;
+      for (int k = 0; k < kSplits; ++k) {
+        const uint32_t upto = a.queue[8 + k], l = kSplitLanes(k), w = (upto - given + l - 1u) / l;
+        if (lanes == 0 && blockIdx.x < warps + w) {
+          lanes = l;
+          deal = given + (blockIdx.x - warps) * l + slot;
+          end = upto;
+        }
+        warps += w;
+        given = upto;
+      }
+      dealt = given + (gridDim.x - warps) * 32u;
+      if (lanes == 0) {
+        lanes = 32;
+        deal = given + slot * (gridDim.x - warps) + (blockIdx.x - warps);
+      }
+      if (deal >= end) deal = p.n_pairs;
+    }
+  }
   LanePair<VW> st{};
   bool drained = slot >= lanes;
   bool first = true;        // nothing handed out to this warp yet
@@ -169,11 +198,7 @@ __global__ void __launch_bounds__(LP * NL) align_batched_kernel(const AlignParam
           quit = __shfl_sync(kMask, quit ? 1u : 0u, leader) != 0u;
         }
       } else {
-        // The first pairs go round the warps lane by lane, so that the longest
-        // ones (handed out first) are spread over all schedulers; then each lane
-        // takes the next one when it is done.
-        const uint32_t dealt = gridDim.x * lanes;
-        uint32_t idx = slot * gridDim.x + blockIdx.x;
+        uint32_t idx = deal;
         if (!first) idx = p.n_pairs > dealt ? dealt + take_next<Shape>(a.queue, wants, lane) : p.n_pairs;
         if (want) {
           if (idx < p.n_pairs) pair = a.order ? a.order[idx] : idx;

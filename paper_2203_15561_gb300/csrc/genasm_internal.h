@@ -121,9 +121,18 @@ cudaError_t launch_ablation(const AlignParams& p, int variant, uint64_t* table_b
 // Longest-read-first order of n pairs (counting sort over kLptBuckets read
 // length buckets): hist must hold kLptBuckets zeroed counters, order n entries.
 // facts (may be null) receives 1 when the pairs are of about one length, else 0,
-// and the lanes of each of `warps` warps that they can use.
+// the lanes of each of `warps` warps that they can use, and with `split` how the
+// longest are split over the warps (n up to 2^22).
 cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* hist, uint32_t* order,
-                             uint32_t warps, uint32_t* facts, cudaStream_t s);
+                             uint32_t warps, bool split, uint32_t* facts, cudaStream_t s);
+
+// Lanes per warp of the long pairs that decide how long a batch takes (see
+// length_split): how many, and their numbers.
+constexpr int kSplits = 9;
+__host__ __device__ constexpr uint32_t kSplitLanes(int k) {
+  constexpr uint32_t lanes[kSplits] = {1, 2, 3, 4, 6, 8, 12, 16, 24};
+  return lanes[k];
+}
 
 // Kernel launches issued by the library (process-wide counter).
 uint64_t launch_count();

@@ -114,6 +114,16 @@ def test_ordering_sizes(n):
     check(datagen.from_pairs([base[q % 300] for q in range(n)]), 64, 24, 64)
 
 
+@pytest.mark.parametrize("n,long", [(2_500, 8), (5_000, 700), (20_000, 90)])
+def test_few_long_pairs_among_many(n, long):
+    # Long pairs that decide how long the batch takes: a few lanes of some warps.
+    some = pairs(n, 24, 5_000, 9_000) + pairs(n + 1, 24, 1_500, 5_000)
+    rest = pairs(n + 2, 200, 30, 600)
+    b = datagen.from_pairs([some[q % 48] if q < long else rest[q % 200] for q in range(n)])
+    check(b, 64, 24, 64)
+    check(b, 32, 12, 32, spans=np.arange(n, dtype=np.uint32) % 90)
+
+
 def test_turns_chosen_for_pairs_of_one_length():
     # More pairs than one warp per scheduler holds, all of one length: the sliced
     # queue takes turns of 64 windows (reads of 70 windows have two).
