@@ -375,7 +375,8 @@ int ga_measure_smem_peak(double out[2], ga_stream_t stream);
  * The kernels read the packed buffers in aligned 4-byte words: the words
  * holding a sequence's first and last bytes are read whole, so those bytes'
  * neighbours must lie in mapped device memory (always true inside one
- * device allocation, whose start is at least 256-byte aligned).
+ * device allocation, whose start is at least 256-byte aligned). Nothing is
+ * read at the offset of an empty sequence.
  * Outputs (device, n_pairs each): d_dist edit distance (-1 unless status OK);
  * d_status GA_PAIR_*; d_ref_consumed reference bases the alignment spans
  * (-1 on failure); d_n_runs CIGAR runs written. d_cigar receives pair p's

@@ -42,6 +42,7 @@
 
 #include "genasm_internal.h"
 #include "genasm_window.cuh"
+#include "genasm_words.h"
 
 namespace ga {
 
@@ -213,9 +214,9 @@ __device__ __forceinline__ void load_words(const uint8_t* seq, uint32_t len, uin
   const uintptr_t a = reinterpret_cast<uintptr_t>(seq) + (pos >> 2);
   const uint32_t* wa = reinterpret_cast<const uint32_t*>(a & ~static_cast<uintptr_t>(3));
   const uint32_t o = 8u * static_cast<uint32_t>(a & 3u) + 2u * (pos & 3u);
-  const uint32_t lim = o + 2u * min(len > pos ? len - pos : 0u, 32u * VW);  // first bit past the window
+  const uint32_t end = bases_end(o, len, pos, 32u * VW);
 #pragma unroll
-  for (int k = 0; k <= 2 * VW; ++k) x[k] = 32u * k < lim ? __ldg(wa + k) : 0u;
+  for (int k = 0; k <= 2 * VW; ++k) x[k] = holds_base(k, o, end) ? __ldg(wa + k) : 0u;
 }
 
 // Starts copying the words from base `pos` on that hold its window's bases and
@@ -227,14 +228,14 @@ __device__ __forceinline__ uint32_t stage_words(const uint8_t* seq, uint32_t len
   const uintptr_t a = reinterpret_cast<uintptr_t>(seq) + (pos >> 2);
   const uint32_t* wa = reinterpret_cast<const uint32_t*>(a & ~static_cast<uintptr_t>(3));
   const uint32_t o = 8u * static_cast<uint32_t>(a & 3u) + 2u * (pos & 3u);
-  const uint32_t lim = o + 2u * min(len > pos ? len - pos : 0u, 16u * kWords);  // first bit past the end
-  if (lim >= 32u * kWords) {
+  const uint32_t end = bases_end(o, len, pos, 16u * kWords);
+  if (end >= 32u * kWords) {
 #pragma unroll
     for (int k = 0; k < kWords; ++k) copy_word(to + 128u * k, wa + k);
   } else {
 #pragma unroll
     for (int k = 0; k < kWords; ++k)
-      if (32u * k < lim) copy_word(to + 128u * k, wa + k);
+      if (holds_base(k, o, end)) copy_word(to + 128u * k, wa + k);
   }
   return static_cast<uint32_t>(a) & ~3u;
 }

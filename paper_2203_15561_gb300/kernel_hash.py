@@ -17,7 +17,7 @@ CSRC = Path(__file__).resolve().parent / "csrc"
 # The translation unit of the batched alignment kernel: the sources its
 # counters depend on.
 KERNEL_SOURCES = [CSRC / "genasm_align.cu", CSRC / "genasm_batch.cuh", CSRC / "genasm_lane.cuh",
-                  CSRC / "genasm_window.cuh", CSRC / "genasm_internal.h",
+                  CSRC / "genasm_window.cuh", CSRC / "genasm_words.h", CSRC / "genasm_internal.h",
                   CSRC.parent.parent / "include" / "genasm.h"]
 
 
