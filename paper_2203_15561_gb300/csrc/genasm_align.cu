@@ -608,10 +608,11 @@ size_t step_smem(int vw, int cols) {
 
 template <int VW>
 cudaError_t step_setup(int cols, int* warps_per_sm) {
+  // (The attribute is the function's, not the server's: a server of another W sets
+  // the same.)
   const size_t smem = step_smem(VW, cols);
-  cudaError_t e = cudaFuncSetAttribute(align_step_kernel<VW>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  const cudaError_t e = cudaFuncSetAttribute(align_step_kernel<VW>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedOptIn);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(warps_per_sm, align_step_kernel<VW>, 32, smem);
 }
