@@ -130,8 +130,11 @@ int ga_workspace_size(uint32_t n_pairs, int W, int O, int k, size_t* bytes_out);
  *                    ones running alone; -1 = off (a pair runs to its end);
  *                    0 = automatic (turns of 64 windows when the pairs
  *                    outnumber the resident lanes, but less than 16 times).
- *                    Turns asked for (> 0) run a lane per pair also where few
- *                    pairs would get a team of lanes each.
+ *                    Turns that a call's own tuning asks for (> 0) run a lane
+ *                    per pair also where few pairs would get a team of lanes
+ *                    each; stored ones (ga_autotune, ga_tuning_set) are taken
+ *                    where the pairs outnumber the resident lanes and are of
+ *                    about one length.
  */
 typedef struct ga_tuning_s {
   int lanes_per_pair;

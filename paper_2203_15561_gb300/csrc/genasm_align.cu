@@ -426,7 +426,7 @@ cudaError_t shape_warps(int dev, const LanePlan& plan, int* warps) {
 
 }  // namespace
 
-cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePlan* plan) {
+cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool lpt, LanePlan* plan) {
   int dev = 0, sms = 0;
   cudaError_t e = device_sms(&dev, &sms);
   if (e != cudaSuccess) return e;
@@ -438,8 +438,10 @@ cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePla
   const int all = up8(p.W), inner = up8(p.W - p.O);
   int per_sm = 0;
   // Few pairs: a team of lanes each, in one wave (no order needed; turns only if
-  // the caller asks for them).
-  plan->team = plan->vw <= 2 && !plan->any_order && slice_windows <= 0 ? team_size(n, sms) : 0;
+  // the call itself asks for them: a stored tuning was chosen for some other batch,
+  // and one pair of 10 kb takes 840 us with its turns, 295 by a team).
+  const bool turns_asked = slice_windows > 0 && asked;
+  plan->team = plan->vw <= 2 && !plan->any_order && !turns_asked ? team_size(n, sms) : 0;
   if (plan->team) {
     plan->lp = 32;
     plan->cols = 32 * plan->vw;
@@ -495,15 +497,19 @@ cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePla
   const uint64_t warps = std::min<uint64_t>(static_cast<uint64_t>(sms) * per_sm, n);
   plan->warps = static_cast<int>(warps);
   plan->lanes = static_cast<int>(std::min<uint64_t>(plan->lp, (n + warps - 1) / warps));
-  // The sliced queue: turns of the tuning's choice, else of 64 windows or a
-  // quarter of the pair when the pairs outnumber the resident lanes less than 16
-  // times over (more pairs than that leave a tail of under a sixteenth of a
-  // round) and are of about one length, which the ordering finds out on the
-  // device (length_facts). A single pair has nobody to take turns with.
+  // The sliced queue: turns of the call's choice, else of 64 windows or a quarter
+  // of the pair when the pairs outnumber the resident lanes less than 16 times over
+  // (more pairs than that leave a tail of under a sixteenth of a round) and are of
+  // about one length, which the ordering finds out on the device (length_facts).
+  // Stored turns are taken where the pairs outnumber the lanes and are of about one
+  // length (stored turns of 64, and without them: 10,000 pairs of 10 kb 1.18 ms,
+  // 0.97; 20,000 of 100 bases-50 kb 5.72, 4.26). A single pair has nobody to take
+  // turns with.
   const uint64_t lanes = warps * plan->lp;
   const bool automatic = slice_windows == 0 && n > lanes && n < 16 * lanes;
-  plan->slice = n < 2 ? 0u : slice_windows > 0 ? static_cast<uint32_t>(slice_windows) : automatic ? 64u : 0u;
-  plan->turns = automatic ? 4u : 0u;
+  const bool stored = slice_windows > 0 && !asked && n > lanes;
+  plan->slice = n < 2 ? 0u : turns_asked || stored ? static_cast<uint32_t>(slice_windows) : automatic ? 64u : 0u;
+  plan->turns = automatic ? 4u : stored ? kFixedTurns : 0u;
   // (waiting lanes take part in the ring as well)
   if (plan->slice) plan->lanes = plan->lp;
   return cudaSuccess;

@@ -57,7 +57,8 @@ struct BatchArgs {
   int cols;               // columns of a lane's table
   int lanes;              // lanes of a warp that take pairs
   uint32_t slice;         // windows per turn (0: a pair runs to its end)
-  uint32_t turns;         // if not 0: a turn is this fraction of a pair, `slice` windows at least
+  uint32_t turns;         // if not 0: turns only where they pay (queue[5]), each this fraction
+                          // of its pair and `slice` windows at least
   uint32_t* ring;         // 2n ring slots: pair ids
   uint32_t* ring_seq;     // 2n: each slot's sequence number
   SlotState* state;       // per pair: saved window state (all zero: not started)

@@ -90,7 +90,7 @@ int plan_batched(const ga::AlignParams& p, int k, const ga_tuning* t, int mode, 
   const int rc = resolve(p.W, p.O, k, t, &r, mode);
   if (rc != GA_OK) return rc;
   if (!d_workspace || ws_bytes < ga::workspace_layout(p.n_pairs).total) return GA_ENOSPC;
-  return cuda_fail(ga::lane_plan(p, r.slice_windows, r.lpt > 0, plan));
+  return cuda_fail(ga::lane_plan(p, r.slice_windows, t != nullptr, r.lpt > 0, plan));
 }
 
 }  // namespace

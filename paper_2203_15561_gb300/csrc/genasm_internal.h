@@ -54,9 +54,13 @@ struct LanePlan {
   bool staged;     // the next window's bases copied ahead (see genasm_lane.cuh)
   bool lpt;        // longest-first hand-out
   uint32_t slice;  // windows per turn of the sliced queue (0: off)
-  uint32_t turns;  // if not 0: a turn is this fraction of a pair, `slice` windows at least
+  uint32_t turns;  // if not 0: turns only for pairs of about one length, each this
+                   // fraction of its pair and `slice` windows at least
   int team;        // lanes of a team (8..32, or 128: a block of four warps); 0: no teams
 };
+
+// `turns` for turns of `slice` windows whatever the pair's length.
+constexpr uint32_t kFixedTurns = 1u << 20;
 
 // What the lanes of a team take on (see genasm_team.cuh).
 constexpr int kTeamLanes = 128;
@@ -173,7 +177,8 @@ cudaError_t resolve_tuning(int W, int O, int k, const struct ga_tuning_s* t, int
                            struct ga_tuning_s* out);
 
 // Launch shape of the batched kernel for p (p.n_pairs, W, O, order) on the
-// current device; slice_windows and lpt as in ga_tuning.
-cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool lpt, LanePlan* plan);
+// current device; slice_windows and lpt as in ga_tuning. `asked`: they come with
+// the call, not from a stored tuning.
+cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool lpt, LanePlan* plan);
 
 }  // namespace ga
