@@ -156,17 +156,20 @@ int ga_tuning_get(int W, int O, int k, ga_tuning* out);
 int ga_tuning_set(int W, int O, int k, const ga_tuning* tuning);
 
 /*
- * ga_autotune - the autotuner of the batched kernel. Runs the current
- * default once on the caller's sample (with statistics), then times a
- * candidate set of (lpt, slice_windows) with CUDA events, one warm-up
- * and one timed run each, and stores the fastest as the default for this
- * device and (W, O, k). Arguments as ga_align_batch (outputs are
- * overwritten; d_n_windows and d_cells are required); the workspace must hold
- * ga_autotune_workspace_size(n_pairs, W, O, k) bytes. Synchronous: returns
- * once every run has finished. *best / *best_ms (either may be NULL) receive
- * the choice and its time. The paper gives no tuning procedure.
+ * ga_autotune - the autotuner of the batched kernel. Runs the current default
+ * once on the caller's sample (with statistics), then times the library's own
+ * choice and, where the pairs outnumber the resident lanes and are of about
+ * one length, turns of 32, 64 and 128 windows (slice_windows) with CUDA
+ * events, one warm-up and one timed run each. Stores the fastest, or the
+ * library's choice where none is 2% faster, as the default for this device and
+ * (W, O, k); pairs stay longest first (lpt 1). Arguments as ga_align_batch
+ * (outputs are overwritten; d_n_windows and d_cells are required); the
+ * workspace must hold ga_autotune_workspace_size(n_pairs, W, O, k) bytes.
+ * Synchronous: returns once every run has finished. *best / *best_ms (either
+ * may be NULL) receive the choice and its time. The paper gives no tuning
+ * procedure.
  * Errors: GA_EINVAL (also for W > GA_MAX_W_ONCHIP: wider windows take no
- * tuning), GA_ENOSPC (no candidate fits the workspace), GA_ECUDA.
+ * tuning), GA_ENOSPC (workspace too small), GA_ECUDA.
  */
 int ga_autotune(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_t* d_read_len,
                 const uint8_t* d_refs, const uint64_t* d_ref_off, const uint32_t* d_ref_len,

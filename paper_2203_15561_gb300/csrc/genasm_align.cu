@@ -515,6 +515,24 @@ cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool 
   return cudaSuccess;
 }
 
+cudaError_t turns_matter(uint32_t n_pairs, int W, int O, const void* ws, cudaStream_t s, bool* yes) {
+  AlignParams p{};
+  p.n_pairs = n_pairs;
+  p.W = W;
+  p.O = O;
+  p.tb_table = tb_table(kTbOrderDefault);
+  LanePlan plan{};
+  *yes = false;
+  cudaError_t e = lane_plan(p, 64, false, true, &plan);
+  if (e != cudaSuccess || !plan.slice) return e;
+  uint32_t alike = 0;
+  const char* fact = static_cast<const char*>(ws) + workspace_layout(n_pairs).queue + 5 * sizeof(uint32_t);
+  e = cudaMemcpyAsync(&alike, fact, sizeof(alike), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  *yes = alike != 0;
+  return e;
+}
+
 WorkspaceLayout workspace_layout(uint32_t n_pairs) {
   auto up = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
   WorkspaceLayout L{};

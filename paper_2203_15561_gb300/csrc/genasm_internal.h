@@ -181,4 +181,9 @@ cudaError_t resolve_tuning(int W, int O, int k, const struct ga_tuning_s* t, int
 // the call, not from a stored tuning.
 cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool lpt, LanePlan* plan);
 
+// Whether stored turns would be taken for n_pairs whose lengths an alignment
+// without turns of its own, longest first, has just left in the workspace (waits
+// for the stream).
+cudaError_t turns_matter(uint32_t n_pairs, int W, int O, const void* ws, cudaStream_t s, bool* yes);
+
 }  // namespace ga

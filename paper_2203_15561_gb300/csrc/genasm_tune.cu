@@ -1,20 +1,20 @@
 // Autotuner and CUDA-graph capture of the batched alignment step.
 //
-// Autotuner: how fast a batch runs depends on the order in which its pairs are
-// handed out and on the windows per turn of the sliced queue. ga_autotune times
-// a candidate set on the caller's batch with CUDA events and stores the fastest
-// as the default for (device, W, O, k); ga_align_batch uses the stored default
-// from then on.
+// Autotuner: how fast a batch of pairs of about one length runs depends on the
+// windows per turn of the sliced queue. ga_autotune times the library's own choice
+// and, where stored turns would be taken, others on the caller's batch with CUDA
+// events and stores the best as the default for (device, W, O, k); ga_align_batch
+// uses the stored default from then on. The hand-out order stays longest first: it
+// costs a batch of one length a few microseconds and gives one of mixed lengths a
+// quarter (20,000 pairs of 100 bases-50 kb in index order 5.57 ms, 4.26).
 //
 // Graph: ga_graph_create captures one whole step (2-bit packing of the ASCII
 // inputs, the workspace reset, the longest-first ordering and the alignment
 // kernel) into a CUDA graph for fixed buffers; ga_graph_launch replays it with
 // one call.
-#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
-#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -64,21 +64,25 @@ int bad_wok(int W, int O, int k) {
   return W < 1 || W > GA_MAX_W_ONCHIP || O < 0 || O >= W || k < 0;
 }
 
-// Candidate tunings: hand-out order and windows per turn. (The batched kernel
-// runs one lane per pair; the launch shape follows from the number of pairs.)
-std::vector<ga_tuning> candidates() {
-  std::vector<ga_tuning> c;
-  for (int lpt : {1, -1})
-    for (int slice : {0, -1, 32, 64, 128}) c.push_back(ga_tuning{8, 8, 39, lpt, 0, slice});
-  return c;
-}
+// slice_windows 0: the library's own choice.
+ga_tuning tuning_of(int slice_windows) { return ga_tuning{8, 8, 39, 1, 0, slice_windows}; }
+
+// The windows per turn that are timed against it. (No turns at all, -1, save a batch of short reads their set-up, a few microseconds,
+// but would cost later batches of long ones a fifth: 24,000 pairs of 10 kb 3.08 ms,
+// 2.57. They are left to ga_tuning_set.)
+constexpr int kTurns[] = {32, 64, 128};
+
+// What a choice of turns has to gain over the library's own to be stored: single
+// runs of one tuning differ by up to 2% (24,000 pairs of 10 kb: 2.52-2.57 ms, in
+// turns of 32 windows 2.47-2.53).
+constexpr float kGain = 0.98f;
 
 }  // namespace
 
 extern "C" int ga_tuning_get(int W, int O, int k, ga_tuning* out) {
   if (!out || bad_wok(W, O, k)) return GA_EINVAL;
   if (ga::stored_tuning(W, O, k, out)) return GA_OK;
-  *out = ga_tuning{8, 8, 39, 1, 0, 0};
+  *out = tuning_of(0);
   return GA_OK;
 }
 
@@ -95,16 +99,8 @@ extern "C" int ga_tuning_set(int W, int O, int k, const ga_tuning* t) {
 
 extern "C" int ga_autotune_workspace_size(uint32_t n_pairs, int W, int O, int k, size_t* bytes) {
   if (!bytes || bad_wok(W, O, k)) return GA_EINVAL;
-  size_t best = 0;
-  for (const ga_tuning& t : candidates()) {
-    size_t b = 0;
-    if (ga_workspace_size_tuned(n_pairs, W, O, k, &t, &b) == GA_OK) best = std::max(best, b);
-  }
-  size_t b = 0;
-  const int rc = ga_workspace_size(n_pairs, W, O, k, &b);
-  if (rc != GA_OK) return rc;
-  *bytes = std::max(best, b);
-  return GA_OK;
+  // (the size does not depend on the tuning)
+  return ga_workspace_size(n_pairs, W, O, k, bytes);
 }
 
 namespace {
@@ -130,12 +126,6 @@ int align_once(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_
                               stream);
 }
 
-int workspace_for(uint32_t n_pairs, int W, int O, int k, const ga_tuning* t, bool locate,
-                  size_t* need) {
-  return locate ? ga_workspace_size_locate(n_pairs, W, O, k, t, need)
-                : ga_workspace_size_tuned(n_pairs, W, O, k, t, need);
-}
-
 int autotune(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_t* d_read_len,
              const uint8_t* d_refs, const uint64_t* d_ref_off, const uint32_t* d_ref_len,
              uint32_t n_pairs, int W, int O, int k, const uint32_t* d_start_span,
@@ -154,44 +144,44 @@ int autotune(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_t*
                       stream);
   if (rc != GA_OK) return rc;
 
-  // Time every candidate (one warm-up run, then one timed run).
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return GA_ECUDA;
   if (cudaEventCreate(&e1) != cudaSuccess) {
     cudaEventDestroy(e0);
     return GA_ECUDA;
   }
-  float best_t = 1e30f;
-  ga_tuning best_c{};
-  rc = GA_OK;
-  for (const ga_tuning& c : candidates()) {
-    size_t need = 0;
-    if (workspace_for(n_pairs, W, O, k, &c, locate, &need) != GA_OK || need > ws_bytes) continue;
-    int r1 = align_once(d_reads, d_read_off, d_read_len, d_refs, d_ref_off, d_ref_len, n_pairs, W,
-                        O, k, d_start_span, d_ref_start, d_dist, d_status, d_ref_consumed, d_cigar,
-                        d_cigar_off, d_n_runs, nullptr, nullptr, d_workspace, ws_bytes, &c,
-                        stream);
-    if (r1 != GA_OK) continue;
-    cudaEventRecord(e0, s);
-    r1 = align_once(d_reads, d_read_off, d_read_len, d_refs, d_ref_off, d_ref_len, n_pairs, W, O,
-                    k, d_start_span, d_ref_start, d_dist, d_status, d_ref_consumed, d_cigar,
-                    d_cigar_off, d_n_runs, nullptr, nullptr, d_workspace, ws_bytes, &c, stream);
-    cudaEventRecord(e1, s);
-    if (r1 != GA_OK || cudaEventSynchronize(e1) != cudaSuccess) {
-      rc = GA_ECUDA;
-      break;
+  // One warm-up run, then one timed run.
+  const auto time_of = [&](const ga_tuning& c, float* ms) -> int {
+    for (int run = 0; run < 2; ++run) {
+      if (run == 1) cudaEventRecord(e0, s);
+      const int r = align_once(d_reads, d_read_off, d_read_len, d_refs, d_ref_off, d_ref_len, n_pairs, W,
+                               O, k, d_start_span, d_ref_start, d_dist, d_status, d_ref_consumed, d_cigar,
+                               d_cigar_off, d_n_runs, nullptr, nullptr, d_workspace, ws_bytes, &c, stream);
+      if (r != GA_OK) return r;
     }
-    float ms = 0;
-    cudaEventElapsedTime(&ms, e0, e1);
-    if (ms < best_t) {
-      best_t = ms;
-      best_c = c;
+    cudaEventRecord(e1, s);
+    if (cudaEventSynchronize(e1) != cudaSuccess) return GA_ECUDA;
+    return cudaEventElapsedTime(ms, e0, e1) == cudaSuccess ? GA_OK : GA_ECUDA;
+  };
+  ga_tuning best_c = tuning_of(0);
+  float best_t = 0;
+  rc = time_of(best_c, &best_t);
+  bool turns = false;
+  if (rc == GA_OK) rc = ga::cuda_fail(ga::turns_matter(n_pairs, W, O, d_workspace, s, &turns));
+  if (turns) {
+    const float automatic = best_t;
+    for (const int slice : kTurns) {
+      float ms = 0;
+      if (rc == GA_OK) rc = time_of(tuning_of(slice), &ms);
+      if (rc == GA_OK && ms < best_t && ms < kGain * automatic) {
+        best_t = ms;
+        best_c = tuning_of(slice);
+      }
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc != GA_OK) return rc;
-  if (best_t >= 1e30f) return GA_ENOSPC;  // no candidate fitted the workspace
   ga::store_tuning(W, O, k, &best_c, mode);
   if (best) *best = best_c;
   if (best_ms) *best_ms = best_t;

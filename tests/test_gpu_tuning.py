@@ -79,3 +79,21 @@ def test_stored_turns_leave_other_batches_as_they_are(slice_windows):
     # A call that asks for turns itself gets them.
     asked = [align(*x, tuning=t) for x in (few, fewer_than_lanes, alike, mixed)]
     assert asked == [(3, True), (3, True), (5, True), (5, True)]
+
+
+@pytest.mark.parametrize("n,lengths", [(1, [900]), (100, [300]), (20 * SMS, [100, 900]),
+                                       (128 * SMS + 500, [100, 200, 900]), (128 * SMS + 500, [300])])
+def test_autotuning_one_batch_leaves_others_as_they_are(n, lengths):
+    few = prepared(100, [300])
+    mixed = prepared(128 * SMS + 500, [100, 200, 900])
+    db, want = prepared(n, lengths)
+    best, ms = db.autotune()
+    np.testing.assert_array_equal(db.results().dist, want[np.arange(n) % 60])
+    stored = ga.ga_tuning_get(W, O, K)
+    assert ms > 0 and stored.slice_windows == best.slice_windows and stored.lpt == best.lpt == 1
+    if n <= 128 * SMS or len(lengths) > 1:  # no turns to choose
+        assert best.slice_windows == 0
+    assert best.slice_windows >= 0
+    assert align(*few) == (1, False)
+    assert align(*mixed) == (5, False)
+    assert align(*prepared(128 * SMS + 500, [300])) == (5, True)
