@@ -46,6 +46,12 @@
 
 namespace ga {
 
+// Places that a walk in an order with I or D before M looks at along the diagonal
+// for edges that come before M. (An op an iteration took one pair of 10 kb without
+// errors 1,280 us; 4 places 885, 8 846, but 8 take one of sequences that do not match
+// 1,567 instead of 1,420.)
+constexpr int kWalkAhead = 4;
+
 // A warp of LP pairs with NL lanes each. One lane per pair: LP = 32, or 16
 // (half a warp) where the tables of 32 would leave schedulers without a warp.
 // Several: LP * NL = 32, lane q of a pair holds word q of the vectors.
@@ -608,6 +614,14 @@ __device__ __forceinline__ uint2 column_bits(uint32_t tab0, uint32_t ct, uint32_
   }
 }
 
+// Bit j of a column's HP, likewise.
+template <int VW, int LP, int NL>
+__device__ __forceinline__ uint32_t hp_bit(uint32_t hp0, uint32_t ct, uint32_t j) {
+  using Shape = LaneShape<VW, LP, NL>;
+  const uint32_t k = VW == 3 ? min(j >> 5, 2u) : (j >> 5) & (VW - 1u);
+  return lds32(hp0 + ct * Shape::kHpBytes + k * Shape::kWord) >> (j & 31u);
+}
+
 // What a walk reads: the window's bit planes and the table's columns.
 template <int VW, int LP, int NL>
 struct Walk {
@@ -615,11 +629,36 @@ struct Walk {
   uint32_t plane_lane;
   uint32_t tab0, hp0;  // column 0's entries
   uint32_t top;        // wp - 1
+  // Orders other than the default: all ones if I, D come before M; the spare column's HP.
+  uint32_t over_i, over_d, hp_end;
   // Where the bases from read position cp and reference position ct on differ
   // (bit 31: the first of them).
   __device__ __forceinline__ uint32_t differ(uint32_t cp, uint32_t ct) const {
     return (plane_at<VW, LP, NL>(pl, plane_lane, 0, cp) ^ plane_at<VW, LP, NL>(tl, plane_lane, 2, ct)) |
            (plane_at<VW, LP, NL>(ph, plane_lane, 1, cp) ^ plane_at<VW, LP, NL>(th, plane_lane, 3, ct));
+  }
+  // Where along the diagonal from there an insertion or a deletion that comes before
+  // M is possible (bit 31: the first place), kWalkAhead places. Bit j - u of column
+  // ct + u is turned to bit 31 - u by the same distance whatever u is. (Places past
+  // the window's end give anything: past the spare column HP's words are read for
+  // columns, of which the table has eight at least, and its last one for HP.)
+  __device__ __forceinline__ uint32_t before_match(uint32_t cp, uint32_t ct) const {
+    using Shape = LaneShape<VW, LP, NL>;
+    const uint32_t j = top - cp;
+    const uint32_t vp = tab0 + ct * Shape::kColBytes + (Shape::kTogether ? 8u : 4u), hp = hp0 + ct * Shape::kHpBytes;
+    uint32_t found = 0;
+#pragma unroll
+    for (int u = 0; u < kWalkAhead; ++u) {
+      uint32_t k = 0;  // its word
+      if constexpr (VW == 2) k = j >= 32u + static_cast<uint32_t>(u) ? 1u : 0u;
+      if constexpr (VW == 3) k = min((j - u) >> 5, 2u);
+      if constexpr (VW == 4) k = ((j - u) >> 5) & 3u;
+      const uint32_t v = lds32(vp + u * Shape::kColBytes + k * (Shape::kTogether ? 4u : 2u * Shape::kWord));
+      const uint32_t h = lds32(min(hp + u * Shape::kHpBytes, hp_end) + k * Shape::kWord);
+      const uint32_t x = (v & over_i) | (h & over_d);
+      found |= __funnelshift_r(x, x, j + 1u) & (0x80000000u >> u);
+    }
+    return found;
   }
 };
 
@@ -640,49 +679,77 @@ __device__ __forceinline__ void book_ops(Runs& st, const LateOps& o) {
   st.run_len += o.edit ? 1u : 0u;
 }
 
-// One iteration of a walk at read base cp and text base ct of the window, up
-// to `goal` and `tend`: with the default order the matches ahead (up to 32 base
-// pairs compared at once) and the edit that ends them, else one op. No
-// branches: a lane whose counts are used up appends nothing.
-template <int VW, int LP, int NL, bool kAny, class Runs>
-__device__ __forceinline__ void walk_step(const Walk<VW, LP, NL>& w, uint64_t tb_table, Runs& st,
-                                          uint32_t& cp, uint32_t& ct, uint32_t goal, uint32_t tend,
-                                          LateOps& late) {
+// One iteration of a walk at read base cp and text base ct of the window, up to
+// `goal` and `tend`: the matches ahead (up to 32 base pairs compared at once) and
+// the edit that ends them. No branches: a lane whose counts are used up appends
+// nothing.
+template <int VW, int LP, int NL, class Runs>
+__device__ __forceinline__ void walk_step(const Walk<VW, LP, NL>& w, Runs& st, uint32_t& cp, uint32_t& ct,
+                                          uint32_t goal, uint32_t tend, LateOps& late) {
   const uint32_t lim = min(min(goal - cp, tend - ct), 32u);
-  if constexpr (!kAny) {
-    const uint32_t z = leading_zeros(w.differ(cp, ct));
-    const uint32_t L = min(z, lim);
-    const uint32_t one = z < lim ? 1u : 0u;  // an edit ends the matches
-    cp += L;
-    ct += L;
-    const uint2 e = column_bits<VW, LP, NL>(w.tab0, ct, w.top - cp);
-    book_ops(st, late);
-    late.matches = L;
-    // S (D0 clear) takes a base of both, I (VP' set) of the read, D of the text.
-    const uint32_t from_p = one & (e.y | ~e.x), from_t = one & ~(e.x & e.y);
-    const uint32_t code = from_p + 2u * from_t;
-    late.edit = code == 3u ? kOpSubst : code;
-    st.edits += one;
-    cp += from_p;
-    ct += from_t;
-  } else {
-    const uint32_t one = lim > 0u ? 1u : 0u;
-    const uint32_t j = w.top - cp;
-    const uint32_t mm = w.differ(cp, ct);
-    const uint2 e = column_bits<VW, LP, NL>(w.tab0, ct, j);
-    const uint32_t k = VW == 3 ? min(j >> 5, 2u) : (j >> 5) & (VW - 1u);
-    const uint32_t h = lds32(w.hp0 + ct * LaneShape<VW, LP, NL>::kHpBytes + k * LaneShape<VW, LP, NL>::kWord);
-    const uint32_t can = (~mm >> 31) << kTbM | (~e.x & 1u) << kTbS | (e.y & 1u) << kTbI |
-                         ((h >> (j & 31u)) & 1u) << kTbD;
-    const uint32_t code = static_cast<uint32_t>(tb_table >> (4 * can)) & 15u;
-    const uint32_t op = (kTbOps >> (4u * code)) & 15u;
-    close_run(st, one != 0u && st.run_op != op);
-    st.run_op = one ? op : st.run_op;
-    st.run_len += one;
-    st.edits += op != kOpMatch ? one : 0u;
-    cp += op != kOpDel ? one : 0u;
-    ct += op != kOpIns ? one : 0u;
-  }
+  const uint32_t z = leading_zeros(w.differ(cp, ct));
+  const uint32_t L = min(z, lim);
+  const uint32_t one = z < lim ? 1u : 0u;  // an edit ends the matches
+  cp += L;
+  ct += L;
+  const uint2 e = column_bits<VW, LP, NL>(w.tab0, ct, w.top - cp);
+  book_ops(st, late);
+  late.matches = L;
+  // S (D0 clear) takes a base of both, I (VP' set) of the read, D of the text.
+  const uint32_t from_p = one & (e.y | ~e.x), from_t = one & ~(e.x & e.y);
+  const uint32_t code = from_p + 2u * from_t;
+  late.edit = code == 3u ? kOpSubst : code;
+  st.edits += one;
+  cp += from_p;
+  ct += from_t;
+}
+
+// The same in any other order, as many matches as are sure to be taken and the op
+// after them: up to a mismatch, or to where an insertion or a deletion that comes
+// before M is possible (a substitution never is where the bases match), kWalkAhead
+// places ahead at most.
+template <int VW, int LP, int NL>
+__device__ __forceinline__ uint32_t any_op(const Walk<VW, LP, NL>& w, uint64_t tb_table, uint32_t cp, uint32_t ct,
+                                           uint32_t mm) {
+  const uint32_t j = w.top - cp;
+  const uint2 e = column_bits<VW, LP, NL>(w.tab0, ct, j);
+  const uint32_t h = hp_bit<VW, LP, NL>(w.hp0, ct, j);
+  const uint32_t can = (~mm >> 31) << kTbM | (~e.x & 1u) << kTbS | (e.y & 1u) << kTbI | (h & 1u) << kTbD;
+  const uint32_t code = static_cast<uint32_t>(tb_table >> (4 * can)) & 15u;
+  return (kTbOps >> (4u * code)) & 15u;
+}
+template <int VW, int LP, int NL, class Runs>
+__device__ __forceinline__ void walk_step_ahead(const Walk<VW, LP, NL>& w, uint64_t tb_table, Runs& st,
+                                                uint32_t& cp, uint32_t& ct, uint32_t goal, uint32_t tend) {
+  const uint32_t lim = min(min(goal - cp, tend - ct), 32u);
+  const uint32_t mm = w.differ(cp, ct);
+  uint32_t ends = mm;
+  if (w.over_i | w.over_d) ends |= w.before_match(cp, ct) | (0x80000000u >> kWalkAhead);
+  const uint32_t z = leading_zeros(ends);
+  const uint32_t L = min(z, lim);
+  const uint32_t one = z < lim ? 1u : 0u;
+  cp += L;
+  ct += L;
+  const uint32_t op = any_op<VW, LP, NL>(w, tb_table, cp, ct, mm << (L & 31u));
+  book_ops(st, LateOps{L, one ? op : 0u});
+  st.edits += op != kOpMatch ? one : 0u;
+  cp += op != kOpDel ? one : 0u;
+  ct += op != kOpIns ? one : 0u;
+}
+
+// One op in any order.
+template <int VW, int LP, int NL, class Runs>
+__device__ __forceinline__ void walk_step_any(const Walk<VW, LP, NL>& w, uint64_t tb_table, Runs& st,
+                                              uint32_t& cp, uint32_t& ct, uint32_t goal, uint32_t tend) {
+  const uint32_t lim = min(min(goal - cp, tend - ct), 32u);
+  const uint32_t one = lim > 0u ? 1u : 0u;
+  const uint32_t op = any_op<VW, LP, NL>(w, tb_table, cp, ct, w.differ(cp, ct));
+  close_run(st, one != 0u && st.run_op != op);
+  st.run_op = one ? op : st.run_op;
+  st.run_len += one;
+  st.edits += op != kOpMatch ? one : 0u;
+  cp += op != kOpDel ? one : 0u;
+  ct += op != kOpIns ? one : 0u;
 }
 
 // Starts loading the bases of the pair's next window: to shared memory, or into
@@ -722,6 +789,12 @@ __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& 
                                             int cols) {
   using Shape = LaneShape<VW, LP, NL>;
   constexpr uint32_t kMask = Shape::kMask;
+  // Another order than the default: whether windows of few edits (every lane's) walk
+  // by matches. One pair of 10 kb, DIMS, without errors: 885 us, an op an iteration
+  // 1,285; at 10% errors 1,080, 1,312. Windows of many edits gain nothing by it (one
+  // pair that does not match: 1,420 us against 1,310), and wide windows by one lane
+  // each lose in both forms to the larger kernel (5,000 pairs at W = 128 7%).
+  constexpr bool kAhead = VW <= 2 || NL > 1;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t q = lane % NL, slot = lane / NL;
   const uint32_t eq_lane = base + lane * Shape::kEqLane;
@@ -773,6 +846,11 @@ __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& 
     }
   }
   w.top = static_cast<uint32_t>(wp) - 1u;
+  if constexpr (kAny) {  // what the table takes of {M, I} and of {M, D}
+    w.over_i = (p.tb_table >> (4 * (1 << kTbM | 1 << kTbI)) & 15u) == kTbI ? ~0u : 0u;
+    w.over_d = (p.tb_table >> (4 * (1 << kTbM | 1 << kTbD)) & 15u) == kTbD ? ~0u : 0u;
+    w.hp_end = hp_lane + static_cast<uint32_t>(cols) * Shape::kHpBytes;
+  }
   const int ncols16 = (p.W + 15) >> 4;
   // A window that stops W - O bases in, before its text can run out, ends when
   // either count gets there; others end with their pattern bases (the text
@@ -821,11 +899,23 @@ __device__ __forceinline__ void lane_window(const AlignParams& p, LanePair<VW>& 
     // Each lane on its own until its counts are used up: a vote of the warp per
     // round costs more than the lanes that wait for the longest walk. Two
     // iterations to a test.
-    while (cp < goal && ct < tend) {
-      walk_step<VW, LP, NL, kAny>(w, p.tb_table, st, cp, ct, goal, tend, late);
-      walk_step<VW, LP, NL, kAny>(w, p.tb_table, st, cp, ct, goal, tend, late);
+    if constexpr (!kAny) {
+      while (cp < goal && ct < tend) {
+        walk_step<VW, LP, NL>(w, st, cp, ct, goal, tend, late);
+        walk_step<VW, LP, NL>(w, st, cp, ct, goal, tend, late);
+      }
+      book_ops(st, late);
+    } else if (kAhead && __all_sync(kMask, (w.over_i | w.over_d) == 0u || !ga || 8 * dmin <= p.W)) {
+      while (cp < goal && ct < tend) {
+        walk_step_ahead<VW, LP, NL>(w, p.tb_table, st, cp, ct, goal, tend);
+        if constexpr (VW <= 2) walk_step_ahead<VW, LP, NL>(w, p.tb_table, st, cp, ct, goal, tend);
+      }
+    } else {
+      while (cp < goal && ct < tend) {
+        walk_step_any<VW, LP, NL>(w, p.tb_table, st, cp, ct, goal, tend);
+        walk_step_any<VW, LP, NL>(w, p.tb_table, st, cp, ct, goal, tend);
+      }
     }
-    if constexpr (!kAny) book_ops(st, late);
     __syncwarp(kMask);
     if (cb + cols >= need || !__any_sync(kMask, cp < goal && ct < text)) break;
   }

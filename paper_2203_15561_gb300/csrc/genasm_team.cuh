@@ -213,8 +213,8 @@ __device__ __forceinline__ void team_windows(const AlignParams& p, TeamPair<VW>&
   WindowRuns rw{0xffffffffu, 0u, 0u, 0u, runs_lane};
   LateOps late{0u, 0u};
   while (cp < goal && ct < text) {
-    walk_step<VW, 32, 1, false>(w, p.tb_table, rw, cp, ct, goal, text, late);
-    walk_step<VW, 32, 1, false>(w, p.tb_table, rw, cp, ct, goal, text, late);
+    walk_step<VW, 32, 1>(w, rw, cp, ct, goal, text, late);
+    walk_step<VW, 32, 1>(w, rw, cp, ct, goal, text, late);
   }
   book_ops(rw, late);
   if (cp < goal && !inner) {  // the text is used up
