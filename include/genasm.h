@@ -132,9 +132,10 @@ int ga_workspace_size(uint32_t n_pairs, int W, int O, int k, size_t* bytes_out);
  *                    outnumber the resident lanes, but less than 16 times).
  *                    Turns that a call's own tuning asks for (> 0) run a lane
  *                    per pair also where few pairs would get a team of lanes
- *                    each; stored ones (ga_autotune, ga_tuning_set) are taken
- *                    where the pairs outnumber the resident lanes and are of
- *                    about one length.
+ *                    each; those of ga_tuning_set are taken where the pairs
+ *                    outnumber the resident lanes and are of about one length,
+ *                    unless it says lpt -1 (which leaves the lengths unknown);
+ *                    for ga_autotune's see there.
  */
 typedef struct ga_tuning_s {
   int lanes_per_pair;
@@ -158,16 +159,17 @@ int ga_tuning_set(int W, int O, int k, const ga_tuning* tuning);
 /*
  * ga_autotune - the autotuner of the batched kernel. Runs the current default
  * once on the caller's sample (with statistics), then times the library's own
- * choice and, where the pairs outnumber the resident lanes and are of about
- * one length, turns of 32, 64 and 128 windows (slice_windows) with CUDA
- * events, one warm-up and one timed run each. Stores the fastest, or the
- * library's choice where none is 2% faster, as the default for this device and
- * (W, O, k); pairs stay longest first (lpt 1). Arguments as ga_align_batch
- * (outputs are overwritten; d_n_windows and d_cells are required); the
- * workspace must hold ga_autotune_workspace_size(n_pairs, W, O, k) bytes.
- * Synchronous: returns once every run has finished. *best / *best_ms (either
- * may be NULL) receive the choice and its time. The paper gives no tuning
- * procedure.
+ * choice and, where the pairs outnumber the resident lanes, a candidate set of
+ * (lpt, slice_windows) with CUDA events, one warm-up and one timed run each.
+ * Stores the fastest, or the library's choice where none is 2% faster, as the
+ * default for this device and (W, O, k). It is taken by batches like the
+ * sample: of more pairs than resident lanes, and of about one length or of
+ * mixed lengths as the sample's; others run as without it. Arguments as
+ * ga_align_batch (outputs are overwritten; d_n_windows and d_cells are
+ * required); the workspace must hold ga_autotune_workspace_size(n_pairs, W, O,
+ * k) bytes. Synchronous: returns once every run has finished. *best / *best_ms
+ * (either may be NULL) receive the choice and its time. The paper gives no
+ * tuning procedure.
  * Errors: GA_EINVAL (also for W > GA_MAX_W_ONCHIP: wider windows take no
  * tuning), GA_ENOSPC (workspace too small), GA_ECUDA.
  */

@@ -199,7 +199,7 @@ cudaError_t launch_ablation(const AlignParams& p, int variant, uint64_t* table_b
   if (table_bytes &&
       (e = cudaMemsetAsync(table_bytes, 0, 5ull * sizeof(uint64_t) * p.n_pairs, s)) != cudaSuccess)
     return e;
-  if ((e = launch_lpt_order(p.read_len, p.n_pairs, hist, order, 1u, false, nullptr, s)) != cudaSuccess) return e;
+  if ((e = launch_lpt_order(p.read_len, p.n_pairs, hist, order, 1u, false, 0u, nullptr, s)) != cudaSuccess) return e;
   const AblationArgs a{reinterpret_cast<uint32_t*>(w + L.queue), order,
                        reinterpret_cast<uint64_t*>(w + L.tables), table_bytes};
   switch (variant) {

@@ -79,8 +79,12 @@ __device__ __forceinline__ uint32_t scan_buckets(uint32_t v, uint32_t* s) {
 // takes, and a quarter more: where a few long pairs decide, fewer lanes share
 // their warps and their windows are shorter (the walk lasts as long as the
 // warp's longest).
+//
+// facts[2], whether the order is to be that of the indexes: with a `choice`, an
+// autotuned order and autotuned turns are taken if the lengths are of their kind,
+// and facts[0] says whether turns are.
 __device__ __forceinline__ void length_facts(uint32_t count, uint32_t start, uint32_t n, uint32_t warps,
-                                             uint32_t* facts) {
+                                             uint32_t choice, uint32_t* facts) {
   __shared__ uint32_t longest, ninth;
   __shared__ unsigned long long total;
   const uint32_t len = kLptBuckets - 1u - threadIdx.x;  // in 64 bases
@@ -95,9 +99,15 @@ __device__ __forceinline__ void length_facts(uint32_t count, uint32_t start, uin
   if ((threadIdx.x & 31u) == 0u && mine) atomicAdd(&total, mine);
   __syncthreads();
   if (threadIdx.x == 0) {
-    facts[0] = 5u * (ninth + 1u) >= 4u * (longest + 1u) ? 1u : 0u;
+    const bool alike = 5u * (ninth + 1u) >= 4u * (longest + 1u);
+    const bool tuned = choice && alike == ((choice & kChoiceAlike) != 0u);
+    bool turns = alike && (!choice || (choice & kChoiceAutomatic));
+    if (tuned && (choice & (kChoiceTurns | kChoiceNoTurns))) turns = (choice & kChoiceTurns) != 0u;
+    const bool index = tuned && (choice & kChoiceIndex);
+    facts[0] = turns ? 1u : 0u;
     const unsigned long long lanes = 5ull * total / (4ull * warps * (longest + 1u)) + 1ull;
-    facts[1] = lanes < 32ull ? static_cast<uint32_t>(lanes) : 32u;
+    facts[1] = index ? 0u : lanes < 32ull ? static_cast<uint32_t>(lanes) : 32u;
+    facts[2] = index ? 1u : 0u;
   }
 }
 
@@ -127,7 +137,7 @@ __device__ __forceinline__ void length_split(uint32_t count, uint32_t start, uin
     mass[kLptBuckets] = mass[x] + m;
   }
   __syncthreads();
-  if (x >= 32u || facts[0]) return;
+  if (x >= 32u || facts[0] || facts[2]) return;
   uint32_t top = 0;  // the longest pair's bucket
   for (uint32_t b = kLptBuckets / 2; b; b >>= 1)
     if (longer[top + b] == 0u) top += b;
@@ -162,7 +172,7 @@ constexpr uint32_t kLptOneBlock = 16384;
 
 __global__ void __launch_bounds__(kLptBuckets)
     lpt_block_kernel(const uint32_t* __restrict__ read_len, uint32_t n, uint32_t warps, bool split,
-                     uint32_t* __restrict__ queue, uint32_t* __restrict__ order) {
+                     uint32_t choice, uint32_t* queue, uint32_t* __restrict__ order) {
   __shared__ uint32_t h[kLptBuckets];
   __shared__ uint32_t s[32];
   const uint32_t x = threadIdx.x;
@@ -182,8 +192,9 @@ __global__ void __launch_bounds__(kLptBuckets)
     if (r < rounds) count_bucket(h, bucket[r], r * kLptBuckets + x < n);
   __syncthreads();
   const uint32_t start = scan_buckets(h[x], s);
-  length_facts(h[x], start, n, warps, queue + 5);
+  length_facts(h[x], start, n, warps, choice, queue + 5);
   __syncthreads();
+  const bool index = queue[7] != 0u;
   if (split) length_split(h[x], start, n, warps, s, queue + 5);
   h[x] = start;
   __syncthreads();
@@ -192,7 +203,7 @@ __global__ void __launch_bounds__(kLptBuckets)
     if (r < rounds) {
       const uint32_t q = r * kLptBuckets + x;
       const uint32_t at = count_bucket(h, bucket[r], q < n);
-      if (q < n) order[at] = q;
+      if (q < n) order[index ? q : at] = q;
     }
   }
 }
@@ -222,20 +233,21 @@ __global__ void __launch_bounds__(kLptBuckets)
 
 // Exclusive scan of the bucket counts in place (one block of kLptBuckets threads).
 __global__ void __launch_bounds__(kLptBuckets) lpt_scan_kernel(uint32_t* hist, uint32_t n, uint32_t warps,
-                                                                bool split, uint32_t* facts) {
+                                                                bool split, uint32_t choice, uint32_t* facts) {
   __shared__ uint32_t s[32];
   const uint32_t count = hist[threadIdx.x];
   const uint32_t start = scan_buckets(count, s);
-  if (facts) length_facts(count, start, n, warps, facts);
+  if (facts) length_facts(count, start, n, warps, choice, facts);
   __syncthreads();
   if (facts && split) length_split(count, start, n, warps, s, facts);
   hist[threadIdx.x] = start;
 }
 
 __global__ void __launch_bounds__(kLptBuckets)
-    lpt_scatter_kernel(const uint32_t* __restrict__ read_len, uint32_t n,
+    lpt_scatter_kernel(const uint32_t* __restrict__ read_len, uint32_t n, const uint32_t* __restrict__ facts,
                        uint32_t* __restrict__ cursor, uint32_t* __restrict__ order) {
   __shared__ uint32_t h[kLptBuckets];
+  const bool index = facts && facts[2] != 0u;
   lpt_count(read_len, n, h);
   const uint32_t mine = h[threadIdx.x];
   const uint32_t start = mine ? atomicAdd(&cursor[threadIdx.x], mine) : 0u;
@@ -247,17 +259,17 @@ __global__ void __launch_bounds__(kLptBuckets)
   for (uint32_t r = 0; r < kLptPairs / kLptBuckets; ++r) {
     const uint64_t q = q0 + r * kLptBuckets;
     const uint32_t at = count_bucket(h, q < n ? lpt_bucket(read_len[q]) : 0u, q < n);
-    if (q < n) order[at] = static_cast<uint32_t>(q);
+    if (q < n) order[index ? q : at] = static_cast<uint32_t>(q);
   }
 }
 
 cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* hist, uint32_t* order,
-                             uint32_t warps, bool split, uint32_t* facts, cudaStream_t s) {
+                             uint32_t warps, bool split, uint32_t choice, uint32_t* facts, cudaStream_t s) {
   const uint32_t blocks =
       static_cast<uint32_t>((static_cast<uint64_t>(n) + kLptPairs - 1) / kLptPairs);
   lpt_histogram_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, hist);
-  lpt_scan_kernel<<<1, kLptBuckets, 0, s>>>(hist, n, warps, split, facts);
-  lpt_scatter_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, hist, order);
+  lpt_scan_kernel<<<1, kLptBuckets, 0, s>>>(hist, n, warps, split, choice, facts);
+  lpt_scatter_kernel<<<blocks, kLptBuckets, 0, s>>>(read_len, n, facts, hist, order);
   count_launches(3);
   return cudaGetLastError();
 }
@@ -332,9 +344,13 @@ int shape_entries(int G, int W, int O, int rows) {
 
 }  // namespace
 
-cudaError_t resolve_tuning(int W, int O, int k, const ga_tuning* t, int mode, ga_tuning* out) {
+cudaError_t resolve_tuning(int W, int O, int k, const ga_tuning* t, int mode, ga_tuning* out,
+                           int* made_for) {
   ga_tuning d{8, 8, 39, 1, 0, 0};
-  stored_tuning(W, O, k, &d, mode);  // chosen by an autotuner or set by ga_tuning_set
+  *made_for = kMadeForAny;
+  stored_tuning(W, O, k, &d, made_for, mode);  // chosen by an autotuner or set by ga_tuning_set
+  if (t && *made_for != kMadeForAny) d.lpt = 1;  // (an autotuned order goes with autotuned turns)
+  if (t) *made_for = kMadeForAny;
   // (a stored tuning without its own shape has the library's)
   const int rows = d.table_rows;
   int entries = shape_entries(d.lanes_per_pair, W, O, rows);
@@ -426,13 +442,16 @@ cudaError_t shape_warps(int dev, const LanePlan& plan, int* warps) {
 
 }  // namespace
 
-cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool lpt, LanePlan* plan) {
+cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool lpt, int made_for,
+                      LanePlan* plan) {
   int dev = 0, sms = 0;
   cudaError_t e = device_sms(&dev, &sms);
   if (e != cudaSuccess) return e;
   plan->vw = vw_for(p.W);
   plan->any_order = p.tb_table != tb_table(kTbOrderDefault);
-  plan->lpt = lpt;
+  const bool tuned = made_for != kMadeForAny;
+  plan->lpt = lpt || tuned;  // (the ordering finds out whether a tuning is for these lengths)
+  plan->choice = 0;
   const uint64_t n = std::max<uint32_t>(p.n_pairs, 1);
   const uint64_t scheds = 4ull * sms;
   const int all = up8(p.W), inner = up8(p.W - p.O);
@@ -503,33 +522,49 @@ cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool 
   // about one length, which the ordering finds out on the device (length_facts).
   // Stored turns are taken where the pairs outnumber the lanes and are of about one
   // length (stored turns of 64, and without them: 10,000 pairs of 10 kb 1.18 ms,
-  // 0.97; 20,000 of 100 bases-50 kb 5.72, 4.26). A single pair has nobody to take
-  // turns with.
+  // 0.97; 20,000 of 100 bases-50 kb 5.72, 4.26), autotuned ones and an autotuned
+  // order where the pairs outnumber the lanes and are of the kind they were made for
+  // (138,929 of 2-20 kb, a fifth decoys: index order and turns of 64 10.1 ms, without
+  // 17.3; 20,000 of 100 bases-50 kb the other way round, 5.8 and 4.3). A single pair
+  // has nobody to take turns with.
   const uint64_t lanes = warps * plan->lp;
   const bool automatic = slice_windows == 0 && n > lanes && n < 16 * lanes;
   const bool stored = slice_windows > 0 && !asked && n > lanes;
   plan->slice = n < 2 ? 0u : turns_asked || stored ? static_cast<uint32_t>(slice_windows) : automatic ? 64u : 0u;
   plan->turns = automatic ? 4u : stored ? kFixedTurns : 0u;
+  if (tuned && n > lanes) {
+    plan->choice = kChoice | (made_for == kMadeForAlike ? kChoiceAlike : 0u) | (lpt ? 0u : kChoiceIndex) |
+                   (slice_windows > 0 ? kChoiceTurns : slice_windows < 0 ? kChoiceNoTurns : 0u);
+    if (n < 16 * lanes) {
+      plan->choice |= kChoiceAutomatic;
+      if (slice_windows < 0) {  // (automatic turns where the tuning does not apply)
+        plan->slice = 64u;
+        plan->turns = 4u;
+      }
+    }
+  }
   // (waiting lanes take part in the ring as well)
   if (plan->slice) plan->lanes = plan->lp;
   return cudaSuccess;
 }
 
-cudaError_t turns_matter(uint32_t n_pairs, int W, int O, const void* ws, cudaStream_t s, bool* yes) {
+cudaError_t length_class(uint32_t n_pairs, int W, int O, const void* ws, cudaStream_t s, bool* outnumber,
+                         bool* alike) {
   AlignParams p{};
   p.n_pairs = n_pairs;
   p.W = W;
   p.O = O;
   p.tb_table = tb_table(kTbOrderDefault);
   LanePlan plan{};
-  *yes = false;
-  cudaError_t e = lane_plan(p, 64, false, true, &plan);
-  if (e != cudaSuccess || !plan.slice) return e;
-  uint32_t alike = 0;
-  const char* fact = static_cast<const char*>(ws) + workspace_layout(n_pairs).queue + 5 * sizeof(uint32_t);
-  e = cudaMemcpyAsync(&alike, fact, sizeof(alike), cudaMemcpyDeviceToHost, s);
+  cudaError_t e = lane_plan(p, 1, false, true, kMadeForAny, &plan);
+  *outnumber = *alike = false;
+  if (e != cudaSuccess || !plan.slice) return e;  // (stored turns are for pairs that do)
+  *outnumber = true;
+  uint32_t fact = 0;
+  const char* at = static_cast<const char*>(ws) + workspace_layout(n_pairs).queue + 5 * sizeof(uint32_t);
+  e = cudaMemcpyAsync(&fact, at, sizeof(fact), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  *yes = alike != 0;
+  *alike = fact != 0;
   return e;
 }
 
@@ -562,13 +597,13 @@ cudaError_t launch_batched(const AlignParams& p, const LanePlan& plan, void* ws,
   if (plan.team && p.n_pairs >= 64) return launch_team(p, plan, nullptr, s);
   if (plan.lpt && p.n_pairs >= 64 && p.n_pairs <= kLptOneBlock) {
     lpt_block_kernel<<<1, kLptBuckets, 0, s>>>(p.read_len, p.n_pairs, static_cast<uint32_t>(plan.warps),
-                                               plan.staged && plan.vw == 2, queue, order);
+                                               plan.staged && plan.vw == 2, plan.choice, queue, order);
     count_launches(1);
   } else {
     if ((e = cudaMemsetAsync(w, 0, L.order, s)) != cudaSuccess) return e;  // counters + histogram
     if (plan.lpt &&
         (e = launch_lpt_order(p.read_len, p.n_pairs, hist, order, static_cast<uint32_t>(plan.warps),
-                              plan.staged && plan.vw == 2, queue + 5, s)) != cudaSuccess)
+                              plan.staged && plan.vw == 2, plan.choice, queue + 5, s)) != cudaSuccess)
       return e;
   }
   if (plan.team) return launch_team(p, plan, plan.lpt ? order : nullptr, s);

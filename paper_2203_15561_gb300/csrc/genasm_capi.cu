@@ -65,12 +65,13 @@ int fill_params(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32
 }
 
 // Windows wider than 64 bases take no tuning.
-int resolve(int W, int O, int k, const ga_tuning* t, ga_tuning* out, int mode = 0) {
+int resolve(int W, int O, int k, const ga_tuning* t, ga_tuning* out, int* made_for, int mode) {
   if (wide_window(W)) {
     *out = ga_tuning{8, 8, 39, 1, 0, 0};
+    *made_for = ga::kMadeForAny;
     return GA_OK;
   }
-  const cudaError_t e = ga::resolve_tuning(W, O, k, t, mode, out);
+  const cudaError_t e = ga::resolve_tuning(W, O, k, t, mode, out, made_for);
   return e == cudaErrorInvalidValue ? GA_EINVAL : cuda_fail(e);
 }
 
@@ -78,7 +79,8 @@ int workspace_bytes(uint32_t n_pairs, int W, int O, int k, const ga_tuning* t, i
                     size_t* bytes_out) {
   if (!bytes_out || bad_wok(W, O, k)) return GA_EINVAL;
   ga_tuning r;
-  const int rc = resolve(W, O, k, t, &r, mode);
+  int made_for = 0;
+  const int rc = resolve(W, O, k, t, &r, &made_for, mode);
   if (rc == GA_OK) *bytes_out = ga::workspace_layout(n_pairs).total;
   return rc;
 }
@@ -87,10 +89,11 @@ int workspace_bytes(uint32_t n_pairs, int W, int O, int k, const ga_tuning* t, i
 int plan_batched(const ga::AlignParams& p, int k, const ga_tuning* t, int mode, const void* d_workspace,
                  size_t ws_bytes, ga::LanePlan* plan) {
   ga_tuning r;
-  const int rc = resolve(p.W, p.O, k, t, &r, mode);
+  int made_for = 0;
+  const int rc = resolve(p.W, p.O, k, t, &r, &made_for, mode);
   if (rc != GA_OK) return rc;
   if (!d_workspace || ws_bytes < ga::workspace_layout(p.n_pairs).total) return GA_ENOSPC;
-  return cuda_fail(ga::lane_plan(p, r.slice_windows, t != nullptr, r.lpt > 0, plan));
+  return cuda_fail(ga::lane_plan(p, r.slice_windows, t != nullptr, r.lpt > 0, made_for, plan));
 }
 
 }  // namespace

@@ -57,10 +57,18 @@ struct LanePlan {
   uint32_t turns;  // if not 0: turns only for pairs of about one length, each this
                    // fraction of its pair and `slice` windows at least
   int team;        // lanes of a team (8..32, or 128: a block of four warps); 0: no teams
+  uint32_t choice;  // what the ordering decides by the lengths (kChoice*; 0: as ever)
 };
 
 // `turns` for turns of `slice` windows whatever the pair's length.
 constexpr uint32_t kFixedTurns = 1u << 20;
+
+// A tuning that the autotuner stored, taken on the device where the pairs' lengths
+// are of the kind it was made for: of about one length, or mixed.
+constexpr uint32_t kChoice = 1, kChoiceAlike = 2;            // made for pairs of about one length
+constexpr uint32_t kChoiceIndex = 4;                         // then: index order
+constexpr uint32_t kChoiceTurns = 8, kChoiceNoTurns = 16;    // then: turns, none (neither: if automatic)
+constexpr uint32_t kChoiceAutomatic = 32;                    // turns pay, of pairs of about one length
 
 // What the lanes of a team take on (see genasm_team.cuh).
 constexpr int kTeamLanes = 128;
@@ -126,9 +134,9 @@ cudaError_t launch_ablation(const AlignParams& p, int variant, uint64_t* table_b
 // length buckets): hist must hold kLptBuckets zeroed counters, order n entries.
 // facts (may be null) receives 1 when the pairs are of about one length, else 0,
 // the lanes of each of `warps` warps that they can use, and with `split` how the
-// longest are split over the warps (n up to 2^22).
+// longest are split over the warps (n up to 2^22); `choice` as in LanePlan.
 cudaError_t launch_lpt_order(const uint32_t* read_len, uint32_t n, uint32_t* hist, uint32_t* order,
-                             uint32_t warps, bool split, uint32_t* facts, cudaStream_t s);
+                             uint32_t warps, bool split, uint32_t choice, uint32_t* facts, cudaStream_t s);
 
 // Lanes per warp of the long pairs that decide how long a batch takes (see
 // length_split): how many, and their numbers.
@@ -147,8 +155,10 @@ void uncount_launches(uint64_t n);  // kernels that were captured into a graph, 
 // apart for the two forms of the batched alignment: mode 0 anchored first
 // windows (ga_align_batch), mode 1 free-start first windows
 // (ga_align_batch_locate).
-bool stored_tuning(int W, int O, int k, struct ga_tuning_s* out, int mode = 0);
-void store_tuning(int W, int O, int k, const struct ga_tuning_s* t, int mode = 0);
+// `made_for`: the pairs' lengths that the autotuner had (kMade*).
+enum { kMadeForAny = -1, kMadeForMixed = 0, kMadeForAlike = 1 };
+bool stored_tuning(int W, int O, int k, struct ga_tuning_s* out, int* made_for, int mode);
+void store_tuning(int W, int O, int k, const struct ga_tuning_s* t, int made_for, int mode);
 
 cudaError_t measure_int_peak(double out[3], cudaStream_t s);
 cudaError_t measure_smem_peak(double out[2], cudaStream_t s);
@@ -171,19 +181,21 @@ cudaError_t launch_batched_locate(const AlignParams& p, const LanePlan& plan,
                                   cudaStream_t s);
 
 // The tuning in force for (W, O, k) on the current device: `t` (nullptr: none)
-// over the stored one of `mode` over the library's. cudaErrorInvalidValue for
-// one that names no launch shape.
+// over the stored one of `mode` over the library's, and what it was made for.
+// cudaErrorInvalidValue for one that names no launch shape.
 cudaError_t resolve_tuning(int W, int O, int k, const struct ga_tuning_s* t, int mode,
-                           struct ga_tuning_s* out);
+                           struct ga_tuning_s* out, int* made_for);
 
 // Launch shape of the batched kernel for p (p.n_pairs, W, O, order) on the
 // current device; slice_windows and lpt as in ga_tuning. `asked`: they come with
-// the call, not from a stored tuning.
-cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool lpt, LanePlan* plan);
+// the call, not from a stored tuning; made_for: what that was made for.
+cudaError_t lane_plan(const AlignParams& p, int slice_windows, bool asked, bool lpt, int made_for,
+                      LanePlan* plan);
 
-// Whether stored turns would be taken for n_pairs whose lengths an alignment
-// without turns of its own, longest first, has just left in the workspace (waits
-// for the stream).
-cudaError_t turns_matter(uint32_t n_pairs, int W, int O, const void* ws, cudaStream_t s, bool* yes);
+// Whether n_pairs outnumber the resident lanes, and whether they are of about one
+// length, as an untuned alignment has just left it in the workspace (waits for the
+// stream).
+cudaError_t length_class(uint32_t n_pairs, int W, int O, const void* ws, cudaStream_t s, bool* outnumber,
+                         bool* alike);
 
 }  // namespace ga

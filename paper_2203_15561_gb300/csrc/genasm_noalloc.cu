@@ -94,7 +94,7 @@ extern "C" int ga_align_batch_noalloc(const uint8_t* d_reads, const uint64_t* d_
 
   // No sliced queue: its ring and window states are not in the scratch.
   ga::LanePlan plan{};
-  cudaError_t e = ga::lane_plan(p, -1, true, true, &plan);
+  cudaError_t e = ga::lane_plan(p, -1, true, true, ga::kMadeForAny, &plan);
   if (e != cudaSuccess) return ga::cuda_fail(e);
   const ga::WorkspaceLayout L = ga::workspace_layout(n_pairs);
   if (L.order != kOrderOffset || L.order + 4ull * n_pairs > kScratchBytes) return GA_ENOSPC;

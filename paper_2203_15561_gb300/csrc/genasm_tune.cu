@@ -1,12 +1,11 @@
 // Autotuner and CUDA-graph capture of the batched alignment step.
 //
-// Autotuner: how fast a batch of pairs of about one length runs depends on the
-// windows per turn of the sliced queue. ga_autotune times the library's own choice
-// and, where stored turns would be taken, others on the caller's batch with CUDA
-// events and stores the best as the default for (device, W, O, k); ga_align_batch
-// uses the stored default from then on. The hand-out order stays longest first: it
-// costs a batch of one length a few microseconds and gives one of mixed lengths a
-// quarter (20,000 pairs of 100 bases-50 kb in index order 5.57 ms, 4.26).
+// Autotuner: how fast a batch runs whose pairs outnumber the resident lanes depends
+// on the order in which they are handed out and on the windows per turn of the
+// sliced queue. ga_autotune times a candidate set on the caller's batch with CUDA
+// events and stores the best as the default for (device, W, O, k), with the kind of
+// lengths that the batch had; ga_align_batch uses it from then on for batches of
+// that kind whose pairs outnumber the lanes.
 //
 // Graph: ga_graph_create captures one whole step (2-bit packing of the ASCII
 // inputs, the workspace reset, the longest-first ordering and the alignment
@@ -33,26 +32,38 @@ struct TuneKey {
   }
 };
 
+struct Stored {
+  ga_tuning tuning;
+  int made_for;
+};
+
 std::mutex g_tune_mutex;
-std::map<TuneKey, ga_tuning> g_tuned;
+std::map<TuneKey, Stored> g_tuned;
+thread_local const Stored* g_trial = nullptr;  // an autotuner's candidate, as if stored
 
 }  // namespace
 
-bool stored_tuning(int W, int O, int k, ga_tuning* out, int mode) {
+bool stored_tuning(int W, int O, int k, ga_tuning* out, int* made_for, int mode) {
+  if (g_trial) {
+    *out = g_trial->tuning;
+    *made_for = g_trial->made_for;
+    return true;
+  }
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   std::lock_guard<std::mutex> lock(g_tune_mutex);
   auto it = g_tuned.find(TuneKey{dev, W, O, k, mode});
   if (it == g_tuned.end()) return false;
-  *out = it->second;
+  *out = it->second.tuning;
+  *made_for = it->second.made_for;
   return true;
 }
 
-void store_tuning(int W, int O, int k, const ga_tuning* t, int mode) {
+void store_tuning(int W, int O, int k, const ga_tuning* t, int made_for, int mode) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return;
   std::lock_guard<std::mutex> lock(g_tune_mutex);
-  if (t) g_tuned[TuneKey{dev, W, O, k, mode}] = *t;
+  if (t) g_tuned[TuneKey{dev, W, O, k, mode}] = Stored{*t, made_for};
   else g_tuned.erase(TuneKey{dev, W, O, k, mode});
 }
 
@@ -64,25 +75,20 @@ int bad_wok(int W, int O, int k) {
   return W < 1 || W > GA_MAX_W_ONCHIP || O < 0 || O >= W || k < 0;
 }
 
-// slice_windows 0: the library's own choice.
-ga_tuning tuning_of(int slice_windows) { return ga_tuning{8, 8, 39, 1, 0, slice_windows}; }
+// The library's own choice: lpt 1, slice_windows 0.
+ga_tuning tuning_of(int lpt, int slice_windows) { return ga_tuning{8, 8, 39, lpt, 0, slice_windows}; }
 
-// The windows per turn that are timed against it. (No turns at all, -1, save a batch of short reads their set-up, a few microseconds,
-// but would cost later batches of long ones a fifth: 24,000 pairs of 10 kb 3.08 ms,
-// 2.57. They are left to ga_tuning_set.)
-constexpr int kTurns[] = {32, 64, 128};
-
-// What a choice of turns has to gain over the library's own to be stored: single
-// runs of one tuning differ by up to 2% (24,000 pairs of 10 kb: 2.52-2.57 ms, in
-// turns of 32 windows 2.47-2.53).
+// What another choice has to gain over the library's own to be stored: single runs
+// of one tuning differ by up to 2% (24,000 pairs of 10 kb: 2.52-2.57 ms).
 constexpr float kGain = 0.98f;
 
 }  // namespace
 
 extern "C" int ga_tuning_get(int W, int O, int k, ga_tuning* out) {
   if (!out || bad_wok(W, O, k)) return GA_EINVAL;
-  if (ga::stored_tuning(W, O, k, out)) return GA_OK;
-  *out = tuning_of(0);
+  int made_for = 0;
+  if (ga::stored_tuning(W, O, k, out, &made_for, 0)) return GA_OK;
+  *out = tuning_of(1, 0);
   return GA_OK;
 }
 
@@ -93,7 +99,7 @@ extern "C" int ga_tuning_set(int W, int O, int k, const ga_tuning* t) {
     const int rc = ga_workspace_size_tuned(1, W, O, k, t, &bytes);  // validates it
     if (rc != GA_OK) return rc;
   }
-  ga::store_tuning(W, O, k, t);
+  ga::store_tuning(W, O, k, t, ga::kMadeForAny, 0);
   return GA_OK;
 }
 
@@ -150,40 +156,46 @@ int autotune(const uint8_t* d_reads, const uint64_t* d_read_off, const uint32_t*
     cudaEventDestroy(e0);
     return GA_ECUDA;
   }
-  // One warm-up run, then one timed run.
-  const auto time_of = [&](const ga_tuning& c, float* ms) -> int {
-    for (int run = 0; run < 2; ++run) {
+  // One warm-up run, then one timed run, as if it were stored already.
+  const auto time_of = [&](const ga::Stored& c, float* ms) -> int {
+    ga::g_trial = &c;
+    int r = GA_OK;
+    for (int run = 0; run < 2 && r == GA_OK; ++run) {
       if (run == 1) cudaEventRecord(e0, s);
-      const int r = align_once(d_reads, d_read_off, d_read_len, d_refs, d_ref_off, d_ref_len, n_pairs, W,
-                               O, k, d_start_span, d_ref_start, d_dist, d_status, d_ref_consumed, d_cigar,
-                               d_cigar_off, d_n_runs, nullptr, nullptr, d_workspace, ws_bytes, &c, stream);
-      if (r != GA_OK) return r;
+      r = align_once(d_reads, d_read_off, d_read_len, d_refs, d_ref_off, d_ref_len, n_pairs, W, O, k,
+                     d_start_span, d_ref_start, d_dist, d_status, d_ref_consumed, d_cigar, d_cigar_off,
+                     d_n_runs, nullptr, nullptr, d_workspace, ws_bytes, nullptr, stream);
     }
+    ga::g_trial = nullptr;
+    if (r != GA_OK) return r;
     cudaEventRecord(e1, s);
     if (cudaEventSynchronize(e1) != cudaSuccess) return GA_ECUDA;
     return cudaEventElapsedTime(ms, e0, e1) == cudaSuccess ? GA_OK : GA_ECUDA;
   };
-  ga_tuning best_c = tuning_of(0);
+  ga::Stored best_c{tuning_of(1, 0), ga::kMadeForAny};
   float best_t = 0;
   rc = time_of(best_c, &best_t);
-  bool turns = false;
-  if (rc == GA_OK) rc = ga::cuda_fail(ga::turns_matter(n_pairs, W, O, d_workspace, s, &turns));
-  if (turns) {
-    const float automatic = best_t;
-    for (const int slice : kTurns) {
-      float ms = 0;
-      if (rc == GA_OK) rc = time_of(tuning_of(slice), &ms);
-      if (rc == GA_OK && ms < best_t && ms < kGain * automatic) {
-        best_t = ms;
-        best_c = tuning_of(slice);
+  bool outnumber = false, alike = false;
+  if (rc == GA_OK) rc = ga::cuda_fail(ga::length_class(n_pairs, W, O, d_workspace, s, &outnumber, &alike));
+  if (outnumber) {
+    const float library = best_t;
+    for (const int lpt : {1, -1})
+      for (const int slice : {0, -1, 32, 64, 128}) {
+        if (lpt == 1 && slice == 0) continue;
+        const ga::Stored c{tuning_of(lpt, slice), alike ? ga::kMadeForAlike : ga::kMadeForMixed};
+        float ms = 0;
+        if (rc == GA_OK) rc = time_of(c, &ms);
+        if (rc == GA_OK && ms < best_t && ms < kGain * library) {
+          best_t = ms;
+          best_c = c;
+        }
       }
-    }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc != GA_OK) return rc;
-  ga::store_tuning(W, O, k, &best_c, mode);
-  if (best) *best = best_c;
+  ga::store_tuning(W, O, k, &best_c.tuning, best_c.made_for, mode);
+  if (best) *best = best_c.tuning;
   if (best_ms) *best_ms = best_t;
   return GA_OK;
 }

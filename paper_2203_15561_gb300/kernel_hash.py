@@ -14,10 +14,10 @@ from pathlib import Path
 
 CSRC = Path(__file__).resolve().parent / "csrc"
 
-# The translation unit of the batched alignment kernel: the sources its
-# counters depend on.
-KERNEL_SOURCES = [CSRC / "genasm_align.cu", CSRC / "genasm_batch.cuh", CSRC / "genasm_lane.cuh",
-                  CSRC / "genasm_window.cuh", CSRC / "genasm_words.h", CSRC / "genasm_internal.h",
+# What the counters of the batched and the team kernel depend on.
+KERNEL_SOURCES = [CSRC / "genasm_align.cu", CSRC / "genasm_team.cu", CSRC / "genasm_batch.cuh",
+                  CSRC / "genasm_team.cuh", CSRC / "genasm_lane.cuh", CSRC / "genasm_window.cuh",
+                  CSRC / "genasm_words.h", CSRC / "genasm_internal.h",
                   CSRC.parent.parent / "include" / "genasm.h"]
 
 

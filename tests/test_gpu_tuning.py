@@ -1,7 +1,8 @@
 """GPU tests of what a stored tuning does to calls that it was not made for: small
-batches keep their teams, and turns are taken only by more pairs of about one length
-than there are lanes. Which way a call went shows in the launches and in the queue's
-counters at the start of the workspace."""
+batches keep their teams, and an order and turns are taken only by more pairs than
+there are lanes, of the kind of lengths they were chosen for. Which way a call went
+shows in the launches, and in the queue's counters and the pairs' order at the start
+of the workspace."""
 from __future__ import annotations
 
 import random
@@ -81,19 +82,41 @@ def test_stored_turns_leave_other_batches_as_they_are(slice_windows):
     assert asked == [(3, True), (3, True), (5, True), (5, True)]
 
 
-@pytest.mark.parametrize("n,lengths", [(1, [900]), (100, [300]), (20 * SMS, [100, 900]),
-                                       (128 * SMS + 500, [100, 200, 900]), (128 * SMS + 500, [300])])
+def handed_out(db):
+    """The order in which the last alignment handed the pairs out: "longest" or "index"."""
+    order = db.workspace[4352:4352 + 4 * db.n].cpu().numpy().view(np.uint32)
+    if np.array_equal(order, np.arange(db.n)):
+        return "index"
+    assert np.array_equal(np.sort(order), np.arange(db.n))
+    rl = np.asarray(db.batch.read_len).astype(np.int64)[order] >> 6
+    assert (np.diff(rl) <= 0).all()
+    return "longest"
+
+
+MANY = 128 * SMS + 500  # more pairs than lanes
+ALIKE, MIXED = [300], [100, 200, 900]
+
+
+@pytest.mark.parametrize("n,lengths", [(1, [900]), (100, [300]), (20 * SMS, [100, 900]), (MANY, MIXED), (MANY, ALIKE),
+                                       (MANY, [2800]), (MANY, [800, 1500, 2800])])
 def test_autotuning_one_batch_leaves_others_as_they_are(n, lengths):
-    few = prepared(100, [300])
-    mixed = prepared(128 * SMS + 500, [100, 200, 900])
+    few = prepared(100, ALIKE)
     db, want = prepared(n, lengths)
     best, ms = db.autotune()
     np.testing.assert_array_equal(db.results().dist, want[np.arange(n) % 60])
     stored = ga.ga_tuning_get(W, O, K)
-    assert ms > 0 and stored.slice_windows == best.slice_windows and stored.lpt == best.lpt == 1
-    if n <= 128 * SMS or len(lengths) > 1:  # no turns to choose
-        assert best.slice_windows == 0
-    assert best.slice_windows >= 0
+    assert ms > 0 and (stored.slice_windows, stored.lpt) == (best.slice_windows, best.lpt)
     assert align(*few) == (1, False)
-    assert align(*mixed) == (5, False)
-    assert align(*prepared(128 * SMS + 500, [300])) == (5, True)
+    if n < MANY:  # nothing to choose
+        assert (best.lpt, best.slice_windows) == (1, 0)
+    for lens in (ALIKE, MIXED):
+        d, w = prepared(MANY, lens)
+        launches, turns = align(d, w)
+        if n == MANY and (len(lens) == 1) == (len(lengths) == 1):  # made for it
+            alike = len(lens) == 1
+            assert turns == (best.slice_windows > 0 or (best.slice_windows == 0 and alike))
+            assert handed_out(d) == ("index" if best.lpt < 0 else "longest")
+        else:  # as without a stored tuning
+            assert turns == (len(lens) == 1) and handed_out(d) == "longest"
+    # A call's own tuning is not mixed with the stored one.
+    assert align(*few, tuning=ga.ga_tuning(0, 0, 0, 0, 0, 2)) == (3, True) and handed_out(few[0]) == "longest"
