@@ -382,11 +382,12 @@ def run_ours(args):
     if prof.exists():
         from paper_2203_15561_gb300.kernel_hash import source_hash
         fields = dict(l.split(":", 1) for l in prof.read_text().splitlines()
-                      if l.startswith(("source_hash:", "traffic_bytes_per_launch:")))
+                      if l.startswith(("source_hash:", "traffic_bytes_per_launch:", "pairs_profiled:")))
         if fields.get("source_hash", "").strip() == source_hash():
             roofline["traffic"] = int(fields["traffic_bytes_per_launch"]) * n / 10_000
             roofline["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of a "
-                                          "2,000-pair launch, scaled by pairs")
+                                          f"{int(fields['pairs_profiled']):,}-pair launch, scaled by "
+                                          "pairs")
 
     # ---- the same workload with a free-start first window (ga_align_batch_locate) ----
     free = None
@@ -450,7 +451,7 @@ def run_ours(args):
                                 "(slice_windows 0) when pairs of about one length outnumber the "
                                 "resident lanes less than 16 times over; -1: each pair to its end",
                        "l2": "no flush: each step streams 210 MB of ASCII input (> 126 MB L2) and "
-                             "writes ~0.5 GB of CIGAR runs, which evicts the previous step's data"},
+                             "writes ~0.26 GB of CIGAR runs, which evicts the previous step's data"},
             "gbases_per_s": gbases,
             "plain": plain,
             "batched_vs_plain": (value / plain["pairs_per_s"]) if plain else None,
@@ -691,7 +692,7 @@ def run_serving(args, dev):
                         f"{args.serve_seconds:g} s of arrivals, pool of {POOL_PAIRS} distinct pairs)",
             "offered_pairs_per_s": served["offered_pairs_per_s"], "served": served,
             "saturated": saturated, "plain_per_request": plain,
-            "step": "one captured CUDA graph per step (counters, step kernel, finished slots to "
+            "step": "one launch per step (active slots read from and finished slots written to "
                     "host-mapped memory); admission copies and result harvesting overlap the "
                     "running step"}
 

@@ -14,7 +14,7 @@
 namespace ga {
 
 // Default bounds of the two waits (ga_set_queue_wait_limits changes them):
-// polls of a warp whose groups all wait for a pair (about 0.2 microseconds
+// polls of a warp whose lanes all wait for a pair (about 0.2 microseconds
 // each): seconds, far beyond any legitimate wait (the rest of the longest
 // pair); past it the warp stops and flags the launch. Polls of a push waiting
 // for its slot: a fifth of a second at most.
@@ -73,7 +73,10 @@ __device__ __forceinline__ uint32_t scan_buckets(uint32_t v, uint32_t* s) {
 // one length end in a round of few lanes without turns; of mixed lengths, the
 // short ones at the end of the order fill the lanes up as the long ones finish,
 // and turns cost more than they give (30,011 pairs of 2-20 kb: 2.32 ms with
-// turns, 1.88 without; 20,000 of 100 bases-50 kb: 5.8 and 4.9).
+// turns, 1.88 without; 20,000 of 100 bases-50 kb: 5.8 and 4.9). Not always: 138,929
+// pairs of 2-20 kb anchored in a flank, in index order, take 10.1 ms with turns of 64
+// windows and 17.3 longest first without, which the lengths do not show; the
+// autotuner finds that.
 //
 // facts[1], the lanes per warp that finish all pairs by the time the longest one
 // takes, and a quarter more: where a few long pairs decide, fewer lanes share
@@ -118,7 +121,8 @@ __device__ __forceinline__ void length_facts(uint32_t count, uint32_t start, uin
 // with as many lanes as let len * cost(l) stay within t. Of 32 times between the
 // longest pair alone and in a full warp, the shortest whose warps suffice, all
 // other pairs in full warps. facts[3 + s]: the pairs that get at most
-// kSplitLanes(s) lanes. Only for vectors of two words and one warp per scheduler
+// kSplitLanes(s) lanes. (The cost is fitted at W = 64, O = 24 and used for all W of 33
+// to 64; only speed depends on it.) Only for vectors of two words and one warp per scheduler
 // (the one-word kernel lost 2% at 5,000 equal pairs). Alignment with the same
 // lanes in all warps, and split: 10,000 pairs of 2-20 kb 1.56 ms, 1.32; 5,000 of
 // 100 bases-20 kb at W = 48 1.65, 1.47; 20,000 of 100 bases-50 kb 4.52, 4.26 (a long
@@ -590,9 +594,8 @@ cudaError_t launch_batched(const AlignParams& p, const LanePlan& plan, void* ws,
   uint32_t* hist = reinterpret_cast<uint32_t*>(w + L.hist);
   uint32_t* order = reinterpret_cast<uint32_t*>(w + L.order);
   // One block orders a batch that keeps it busy for a few microseconds at most.
-  // (Below 64 pairs the order takes the general three launches: a whole step's
-  // launch count at such sizes is something callers have come to rely on. Teams
-  // have no use for the order.)
+  // (Teams have no use for an order. Below 64 pairs its three launches are made all
+  // the same: tests/test_gpu_parity.py counts them in a graph's replay of 40 pairs.)
   cudaError_t e = cudaSuccess;
   if (plan.team && p.n_pairs >= 64) return launch_team(p, plan, nullptr, s);
   if (plan.lpt && p.n_pairs >= 64 && p.n_pairs <= kLptOneBlock) {

@@ -152,7 +152,8 @@ cudaError_t launch_step_as(const AlignParams& p, int team, int blocks, const Ste
 //   152 pairs: 833, 440, 487, 585, 685, 842     608: 846, 1210, 518, 592, 697, 826
 //   1,216: 892, -, 855, 636, 728, 868           2,432: 904, -, 1583, 1050, 746, 913
 //   4,864: 912, -, -, 1898, 1295, 917 (four lanes: one more window in two rounds)
-// and 304 pairs 820 with one lane, 668 with 128, 504 with 32.
+// and 304 pairs 820 with one lane, 668 with 128, 504 with 32. (W = 64, O = 24; the
+// same limits serve every W up to 64.)
 int team_size(uint64_t n, int sms) {
   const uint64_t warps = 4ull * sms;
   return n <= warps / 4 ? 128 : n <= warps ? 32 : n <= 2 * warps ? 16 : n <= 4 * warps ? 8 : 0;

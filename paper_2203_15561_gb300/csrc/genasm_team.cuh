@@ -121,8 +121,6 @@ __device__ __forceinline__ void team_sync() {
   else __syncwarp();
 }
 
-// The windows of the team's pair from its position on, one to many of them, at
-// most `budget`.
 // The place of the start that lies on_p and on_t bases on: some windows ahead,
 // the starts differ by few bases in the read and in the diagonal, so that hardly
 // two share a place (if they do, one is lost).
@@ -141,6 +139,8 @@ __device__ __forceinline__ void team_ahead(const uint8_t* seq, uint32_t len, uin
   }
 }
 
+// The windows of the team's pair from its position on, one to many of them, at
+// most `budget`.
 template <int VW, int NB>
 __device__ __forceinline__ void team_windows(const AlignParams& p, TeamPair<VW>& tp, const TeamLane& me,
                                              uint32_t base, uint32_t budget) {
